@@ -7,13 +7,19 @@
 // representative below p; it is applied only when a result leaves the
 // library or when a value must be compared.
 //
-// Multiplication: 8x8-limb operand scanning, one row per limb of b.  Each
-// limb product is a single 32x32->64-bit multiply-add (mad.wide.u32, which
-// also adds the row's running word), and the high halves are folded in with
-// one add-with-carry chain per row: 64 wide products and 64 carry adds.
-// (On sm_103a a wide multiply-add costs as much as a high-half multiply, and
-// twice a low-half multiply, so separate lo/hi products would cost 1.5x.)
-// Squaring: 28 cross products, doubled, plus 8 diagonal squares.  Products
+// Multiplication: 8x8-limb operand scanning, one row per limb of b, with the
+// products of even and odd word positions in two accumulators, so that every
+// limb product is one 64-bit multiply-add with carry in and out (a mad.lo.cc /
+// madc.hi.cc pair) and almost no separate carry additions are left: 64 wide
+// multiply-adds and 24 ALU additions.  Measured per warp and scheduler at
+// eight warps each: a wide multiply-add takes 4.2 cycles of the FMA pipe
+// (30 a clock and SM; a low-half one 2.1) and an addition with carry 2.1 of
+// the ALU pipe, so a product is bound by 270 FMA cycles.  Adding each row's
+// running word as a zero-extended 64-bit addend and folding the high halves
+// in with addc took a register move per product beside 57 additions:
+// 385 cycles a product against 290, 530 a multiplication against 437.
+// Squaring: 28 cross products, doubled, plus 8 diagonal squares (420 -> 350
+// cycles with the reduction).  Products
 // and reductions live in out-of-line functions (fmul, fsqr): inlining them
 // into every call site of a point formula overflows the instruction cache.
 // Reduction of the 512-bit product uses the
@@ -327,174 +333,140 @@ __device__ __forceinline__ void fe_reduce(fe& r, const uint32_t c[16]) {
     if (e1 + b1) fe_add_K_masked(r, 0xffffffffu);
 }
 
-// t[0..15] = a * b.  Row i: p_j = a_j b_i + t[i+j] (one wide multiply-add,
-// never overflowing 64 bits), t[i] = lo(p_0), t[i+j] = lo(p_j) + hi(p_j-1)
-// + carry, t[i+8] = hi(p_7) + carry.
+// Rows of fused wide multiply-adds.  A 64-bit product a_j b_i lands on words
+// i + j and i + j + 1; products whose i + j has one parity tile the word
+// positions without overlap, so a row's four even (or four odd) products join
+// one carry chain of mad.lo.cc / madc.hi.cc pairs, and each pair is a single
+// 64-bit multiply-add with carry in and out.
+
+// e[0..7] = the four products of a row (nothing accumulated yet).
+__device__ __forceinline__ void row_first(uint32_t* e, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
+                                          uint32_t b) {
+    uint64_t p = (uint64_t)x0 * b;
+    e[0] = (uint32_t)p; e[1] = (uint32_t)(p >> 32);
+    p = (uint64_t)x1 * b;
+    e[2] = (uint32_t)p; e[3] = (uint32_t)(p >> 32);
+    p = (uint64_t)x2 * b;
+    e[4] = (uint32_t)p; e[5] = (uint32_t)(p >> 32);
+    p = (uint64_t)x3 * b;
+    e[6] = (uint32_t)p; e[7] = (uint32_t)(p >> 32);
+}
+
+// e[0..7] += the four products; the carry out becomes e[8].
+__device__ __forceinline__ void row_carry(uint32_t* e, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
+                                          uint32_t b) {
+    asm("mad.lo.cc.u32 %0, %9, %13, %0;\n\tmadc.hi.cc.u32 %1, %9, %13, %1;\n\t"
+        "madc.lo.cc.u32 %2, %10, %13, %2;\n\tmadc.hi.cc.u32 %3, %10, %13, %3;\n\t"
+        "madc.lo.cc.u32 %4, %11, %13, %4;\n\tmadc.hi.cc.u32 %5, %11, %13, %5;\n\t"
+        "madc.lo.cc.u32 %6, %12, %13, %6;\n\tmadc.hi.cc.u32 %7, %12, %13, %7;\n\t"
+        "addc.u32 %8, 0, 0;"
+        : "+r"(e[0]), "+r"(e[1]), "+r"(e[2]), "+r"(e[3]), "+r"(e[4]), "+r"(e[5]), "+r"(e[6]), "+r"(e[7]),
+          "=r"(e[8])
+        : "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(b));
+}
+
+// e[0..6] += the four products, whose top word becomes e[7]: e[7] was not
+// written before and e[6] held at most a carry, so nothing carries out.
+__device__ __forceinline__ void row_top(uint32_t* e, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3,
+                                        uint32_t b) {
+    asm("mad.lo.cc.u32 %0, %8, %12, %0;\n\tmadc.hi.cc.u32 %1, %8, %12, %1;\n\t"
+        "madc.lo.cc.u32 %2, %9, %12, %2;\n\tmadc.hi.cc.u32 %3, %9, %12, %3;\n\t"
+        "madc.lo.cc.u32 %4, %10, %12, %4;\n\tmadc.hi.cc.u32 %5, %10, %12, %5;\n\t"
+        "madc.lo.cc.u32 %6, %11, %12, %6;\n\tmadc.hi.u32 %7, %11, %12, 0;"
+        : "+r"(e[0]), "+r"(e[1]), "+r"(e[2]), "+r"(e[3]), "+r"(e[4]), "+r"(e[5]), "+r"(e[6]), "=r"(e[7])
+        : "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(b));
+}
+
+// t[0..15] = a * b: e collects the products at even word positions, o those
+// at odd positions (one word lower), and t = e + 2^32 o.
 __device__ __forceinline__ void mul_wide(uint32_t t[16], const fe& a, const fe& b) {
-    uint64_t p[8];
-#pragma unroll
-    for (int j = 0; j < 8; j++) p[j] = (uint64_t)a.v[j] * b.v[0];
-    t[0] = (uint32_t)p[0];
-    asm("add.cc.u32 %0, %8, %15;\n\taddc.cc.u32 %1, %9, %16;\n\taddc.cc.u32 %2, %10, %17;\n\t"
-        "addc.cc.u32 %3, %11, %18;\n\taddc.cc.u32 %4, %12, %19;\n\taddc.cc.u32 %5, %13, %20;\n\t"
-        "addc.cc.u32 %6, %14, %21;\n\taddc.u32 %7, %22, 0;"
-        : "=r"(t[1]), "=r"(t[2]), "=r"(t[3]), "=r"(t[4]), "=r"(t[5]), "=r"(t[6]), "=r"(t[7]), "=r"(t[8])
-        : "r"((uint32_t)p[1]), "r"((uint32_t)p[2]), "r"((uint32_t)p[3]), "r"((uint32_t)p[4]), "r"((uint32_t)p[5]),
-          "r"((uint32_t)p[6]), "r"((uint32_t)p[7]), "r"((uint32_t)(p[0] >> 32)), "r"((uint32_t)(p[1] >> 32)),
-          "r"((uint32_t)(p[2] >> 32)), "r"((uint32_t)(p[3] >> 32)), "r"((uint32_t)(p[4] >> 32)),
-          "r"((uint32_t)(p[5] >> 32)), "r"((uint32_t)(p[6] >> 32)), "r"((uint32_t)(p[7] >> 32)));
+    uint32_t e[16], o[15];
+    row_first(e, a.v[0], a.v[2], a.v[4], a.v[6], b.v[0]);
+    row_first(o, a.v[1], a.v[3], a.v[5], a.v[7], b.v[0]);
+    e[8] = 0;
 #pragma unroll
     for (int i = 1; i < 8; i++) {
-#pragma unroll
-        for (int j = 0; j < 8; j++) p[j] = (uint64_t)a.v[j] * b.v[i] + t[i + j];
-        t[i] = (uint32_t)p[0];
-        asm("add.cc.u32 %0, %8, %15;\n\taddc.cc.u32 %1, %9, %16;\n\taddc.cc.u32 %2, %10, %17;\n\t"
-            "addc.cc.u32 %3, %11, %18;\n\taddc.cc.u32 %4, %12, %19;\n\taddc.cc.u32 %5, %13, %20;\n\t"
-            "addc.cc.u32 %6, %14, %21;\n\taddc.u32 %7, %22, 0;"
-            : "=r"(t[i + 1]), "=r"(t[i + 2]), "=r"(t[i + 3]), "=r"(t[i + 4]), "=r"(t[i + 5]), "=r"(t[i + 6]),
-              "=r"(t[i + 7]), "=r"(t[i + 8])
-            : "r"((uint32_t)p[1]), "r"((uint32_t)p[2]), "r"((uint32_t)p[3]), "r"((uint32_t)p[4]), "r"((uint32_t)p[5]),
-              "r"((uint32_t)p[6]), "r"((uint32_t)p[7]), "r"((uint32_t)(p[0] >> 32)), "r"((uint32_t)(p[1] >> 32)),
-              "r"((uint32_t)(p[2] >> 32)), "r"((uint32_t)(p[3] >> 32)), "r"((uint32_t)(p[4] >> 32)),
-              "r"((uint32_t)(p[5] >> 32)), "r"((uint32_t)(p[6] >> 32)), "r"((uint32_t)(p[7] >> 32)));
+        if (i & 1) {
+            row_top(e + i + 1, a.v[1], a.v[3], a.v[5], a.v[7], b.v[i]);
+            row_carry(o + i - 1, a.v[0], a.v[2], a.v[4], a.v[6], b.v[i]);
+        } else {
+            row_carry(e + i, a.v[0], a.v[2], a.v[4], a.v[6], b.v[i]);
+            row_top(o + i, a.v[1], a.v[3], a.v[5], a.v[7], b.v[i]);
+        }
     }
+    t[0] = e[0];
+    asm("add.cc.u32  %0, %15, %30;\n\taddc.cc.u32 %1, %16, %31;\n\taddc.cc.u32 %2, %17, %32;\n\t"
+        "addc.cc.u32 %3, %18, %33;\n\taddc.cc.u32 %4, %19, %34;\n\taddc.cc.u32 %5, %20, %35;\n\t"
+        "addc.cc.u32 %6, %21, %36;\n\taddc.cc.u32 %7, %22, %37;\n\taddc.cc.u32 %8, %23, %38;\n\t"
+        "addc.cc.u32 %9, %24, %39;\n\taddc.cc.u32 %10, %25, %40;\n\taddc.cc.u32 %11, %26, %41;\n\t"
+        "addc.cc.u32 %12, %27, %42;\n\taddc.cc.u32 %13, %28, %43;\n\taddc.u32 %14, %29, %44;"
+        : "=r"(t[1]), "=r"(t[2]), "=r"(t[3]), "=r"(t[4]), "=r"(t[5]), "=r"(t[6]), "=r"(t[7]), "=r"(t[8]),
+          "=r"(t[9]), "=r"(t[10]), "=r"(t[11]), "=r"(t[12]), "=r"(t[13]), "=r"(t[14]), "=r"(t[15])
+        : "r"(e[1]), "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(e[8]), "r"(e[9]),
+          "r"(e[10]), "r"(e[11]), "r"(e[12]), "r"(e[13]), "r"(e[14]), "r"(e[15]), "r"(o[0]), "r"(o[1]),
+          "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]), "r"(o[8]), "r"(o[9]), "r"(o[10]),
+          "r"(o[11]), "r"(o[12]), "r"(o[13]), "r"(o[14]));
 }
 
-// out[k] = lo[k] + hi[k] + carry (k < N), out[N] = hi[N] + carry: one carry
-// chain, kept inside a single asm statement so the carry flag survives.
-template <int N> __device__ __forceinline__ void chain_add(uint32_t* out, const uint32_t* lo, const uint32_t* hi);
-template <> __device__ __forceinline__ void chain_add<1>(uint32_t* out, const uint32_t* lo, const uint32_t* hi) {
-    asm("add.cc.u32  %0, %2, %3;\n\t"
-        "addc.u32 %1, %4, 0;"
-        : "=r"(out[0]), "=r"(out[1])
-        : "r"(lo[0]), "r"(hi[0]), "r"(hi[1]));
-}
-template <> __device__ __forceinline__ void chain_add<2>(uint32_t* out, const uint32_t* lo, const uint32_t* hi) {
-    asm("add.cc.u32  %0, %3, %5;\n\t"
-        "addc.cc.u32 %1, %4, %6;\n\t"
-        "addc.u32 %2, %7, 0;"
-        : "=r"(out[0]), "=r"(out[1]), "=r"(out[2])
-        : "r"(lo[0]), "r"(lo[1]), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]));
-}
-template <> __device__ __forceinline__ void chain_add<3>(uint32_t* out, const uint32_t* lo, const uint32_t* hi) {
-    asm("add.cc.u32  %0, %4, %7;\n\t"
-        "addc.cc.u32 %1, %5, %8;\n\t"
-        "addc.cc.u32 %2, %6, %9;\n\t"
-        "addc.u32 %3, %10, 0;"
-        : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3])
-        : "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]), "r"(hi[3]));
-}
-template <> __device__ __forceinline__ void chain_add<4>(uint32_t* out, const uint32_t* lo, const uint32_t* hi) {
-    asm("add.cc.u32  %0, %5, %9;\n\t"
-        "addc.cc.u32 %1, %6, %10;\n\t"
-        "addc.cc.u32 %2, %7, %11;\n\t"
-        "addc.cc.u32 %3, %8, %12;\n\t"
-        "addc.u32 %4, %13, 0;"
-        : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3]), "=r"(out[4])
-        : "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]), "r"(hi[3]), "r"(hi[4]));
-}
-template <> __device__ __forceinline__ void chain_add<5>(uint32_t* out, const uint32_t* lo, const uint32_t* hi) {
-    asm("add.cc.u32  %0, %6, %11;\n\t"
-        "addc.cc.u32 %1, %7, %12;\n\t"
-        "addc.cc.u32 %2, %8, %13;\n\t"
-        "addc.cc.u32 %3, %9, %14;\n\t"
-        "addc.cc.u32 %4, %10, %15;\n\t"
-        "addc.u32 %5, %16, 0;"
-        : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3]), "=r"(out[4]), "=r"(out[5])
-        : "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]), "r"(lo[4]), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]), "r"(hi[3]), "r"(hi[4]), "r"(hi[5]));
-}
-template <> __device__ __forceinline__ void chain_add<6>(uint32_t* out, const uint32_t* lo, const uint32_t* hi) {
-    asm("add.cc.u32  %0, %7, %13;\n\t"
-        "addc.cc.u32 %1, %8, %14;\n\t"
-        "addc.cc.u32 %2, %9, %15;\n\t"
-        "addc.cc.u32 %3, %10, %16;\n\t"
-        "addc.cc.u32 %4, %11, %17;\n\t"
-        "addc.cc.u32 %5, %12, %18;\n\t"
-        "addc.u32 %6, %19, 0;"
-        : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3]), "=r"(out[4]), "=r"(out[5]), "=r"(out[6])
-        : "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]), "r"(lo[4]), "r"(lo[5]), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]), "r"(hi[3]), "r"(hi[4]), "r"(hi[5]), "r"(hi[6]));
-}
-template <> __device__ __forceinline__ void chain_add<7>(uint32_t* out, const uint32_t* lo, const uint32_t* hi) {
-    asm("add.cc.u32  %0, %8, %15;\n\t"
-        "addc.cc.u32 %1, %9, %16;\n\t"
-        "addc.cc.u32 %2, %10, %17;\n\t"
-        "addc.cc.u32 %3, %11, %18;\n\t"
-        "addc.cc.u32 %4, %12, %19;\n\t"
-        "addc.cc.u32 %5, %13, %20;\n\t"
-        "addc.cc.u32 %6, %14, %21;\n\t"
-        "addc.u32 %7, %22, 0;"
-        : "=r"(out[0]), "=r"(out[1]), "=r"(out[2]), "=r"(out[3]), "=r"(out[4]), "=r"(out[5]), "=r"(out[6]), "=r"(out[7])
-        : "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]), "r"(lo[4]), "r"(lo[5]), "r"(lo[6]), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]), "r"(hi[3]), "r"(hi[4]), "r"(hi[5]), "r"(hi[6]), "r"(hi[7]));
-}
-
-// Squaring with wide products: cross products row by row, doubled, plus squares.
+// t[0..15] = a^2: the 28 products a_i a_j with i < j in the same even and odd
+// columns, doubled, then one carry chain of the eight squares a_i^2.
 __device__ __forceinline__ void sqr_wide(uint32_t t[16], const fe& a) {
-    uint32_t lo[8], hi[8];
-    // row 0: a0 * a1..a7 -> t[1..8]
-#pragma unroll
-    for (int j = 1; j < 8; j++) {
-        uint64_t p = (uint64_t)a.v[0] * a.v[j];
-        lo[j] = (uint32_t)p; hi[j] = (uint32_t)(p >> 32);
-    }
-    t[1] = lo[1];
-    chain_add<6>(&t[2], &lo[2], &hi[1]);
-#define SQROW(I)                                                        \
-    {                                                                   \
-        _Pragma("unroll") for (int j = I + 1; j < 8; j++) {             \
-            uint64_t p = (uint64_t)a.v[I] * a.v[j] + t[I + j];          \
-            lo[j] = (uint32_t)p; hi[j] = (uint32_t)(p >> 32);           \
-        }                                                               \
-        t[2 * I + 1] = lo[I + 1];                                       \
-        chain_add<6 - I>(&t[2 * I + 2], &lo[I + 2], &hi[I + 1]);        \
-    }
-    SQROW(1) SQROW(2) SQROW(3) SQROW(4) SQROW(5)
-#undef SQROW
-    {
-        uint64_t p = (uint64_t)a.v[6] * a.v[7] + t[13];
-        t[13] = (uint32_t)p;
-        t[14] = (uint32_t)(p >> 32);
-    }
-    // double u[1..14] and add the squares a_i^2 at 2i
-    uint64_t d[8];
-#pragma unroll
-    for (int i = 0; i < 8; i++) d[i] = (uint64_t)a.v[i] * a.v[i];
-    asm("add.cc.u32  %1, %1, %1;\n\t"
-        "addc.cc.u32 %2, %2, %2;\n\t"
-        "addc.cc.u32 %3, %3, %3;\n\t"
-        "addc.cc.u32 %4, %4, %4;\n\t"
-        "addc.cc.u32 %5, %5, %5;\n\t"
-        "addc.cc.u32 %6, %6, %6;\n\t"
-        "addc.cc.u32 %7, %7, %7;\n\t"
-        "addc.cc.u32 %8, %8, %8;\n\t"
-        "addc.cc.u32 %9, %9, %9;\n\t"
-        "addc.cc.u32 %10, %10, %10;\n\t"
-        "addc.cc.u32 %11, %11, %11;\n\t"
-        "addc.cc.u32 %12, %12, %12;\n\t"
-        "addc.cc.u32 %13, %13, %13;\n\t"
-        "addc.cc.u32 %14, %14, %14;\n\t"
-        "addc.u32    %15, 0, 0;\n\t"
-        "mov.b32     %0, %16;\n\t"
-        "add.cc.u32  %1, %1, %17;\n\t"
-        "addc.cc.u32 %2, %2, %18;\n\t"
-        "addc.cc.u32 %3, %3, %19;\n\t"
-        "addc.cc.u32 %4, %4, %20;\n\t"
-        "addc.cc.u32 %5, %5, %21;\n\t"
-        "addc.cc.u32 %6, %6, %22;\n\t"
-        "addc.cc.u32 %7, %7, %23;\n\t"
-        "addc.cc.u32 %8, %8, %24;\n\t"
-        "addc.cc.u32 %9, %9, %25;\n\t"
-        "addc.cc.u32 %10, %10, %26;\n\t"
-        "addc.cc.u32 %11, %11, %27;\n\t"
-        "addc.cc.u32 %12, %12, %28;\n\t"
-        "addc.cc.u32 %13, %13, %29;\n\t"
-        "addc.cc.u32 %14, %14, %30;\n\t"
-        "addc.u32    %15, %15, %31;"
-        : "=r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]),
-          "+r"(t[8]), "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12]), "+r"(t[13]), "+r"(t[14]), "=r"(t[15])
-        : "r"((uint32_t)d[0]), "r"((uint32_t)(d[0] >> 32)), "r"((uint32_t)d[1]), "r"((uint32_t)(d[1] >> 32)),
-          "r"((uint32_t)d[2]), "r"((uint32_t)(d[2] >> 32)), "r"((uint32_t)d[3]), "r"((uint32_t)(d[3] >> 32)),
-          "r"((uint32_t)d[4]), "r"((uint32_t)(d[4] >> 32)), "r"((uint32_t)d[5]), "r"((uint32_t)(d[5] >> 32)),
-          "r"((uint32_t)d[6]), "r"((uint32_t)(d[6] >> 32)), "r"((uint32_t)d[7]), "r"((uint32_t)(d[7] >> 32)));
+    uint32_t e[14], o[14];
+    // Row 0: a_0 a_1, a_3, a_5, a_7 at words 1, 3, 5, 7 (o) and a_0 a_2, a_4, a_6 at 2, 4, 6 (e).
+    uint64_t p;
+#define PUT(arr, k, x, y) p = (uint64_t)(x) * (y); arr[k] = (uint32_t)p; arr[(k) + 1] = (uint32_t)(p >> 32);
+    PUT(o, 0, a.v[0], a.v[1]) PUT(o, 2, a.v[0], a.v[3]) PUT(o, 4, a.v[0], a.v[5]) PUT(o, 6, a.v[0], a.v[7])
+    PUT(e, 2, a.v[0], a.v[2]) PUT(e, 4, a.v[0], a.v[4]) PUT(e, 6, a.v[0], a.v[6])
+    // Row 1: words 3, 5, 7 (o, carry out) and 4, 6, 8 (e).
+    asm("mad.lo.cc.u32 %0,%7,%10,%0;\n\tmadc.hi.cc.u32 %1,%7,%10,%1;\n\tmadc.lo.cc.u32 %2,%8,%10,%2;\n\tmadc.hi.cc.u32 %3,%8,%10,%3;\n\t"
+        "madc.lo.cc.u32 %4,%9,%10,%4;\n\tmadc.hi.cc.u32 %5,%9,%10,%5;\n\taddc.u32 %6,0,0;"
+        : "+r"(o[2]), "+r"(o[3]), "+r"(o[4]), "+r"(o[5]), "+r"(o[6]), "+r"(o[7]), "=r"(o[8]) : "r"(a.v[2]), "r"(a.v[4]), "r"(a.v[6]), "r"(a.v[1]));
+    asm("mad.lo.cc.u32 %0,%6,%9,%0;\n\tmadc.hi.cc.u32 %1,%6,%9,%1;\n\tmadc.lo.cc.u32 %2,%7,%9,%2;\n\tmadc.hi.cc.u32 %3,%7,%9,%3;\n\t"
+        "madc.lo.cc.u32 %4,%8,%9,0;\n\tmadc.hi.u32 %5,%8,%9,0;"
+        : "+r"(e[4]), "+r"(e[5]), "+r"(e[6]), "+r"(e[7]), "=r"(e[8]), "=r"(e[9]) : "r"(a.v[3]), "r"(a.v[5]), "r"(a.v[7]), "r"(a.v[1]));
+    // Row 2: words 5, 7, 9 (o) and 6, 8 (e, carry out).
+    asm("mad.lo.cc.u32 %0,%6,%9,%0;\n\tmadc.hi.cc.u32 %1,%6,%9,%1;\n\tmadc.lo.cc.u32 %2,%7,%9,%2;\n\tmadc.hi.cc.u32 %3,%7,%9,%3;\n\t"
+        "madc.lo.cc.u32 %4,%8,%9,%4;\n\tmadc.hi.u32 %5,%8,%9,0;"
+        : "+r"(o[4]), "+r"(o[5]), "+r"(o[6]), "+r"(o[7]), "+r"(o[8]), "=r"(o[9]) : "r"(a.v[3]), "r"(a.v[5]), "r"(a.v[7]), "r"(a.v[2]));
+    asm("mad.lo.cc.u32 %0,%5,%7,%0;\n\tmadc.hi.cc.u32 %1,%5,%7,%1;\n\tmadc.lo.cc.u32 %2,%6,%7,%2;\n\tmadc.hi.cc.u32 %3,%6,%7,%3;\n\taddc.u32 %4,0,0;"
+        : "+r"(e[6]), "+r"(e[7]), "+r"(e[8]), "+r"(e[9]), "=r"(e[10]) : "r"(a.v[4]), "r"(a.v[6]), "r"(a.v[2]));
+    // Row 3: words 7, 9 (o, carry out) and 8, 10 (e).
+    asm("mad.lo.cc.u32 %0,%5,%7,%0;\n\tmadc.hi.cc.u32 %1,%5,%7,%1;\n\tmadc.lo.cc.u32 %2,%6,%7,%2;\n\tmadc.hi.cc.u32 %3,%6,%7,%3;\n\taddc.u32 %4,0,0;"
+        : "+r"(o[6]), "+r"(o[7]), "+r"(o[8]), "+r"(o[9]), "=r"(o[10]) : "r"(a.v[4]), "r"(a.v[6]), "r"(a.v[3]));
+    asm("mad.lo.cc.u32 %0,%4,%6,%0;\n\tmadc.hi.cc.u32 %1,%4,%6,%1;\n\tmadc.lo.cc.u32 %2,%5,%6,%2;\n\tmadc.hi.u32 %3,%5,%6,0;"
+        : "+r"(e[8]), "+r"(e[9]), "+r"(e[10]), "=r"(e[11]) : "r"(a.v[5]), "r"(a.v[7]), "r"(a.v[3]));
+    // Row 4: words 9, 11 (o) and 10 (e, carry out).
+    asm("mad.lo.cc.u32 %0,%4,%6,%0;\n\tmadc.hi.cc.u32 %1,%4,%6,%1;\n\tmadc.lo.cc.u32 %2,%5,%6,%2;\n\tmadc.hi.u32 %3,%5,%6,0;"
+        : "+r"(o[8]), "+r"(o[9]), "+r"(o[10]), "=r"(o[11]) : "r"(a.v[5]), "r"(a.v[7]), "r"(a.v[4]));
+    asm("mad.lo.cc.u32 %0,%3,%4,%0;\n\tmadc.hi.cc.u32 %1,%3,%4,%1;\n\taddc.u32 %2,0,0;"
+        : "+r"(e[10]), "+r"(e[11]), "=r"(e[12]) : "r"(a.v[6]), "r"(a.v[4]));
+    // Row 5: words 11 (o, carry out) and 12 (e).
+    asm("mad.lo.cc.u32 %0,%3,%4,%0;\n\tmadc.hi.cc.u32 %1,%3,%4,%1;\n\taddc.u32 %2,0,0;"
+        : "+r"(o[10]), "+r"(o[11]), "=r"(o[12]) : "r"(a.v[6]), "r"(a.v[5]));
+    asm("mad.lo.cc.u32 %0,%2,%3,%0;\n\tmadc.hi.u32 %1,%2,%3,0;" : "+r"(e[12]), "=r"(e[13]) : "r"(a.v[7]), "r"(a.v[5]));
+    // Row 6: word 13 (o).
+    asm("mad.lo.cc.u32 %0,%2,%3,%0;\n\tmadc.hi.u32 %1,%2,%3,0;" : "+r"(o[12]), "=r"(o[13]) : "r"(a.v[7]), "r"(a.v[6]));
+    // Cross products e + 2^32 o (words 1..14).
+    t[1] = o[0];
+    asm("add.cc.u32 %0,%13,%25;\n\taddc.cc.u32 %1,%14,%26;\n\taddc.cc.u32 %2,%15,%27;\n\taddc.cc.u32 %3,%16,%28;\n\taddc.cc.u32 %4,%17,%29;\n\t"
+        "addc.cc.u32 %5,%18,%30;\n\taddc.cc.u32 %6,%19,%31;\n\taddc.cc.u32 %7,%20,%32;\n\taddc.cc.u32 %8,%21,%33;\n\taddc.cc.u32 %9,%22,%34;\n\t"
+        "addc.cc.u32 %10,%23,%35;\n\taddc.cc.u32 %11,%24,%36;\n\taddc.u32 %12,%37,0;"
+        : "=r"(t[2]), "=r"(t[3]), "=r"(t[4]), "=r"(t[5]), "=r"(t[6]), "=r"(t[7]), "=r"(t[8]), "=r"(t[9]), "=r"(t[10]), "=r"(t[11]), "=r"(t[12]), "=r"(t[13]), "=r"(t[14])
+        : "r"(e[2]), "r"(e[3]), "r"(e[4]), "r"(e[5]), "r"(e[6]), "r"(e[7]), "r"(e[8]), "r"(e[9]), "r"(e[10]), "r"(e[11]), "r"(e[12]), "r"(e[13]),
+          "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]), "r"(o[8]), "r"(o[9]), "r"(o[10]), "r"(o[11]), "r"(o[12]), "r"(o[13]));
+    // Doubled, plus the squares.
+    asm("add.cc.u32 %0,%0,%0;\n\taddc.cc.u32 %1,%1,%1;\n\taddc.cc.u32 %2,%2,%2;\n\taddc.cc.u32 %3,%3,%3;\n\taddc.cc.u32 %4,%4,%4;\n\t"
+        "addc.cc.u32 %5,%5,%5;\n\taddc.cc.u32 %6,%6,%6;\n\taddc.cc.u32 %7,%7,%7;\n\taddc.cc.u32 %8,%8,%8;\n\taddc.cc.u32 %9,%9,%9;\n\t"
+        "addc.cc.u32 %10,%10,%10;\n\taddc.cc.u32 %11,%11,%11;\n\taddc.cc.u32 %12,%12,%12;\n\taddc.cc.u32 %13,%13,%13;\n\taddc.u32 %14,0,0;"
+        : "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "+r"(t[8]), "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12]), "+r"(t[13]), "+r"(t[14]), "=r"(t[15]));
+    t[0] = 0;
+    asm("mad.lo.cc.u32 %0,%16,%16,0;\n\tmadc.hi.cc.u32 %1,%16,%16,%1;\n\tmadc.lo.cc.u32 %2,%17,%17,%2;\n\tmadc.hi.cc.u32 %3,%17,%17,%3;\n\t"
+        "madc.lo.cc.u32 %4,%18,%18,%4;\n\tmadc.hi.cc.u32 %5,%18,%18,%5;\n\tmadc.lo.cc.u32 %6,%19,%19,%6;\n\tmadc.hi.cc.u32 %7,%19,%19,%7;\n\t"
+        "madc.lo.cc.u32 %8,%20,%20,%8;\n\tmadc.hi.cc.u32 %9,%20,%20,%9;\n\tmadc.lo.cc.u32 %10,%21,%21,%10;\n\tmadc.hi.cc.u32 %11,%21,%21,%11;\n\t"
+        "madc.lo.cc.u32 %12,%22,%22,%12;\n\tmadc.hi.cc.u32 %13,%22,%22,%13;\n\tmadc.lo.cc.u32 %14,%23,%23,%14;\n\tmadc.hi.u32 %15,%23,%23,%15;"
+        : "+r"(t[0]), "+r"(t[1]), "+r"(t[2]), "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "+r"(t[8]), "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12]), "+r"(t[13]), "+r"(t[14]), "+r"(t[15])
+        : "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]), "r"(a.v[6]), "r"(a.v[7]));
+#undef PUT
 }
 
 __device__ __forceinline__ void fe_mul(fe& r, const fe& a, const fe& b) {
