@@ -2,7 +2,8 @@
 // points G and H by random scalars; decryption checks candidate messages
 // against multiples of G).  The table of a point X has 32 windows of 8
 // bits; entry (window i, value v) is (v 2^(8i)) X, stored affine and
-// quad-planar with stride COMB_POINTS (entries with v = 0 are unused).
+// quad-planar with stride COMB_POINTS, in canonical standard coordinates
+// (entries with v = 0 are unused).
 #pragma once
 #include <stdint.h>
 
@@ -23,6 +24,7 @@ __device__ __forceinline__ void comb_mul_u64(jac& R, const uint4* __restrict__ t
         const uint32_t v = (uint32_t)(s >> (8 * win)) & 0xffu;
         if (v) {
             load_aff(T, tab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
+            aff_to_mont(T);
             jac_madd(R, T);
         }
     }

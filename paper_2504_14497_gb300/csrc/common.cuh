@@ -151,7 +151,7 @@ __device__ __forceinline__ bool group_all(bool x, bool shared) {
     return shared ? __syncthreads_and(x) != 0 : __all_sync(0xffffffffu, x);
 }
 
-// Normalise E Jacobian points held in each lane's registers to canonical
+// Normalise E Jacobian points held in each lane's registers to
 // affine coordinates; infinity (Z = 0) becomes (0, 0).  One inversion per
 // warp for 32 * E points.  All 32 lanes must call.
 template <int E>

@@ -460,7 +460,7 @@ __device__ __forceinline__ void lp_pref_step(fe& acc, bool& ones, const fe& Z, u
 }
 
 // Backward half of the normalisation of E lane-planar Jacobian entries to
-// canonical affine (infinity -> (0, 0)), each handed to store(e, point):
+// affine (infinity -> (0, 0)), each handed to store(e, point):
 // pref holds the per-lane prefix products of the Z's and acc their total
 // (lp_pref_step).  One warp-wide inversion; when every Z in the warp is 1 the
 // entries are copied without any.  The loads of entry e - 2 are prefetched
@@ -476,8 +476,8 @@ __device__ __forceinline__ void lp_normalize_back(const uint4* src, int E, const
             jac Pe;
             lp_load_jac(Pe, src, e, lane);
             aff out;
-            fe_canon(out.x, Pe.X);
-            fe_canon(out.y, Pe.Y);
+            out.x = Pe.X;
+            out.y = Pe.Y;
             store(e, out);
         }
         return;
@@ -540,7 +540,10 @@ __device__ __forceinline__ void lp_normalize(const uint4* src, int E, uint4* pre
 // ZZ^-1 and ZZZ^-1 of the last entry; going backwards each step multiplies
 // them by the entry's factors: 4M per entry in all.  ones: every factor of
 // this lane is 1.  With `shared` all threads of the block must call.
-template <class Store>
+// STD: the points handed to store are canonical standard coordinates (the
+// walk then starts from ZZ^-1 / R and ZZZ^-1 / R, and every product with X and
+// Y is standard); otherwise they stay in the Montgomery domain.
+template <bool STD, class Store>
 __device__ __forceinline__ void lp_normalize_zz(const uint4* src, int E, const uint4* rat, unsigned lane,
                                                 const fe& zz, const fe& zzz, bool ones, Store store,
                                                 bool shared) {
@@ -551,8 +554,7 @@ __device__ __forceinline__ void lp_normalize_zz(const uint4* src, int E, const u
             aff out;
             fe_from_quads(out.x, b[0], b[32]);
             fe_from_quads(out.y, b[64], b[96]);
-            fe_canon(out.x, out.x);
-            fe_canon(out.y, out.y);
+            if (STD) aff_from_mont(out);
             store(e, out);
         }
         return;
@@ -561,6 +563,10 @@ __device__ __forceinline__ void lp_normalize_zz(const uint4* src, int E, const u
     group_inverse(inv, fmul(zz, zzz), shared);
     fe zzinv = fmul(inv, zzz);
     fe zzzinv = fmul(inv, zz);
+    if (STD) {
+        fe_from_mont(zzinv, zzinv);
+        fe_from_mont(zzzinv, zzzinv);
+    }
     for (int e = E - 1; e >= 0; e--) {
         if (e >= 2) {
             // lanes 0-23: the 24 lines of slot e - 2; 24-31: its ZZ factor.
@@ -575,8 +581,10 @@ __device__ __forceinline__ void lp_normalize_zz(const uint4* src, int E, const u
         aff out;
         out.x = fmul(X, zzinv);
         out.y = fmul(Y, zzzinv);
-        fe_canon(out.x, out.x);
-        fe_canon(out.y, out.y);
+        if (STD) {
+            fe_canon(out.x, out.x);
+            fe_canon(out.y, out.y);
+        }
         store(e, out);
         if (e > 0) {
             fe r2, r3;
@@ -646,8 +654,15 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
 
     const int E = P.nent[s];
     const size_t tbase = (size_t)s_local * a.emax;
+    // The strip table holds canonical standard coordinates; everything else
+    // in this function is in the Montgomery domain.
     auto store_table = [&](int e, const aff& q) {
         store_aff(a.table, a.table_points, ((tbase + e) * 2 + c) * a.lp + j, q);
+    };
+    auto store_table_mont = [&](int e, const aff& q) {
+        aff t = q;
+        aff_from_mont(t);
+        store_table(e, t);
     };
     bool bad = false, dbad = false;
 
@@ -655,6 +670,7 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
         const int col = c0 + t;
         aff Pb;
         load_aff(Pb, Bc, nl, (size_t)col * a.l + jj);
+        aff_to_mont(Pb);
         int lens[NLEV];
 #pragma unroll
         for (int q = 0; q < NLEV; q++) lens[q] = P.col_len[(size_t)col * NLEV + q];
@@ -719,7 +735,7 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
             bool ones2, ok2;
             lp_affine_chain(l2aff, col_level_ptr(P, col, 2), lens[1], alt, pref, lane, acc2, ones2, ok2);
             if (group_all(ok2, a.bshare)) {
-                lp_normalize_zz(alt, lens[1], pref, lane, acc2.ZZ, acc2.ZZZ, ones2, store_l2, a.bshare);
+                lp_normalize_zz<false>(alt, lens[1], pref, lane, acc2.ZZ, acc2.ZZZ, ones2, store_l2, a.bshare);
             } else {
                 jacobian_level(2);
                 lp_normalize_back(alt, lens[1], pref, lane, pacc, pones, store_l2, a.bshare);
@@ -750,11 +766,11 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
         auto store_col = [&](int e, const aff& q) { lp_store_aff(ca, e, lane, q); };
         if (a.k == 1) {
             // The column table is the strip table (E = lens[0] entries).
-            if (chain_ok) lp_normalize_zz(coltab, E, pref, lane, acc.ZZ, acc.ZZZ, cones, store_table, a.bshare);
-            else lp_normalize(coltab, E, pref, lane, store_table, a.bshare);
+            if (chain_ok) lp_normalize_zz<true>(coltab, E, pref, lane, acc.ZZ, acc.ZZZ, cones, store_table, a.bshare);
+            else lp_normalize(coltab, E, pref, lane, store_table_mont, a.bshare);
             return;
         }
-        if (chain_ok) lp_normalize_zz(coltab, lens[0], pref, lane, acc.ZZ, acc.ZZZ, cones, store_col, a.bshare);
+        if (chain_ok) lp_normalize_zz<false>(coltab, lens[0], pref, lane, acc.ZZ, acc.ZZZ, cones, store_col, a.bshare);
         else lp_normalize(coltab, lens[0], pref, lane, store_col, a.bshare);
     }
     if (bad) {
@@ -864,8 +880,6 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
                 fe_sub(t0, Pp.x, R.x);
                 t0 = fmul(lam, t0);
                 fe_sub(R.y, t0, Pp.y);             // y3 = lam (x1 - x3) - y1
-                fe_canon(R.x, R.x);
-                fe_canon(R.y, R.y);
             } else {
                 jac J;
                 jac_from_aff(J, Pp);
@@ -888,7 +902,7 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
         aff R;
         if (comp(code, 1, v1) < 0) col_entry(R, comp(code, 0, v0), v0);   // a single component
         else lp_load_aff(R, part, e, lane);
-        store_table(e, R);
+        store_table_mont(e, R);
     }
 }
 
@@ -925,7 +939,8 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, const PlanPtrs&
     const size_t ml = (size_t)a.m * a.l;
     uint4* Cc = (a.parts > 1 ? a.partial + (size_t)part * 12 * ml : a.ctC) + (size_t)c * 6 * ml;
     // The running sum is kept as (X, Y, Z^2, Z^3): its mixed additions then
-    // cost 8M + 2S, and Z itself is rebuilt once at the end.
+    // cost 8M + 2S, and Z itself is rebuilt once at the end.  The table
+    // entries are standard, so Z^2 and Z^3 carry the factor R (ec.cuh).
     jacz acc;
     if (a.first || a.parts > 1 || j >= a.l) {
         jacz_set_inf(acc);
@@ -933,13 +948,49 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, const PlanPtrs&
         jac prev;
         if (CG) load_jac_cg(prev, Cc, ml, (size_t)i * a.l + j);
         else load_jac(prev, Cc, ml, (size_t)i * a.l + j);
+        jac_to_mont(prev);
         jacz_from_jac(acc, prev);
+        jacz_add_R(acc);
     }
     const uint16_t* rk = P.rank + (size_t)a.s0 * a.m + i;
     aff T;
     const int s_lo = (int)((long long)a.nstrips_chunk * part / a.parts);
     const int s_hi = (int)((long long)a.nstrips_chunk * (part + 1) / a.parts);
-    for (int sl = s_lo; sl < s_hi; sl++) {
+    auto entry = [&](aff& Q, int sl, uint16_t code) {
+        const size_t ti = (((size_t)sl * a.emax + code) * 2 + c) * a.lp + j;
+        if (CG) load_aff_cg(Q, a.table, a.table_points, ti);
+        else load_aff(Q, a.table, a.table_points, ti);
+    };
+    int sl = s_lo;
+#ifndef PCMM_DEBUG_BOUNDS
+    if (a.first || a.parts > 1) {
+        // The first entry starts the sum; if no second one follows, the sum is
+        // that entry and leaves as it is, with Z = 1 (0 at infinity).
+        while (sl < s_hi && rk[(size_t)sl * a.m] == NO_RANK) sl++;
+        if (sl < s_hi) {
+            entry(T, sl, rk[(size_t)sl * a.m]);
+            sl++;
+            while (sl < s_hi && rk[(size_t)sl * a.m] == NO_RANK) sl++;
+            if (sl == s_hi) {
+                jac out;
+                out.X = T.x;
+                out.Y = T.y;
+                fe_zero(out.Z);
+                out.Z.v[0] = aff_is_inf(T) ? 0u : 1u;
+                if (a.parts > 1) jac_to_mont(out);
+                if (j < a.l) store_jac(Cc, ml, (size_t)i * a.l + j, out);
+                return;
+            }
+            if (!aff_is_inf(T)) {
+                fe_to_mont(acc.X, T.x);
+                fe_to_mont(acc.Y, T.y);
+                fe_set_R2(acc.ZZ);
+                fe_set_R2(acc.ZZZ);
+            }
+        }
+    }
+#endif
+    for (; sl < s_hi; sl++) {
         const uint16_t code = rk[(size_t)sl * a.m];
         if (code == NO_RANK) continue;
 #ifdef PCMM_DEBUG_BOUNDS
@@ -948,14 +999,14 @@ __device__ __forceinline__ void gather_item(const GatherArgs& a, const PlanPtrs&
             continue;
         }
 #endif
-        const size_t ti = (((size_t)sl * a.emax + code) * 2 + c) * a.lp + j;
-        if (CG) load_aff_cg(T, a.table, a.table_points, ti);
-        else load_aff(T, a.table, a.table_points, ti);
-        jacz_madd_t<PCMM_GATHER_INLINE>(acc, T);
+        entry(T, sl, code);
+        jacz_madd_t<PCMM_GATHER_INLINE, true>(acc, T);
     }
     if (j < a.l) {
         jac out;
+        jacz_drop_R(acc);
         jac_from_jacz(out, acc);
+        if (a.parts == 1) jac_from_mont(out);   // partial sums stay in the Montgomery domain
         store_jac(Cc, ml, (size_t)i * a.l + j, out);
     }
 }

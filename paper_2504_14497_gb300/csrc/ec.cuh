@@ -18,6 +18,10 @@
 // (doubling) and P = -Q (result infinity) are detected and handled on a rare
 // branch.
 //
+// Inside the kernels coordinates are in the Montgomery domain (fp256.cuh);
+// *_to_mont and *_from_mont convert points at loads and stores of standard
+// coordinates.  Only the point at infinity looks the same in both.
+//
 // Point arrays in global memory are QUAD-PLANAR: an array of N points stores
 // coordinate quad q (4 consecutive 32-bit limbs) of point i at uint4 index
 // q * N + i.  Affine points have 4 quads (x lo, x hi, y lo, y hi), Jacobian
@@ -35,6 +39,31 @@ struct aff {
 struct jac {
     fe X, Y, Z;
 };
+
+__device__ __forceinline__ void aff_to_mont(aff& Q) {
+    fe_to_mont(Q.x, Q.x);
+    fe_to_mont(Q.y, Q.y);
+}
+
+// Canonical standard coordinates.
+__device__ __forceinline__ void aff_from_mont(aff& Q) {
+    fe_from_mont(Q.x, Q.x);
+    fe_from_mont(Q.y, Q.y);
+    fe_canon(Q.x, Q.x);
+    fe_canon(Q.y, Q.y);
+}
+
+__device__ __forceinline__ void jac_to_mont(jac& P) {
+    fe_to_mont(P.X, P.X);
+    fe_to_mont(P.Y, P.Y);
+    fe_to_mont(P.Z, P.Z);
+}
+
+__device__ __forceinline__ void jac_from_mont(jac& P) {
+    fe_from_mont(P.X, P.X);
+    fe_from_mont(P.Y, P.Y);
+    fe_from_mont(P.Z, P.Z);
+}
 
 __device__ __forceinline__ void jac_set_inf(jac& P) {
     fe_one(P.X);
@@ -169,10 +198,27 @@ __device__ __forceinline__ void jac_from_jacz(jac& R, const jacz& P) {
     R.Z = fmul(P.ZZ, P.ZZZ);
 }
 
+// An accumulator of points whose affine coordinates are STANDARD residues
+// (table entries and comb entries as they lie in memory) is a jacz whose ZZ
+// and ZZZ hold an additional factor R: U2 = ZZ x and S2 = ZZZ y then come out
+// in the Montgomery domain without converting x and y, the updates ZZ H^2 and
+// ZZZ H^3 keep the factor, and nothing else in the addition sees it.
+// jacz_drop_R and jacz_add_R convert between the two forms.
+__device__ __forceinline__ void jacz_drop_R(jacz& P) {
+    fe_from_mont(P.ZZ, P.ZZ);
+    fe_from_mont(P.ZZZ, P.ZZZ);
+}
+
+__device__ __forceinline__ void jacz_add_R(jacz& P) {
+    fe_to_mont(P.ZZ, P.ZZ);
+    fe_to_mont(P.ZZZ, P.ZZZ);
+}
+
+// STD: Q has standard coordinates and P the additional factor R (above).
 // INL: which field operations are inlined (bit 0 the squarings, bit 1 the
 // fused a b - c d, bit 2 U2 and S2, bit 3 H^3 and the ZZ, ZZZ updates,
 // bit 4 X1 H^2); the rest run out of line.
-template <int INL>
+template <int INL, bool STD>
 __device__ __forceinline__ void jacz_madd_t(jacz& P, const aff& Q) {
     constexpr bool IS = (INL & 1) != 0, IF = (INL & 2) != 0, IU = (INL & 4) != 0, IZ = (INL & 8) != 0,
                    IX = (INL & 16) != 0;
@@ -180,8 +226,15 @@ __device__ __forceinline__ void jacz_madd_t(jacz& P, const aff& Q) {
     if (fe_is_zero(P.ZZ)) {
         P.X = Q.x;
         P.Y = Q.y;
-        fe_one(P.ZZ);
-        fe_one(P.ZZZ);
+        if (STD) {
+            fe_to_mont(P.X, P.X);
+            fe_to_mont(P.Y, P.Y);
+            fe_set_R2(P.ZZ);
+            fe_set_R2(P.ZZZ);
+        } else {
+            fe_one(P.ZZ);
+            fe_one(P.ZZZ);
+        }
         return;
     }
     fe t1, t2, t3, t4, x3;
@@ -191,10 +244,13 @@ __device__ __forceinline__ void jacz_madd_t(jacz& P, const aff& Q) {
     fe_sub(t2, t2, P.Y);             // R
     if (fe_is_zero(t1)) {
         if (fe_is_zero(t2)) {        // P = Q: the result is 2Q, from Q's affine coordinates
+            aff M = Q;
+            if (STD) aff_to_mont(M);
             jac D;
-            jac_from_aff(D, Q);
+            jac_from_aff(D, M);
             jac_dbl(D);
             jacz_from_jac(P, D);
+            if (STD) jacz_add_R(P);
         } else {                     // P = -Q
             jacz_set_inf(P);
         }
@@ -213,8 +269,6 @@ __device__ __forceinline__ void jacz_madd_t(jacz& P, const aff& Q) {
     P.Y = mulsub_t<IF>(t4, t2, t3, P.Y);  // Y3 = R (X1 H^2 - X3) - Y1 H^3
     P.X = x3;
 }
-
-__device__ __forceinline__ void jacz_madd(jacz& P, const aff& Q) { jacz_madd_t<0>(P, Q); }
 
 // Doubling in (X, Y, ZZ, ZZZ) coordinates (dbl-2001-b with delta = ZZ): Z
 // would become 2 Y Z, so ZZ is multiplied by rr2 = 4 Y^2 and ZZZ by
@@ -421,14 +475,12 @@ __device__ __forceinline__ void store_fe(uint4* __restrict__ base, size_t stride
     base[stride + i] = fe_hi(a);
 }
 
-// Affine from Jacobian given zinv = Z^-1 (Z != 0); canonical output.
+// Affine from Jacobian given zinv = Z^-1 (Z != 0).
 __device__ __forceinline__ void jac_to_aff_with_zinv(aff& Q, const jac& P, const fe& zinv) {
     fe z2 = fsqr(zinv);
     fe z3 = fmul(z2, zinv);
     Q.x = fmul(P.X, z2);
     Q.y = fmul(P.Y, z3);
-    fe_canon(Q.x, Q.x);
-    fe_canon(Q.y, Q.y);
 }
 
 }  // namespace pcmm

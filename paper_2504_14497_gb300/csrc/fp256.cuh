@@ -1,11 +1,14 @@
 // Prime-field arithmetic in F_p for NIST P-256, p = 2^256 - 2^224 + 2^192 + 2^96 - 1
 // (Section 4.1), on sm_103a.
 //
-// Representation: 8 x 32-bit little-endian limbs held in registers.  Values
-// are kept WEAKLY reduced: any integer in [0, 2^256) that is congruent to the
-// field element (so 0 may appear as 0 or as p).  fe_canon() gives the unique
-// representative below p; it is applied only when a result leaves the
-// library or when a value must be compared.
+// Representation: 8 x 32-bit little-endian limbs held in registers, in the
+// MONTGOMERY domain with R = 2^256: the field element x is held as x R mod p.
+// Values are kept WEAKLY reduced: any integer in [0, 2^256) that is congruent
+// to x R (so 0 may appear as 0 or as p).  fe_canon() gives the unique
+// representative below p.  Everything outside the kernels (inputs, strip
+// tables, results, comb tables) is standard: fe_to_mont and fe_from_mont
+// convert at the kernels' loads and stores, or the conversion is folded into
+// a factor that is there anyway (see jacz in ec.cuh).
 //
 // Multiplication: 8x8-limb operand scanning, one row per limb of b, with the
 // products of even and odd word positions in two accumulators, so that every
@@ -18,18 +21,20 @@
 // running word as a zero-extended 64-bit addend and folding the high halves
 // in with addc took a register move per product beside 57 additions:
 // 385 cycles a product against 290, 530 a multiplication against 437.
-// Squaring: 28 cross products, doubled, plus 8 diagonal squares (420 -> 350
-// cycles with the reduction).  Products
+// Squaring: 28 cross products, doubled, plus 8 diagonal squares.  Products
 // and reductions live in out-of-line functions (fmul, fsqr): inlining them
 // into every call site of a point formula overflows the instruction cache.
-// Reduction of the 512-bit product uses the
-// special form of p (Solinas, FIPS 186-4 D.2): with 2^256 = 2^224 - 2^192 -
-// 2^96 + 1 (mod p), the product c = (c15..c0) reduces to
-//     T + 2 S1 + 2 S2 + S3 + S4 - D1 - D2 - D3 - D4       (mod p)
-// where each term is an 8-word rearrangement of the c_i (spelled out in
-// fe_reduce).  A bias of 5p keeps the intermediate non-negative, after which
-// two folds of the top word by 2^256 = K (mod p) bring it below 2^256.
-// No multiplications are spent on reduction.
+//
+// Reduction of the 512-bit product t to t / R mod p: since p = -1 mod 2^96,
+// the three lowest words q of t cancel against q p, which leaves (after the
+// shift by 96 bits) t / 2^96 + q (2^160 - 2^128 + 2^96 + 1): with D = q (2^64
+// - 2^32 + 1), five words from seven additions, one carry chain of eight adds
+// (q, D).  Steps of 3, 3 and 2 words clear all eight: about 54 additions and
+// no multiplications.  Measured per warp and scheduler: 104 cycles, against
+// 205 for the special-form (Solinas) reduction of a standard residue, whose
+// nine rearranged terms need 96 additions; a multiplication takes 323 cycles
+// inlined and 352 called (437 and 448 with the special-form reduction), a
+// squaring 270 and 280.
 #pragma once
 #include <stdint.h>
 
@@ -49,10 +54,23 @@ __device__ __forceinline__ void fe_zero(fe& r) {
     for (int i = 0; i < 8; i++) r.v[i] = 0;
 }
 
+// The field element 1: R mod p = K.
 __device__ __forceinline__ void fe_one(fe& r) {
-    r.v[0] = 1;
-#pragma unroll
-    for (int i = 1; i < 8; i++) r.v[i] = 0;
+    r.v[0] = PCMM_K0;
+    r.v[1] = r.v[2] = 0;
+    r.v[3] = r.v[4] = r.v[5] = PCMM_K3;
+    r.v[6] = PCMM_K6;
+    r.v[7] = 0;
+}
+
+// R^2 mod p and R^3 mod p.
+__device__ __forceinline__ void fe_set_R2(fe& r) {
+    r.v[0] = 3u; r.v[1] = 0u; r.v[2] = 0xffffffffu; r.v[3] = 0xfffffffbu;
+    r.v[4] = 0xfffffffeu; r.v[5] = 0xffffffffu; r.v[6] = 0xfffffffdu; r.v[7] = 4u;
+}
+__device__ __forceinline__ void fe_set_R3(fe& r) {
+    r.v[0] = 0x0000000au; r.v[1] = 0xfffffffdu; r.v[2] = 0xfffffff7u; r.v[3] = 0xffffffedu;
+    r.v[4] = 0xfffffffcu; r.v[5] = 0x00000005u; r.v[6] = 0x00000001u; r.v[7] = 0x00000018u;
 }
 
 // r += mask & K (mask is 0 or 0xffffffff); returns the carry out.
@@ -176,161 +194,89 @@ __device__ __forceinline__ bool fe_equal(const fe& a, const fe& b) {
     return fe_is_zero(d);
 }
 
-// Whether a holds exactly the word representation of 1 (a value of 1 + p,
-// which weakly reduced arithmetic could produce, is not recognised; callers
-// use this only to skip work when it says yes).
+// Whether a holds exactly the canonical words of 1 (the congruent value
+// above p, which weakly reduced arithmetic could produce, is not recognised;
+// callers use this only to skip work when it says yes).
 __device__ __forceinline__ bool fe_is_one(const fe& a) {
-    uint32_t z = (a.v[0] ^ 1u) | a.v[1] | a.v[2] | a.v[3] | a.v[4] | a.v[5] | a.v[6] | a.v[7];
+    uint32_t z = (a.v[0] ^ PCMM_K0) | a.v[1] | a.v[2] | (a.v[3] ^ PCMM_K3) | (a.v[4] ^ PCMM_K3) |
+                 (a.v[5] ^ PCMM_K3) | (a.v[6] ^ PCMM_K6) | a.v[7];
     return z == 0u;
 }
 
-// Reduce the 512-bit value c[0..15] modulo p into r (weak).
-__device__ __forceinline__ void fe_reduce(fe& r, const uint32_t c[16]) {
-    uint32_t a0, a1, a2, a3, a4, a5, a6, a7, a8;
-    uint32_t u3, u4, u5, u6, u7, u8;
-    // u = S1 + S2 on words 3..8:  S1 = (c11..c15) at words 3..7,
-    //                             S2 = (c12..c15) at words 3..6.
-    asm("add.cc.u32  %0, %6, %7;\n\t"
-        "addc.cc.u32 %1, %7, %8;\n\t"
-        "addc.cc.u32 %2, %8, %9;\n\t"
-        "addc.cc.u32 %3, %9, %10;\n\t"
-        "addc.cc.u32 %4, %10, 0;\n\t"
-        "addc.u32    %5, 0, 0;\n\t"
-        // u = 2u
-        "add.cc.u32  %0, %0, %0;\n\t"
-        "addc.cc.u32 %1, %1, %1;\n\t"
-        "addc.cc.u32 %2, %2, %2;\n\t"
-        "addc.cc.u32 %3, %3, %3;\n\t"
-        "addc.cc.u32 %4, %4, %4;\n\t"
-        "addc.u32    %5, %5, %5;"
-        : "=r"(u3), "=r"(u4), "=r"(u5), "=r"(u6), "=r"(u7), "=r"(u8)
-        : "r"(c[11]), "r"(c[12]), "r"(c[13]), "r"(c[14]), "r"(c[15]));
-    // a = T + 5p, with 5p = (4, fffffffb, 5, 0, 0, 4, ffffffff, ffffffff, fffffffb)
-    //                       word 8 .................................... word 0
-    asm("add.cc.u32  %0, %9, 0xfffffffb;\n\t"
-        "addc.cc.u32 %1, %10, 0xffffffff;\n\t"
-        "addc.cc.u32 %2, %11, 0xffffffff;\n\t"
-        "addc.cc.u32 %3, %12, 4;\n\t"
-        "addc.cc.u32 %4, %13, 0;\n\t"
-        "addc.cc.u32 %5, %14, 0;\n\t"
-        "addc.cc.u32 %6, %15, 5;\n\t"
-        "addc.cc.u32 %7, %16, 0xfffffffb;\n\t"
-        "addc.u32    %8, 4, 0;"
-        : "=r"(a0), "=r"(a1), "=r"(a2), "=r"(a3), "=r"(a4), "=r"(a5), "=r"(a6), "=r"(a7),
-          "=r"(a8)
-        : "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]), "r"(c[4]), "r"(c[5]), "r"(c[6]),
-          "r"(c[7]));
-    // a += 2 (S1 + S2)
-    asm("add.cc.u32  %0, %0, %6;\n\t"
-        "addc.cc.u32 %1, %1, %7;\n\t"
-        "addc.cc.u32 %2, %2, %8;\n\t"
-        "addc.cc.u32 %3, %3, %9;\n\t"
-        "addc.cc.u32 %4, %4, %10;\n\t"
-        "addc.u32    %5, %5, %11;"
-        : "+r"(a3), "+r"(a4), "+r"(a5), "+r"(a6), "+r"(a7), "+r"(a8)
-        : "r"(u3), "r"(u4), "r"(u5), "r"(u6), "r"(u7), "r"(u8));
-    // a += S3 = (c15, c14, 0, 0, 0, c10, c9, c8)
-    // a += S4 = (c8, c13, c15, c14, c13, c11, c10, c9)
+// r = t / R mod p (weak) for any 512-bit t; t is clobbered.
+__device__ __forceinline__ void fe_reduce(fe& r, uint32_t t[16]) {
+    uint32_t D1, D2, D3, D4, c;
+    // Words 0..2 (q): D = q (2^64 - 2^32 + 1) = (q0, D1, D2, D3, D4), then
+    // words 3..10 += (q0, q1, q2, q0, D1, D2, D3, D4), carry c into word 11.
+    asm("add.cc.u32  %1, %6, %4;\n\t"
+        "addc.cc.u32 %2, %5, 0;\n\t"
+        "addc.u32    %3, %6, 0;\n\t"
+        "sub.cc.u32  %0, %5, %4;\n\t"
+        "subc.cc.u32 %1, %1, %5;\n\t"
+        "subc.cc.u32 %2, %2, %6;\n\t"
+        "subc.u32    %3, %3, 0;"
+        : "=&r"(D1), "=&r"(D2), "=&r"(D3), "=&r"(D4)
+        : "r"(t[0]), "r"(t[1]), "r"(t[2]));
     asm("add.cc.u32  %0, %0, %9;\n\t"
         "addc.cc.u32 %1, %1, %10;\n\t"
         "addc.cc.u32 %2, %2, %11;\n\t"
-        "addc.cc.u32 %3, %3, 0;\n\t"
-        "addc.cc.u32 %4, %4, 0;\n\t"
-        "addc.cc.u32 %5, %5, 0;\n\t"
-        "addc.cc.u32 %6, %6, %15;\n\t"
-        "addc.cc.u32 %7, %7, %16;\n\t"
-        "addc.u32    %8, %8, 0;\n\t"
-        "add.cc.u32  %0, %0, %10;\n\t"
-        "addc.cc.u32 %1, %1, %11;\n\t"
-        "addc.cc.u32 %2, %2, %12;\n\t"
-        "addc.cc.u32 %3, %3, %14;\n\t"
-        "addc.cc.u32 %4, %4, %15;\n\t"
-        "addc.cc.u32 %5, %5, %16;\n\t"
+        "addc.cc.u32 %3, %3, %9;\n\t"
+        "addc.cc.u32 %4, %4, %12;\n\t"
+        "addc.cc.u32 %5, %5, %13;\n\t"
         "addc.cc.u32 %6, %6, %14;\n\t"
-        "addc.cc.u32 %7, %7, %9;\n\t"
-        "addc.u32    %8, %8, 0;"
-        : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3), "+r"(a4), "+r"(a5), "+r"(a6), "+r"(a7),
-          "+r"(a8)
-        : "r"(c[8]), "r"(c[9]), "r"(c[10]), "r"(c[11]), "r"(c[12]), "r"(c[13]), "r"(c[14]),
-          "r"(c[15]));
-    // a -= D1 = (c10, c8, 0, 0, 0, c13, c12, c11)
-    // a -= D2 = (c11, c9, 0, 0, c15, c14, c13, c12)
-    asm("sub.cc.u32  %0, %0, %12;\n\t"
-        "subc.cc.u32 %1, %1, %13;\n\t"
-        "subc.cc.u32 %2, %2, %14;\n\t"
-        "subc.cc.u32 %3, %3, 0;\n\t"
-        "subc.cc.u32 %4, %4, 0;\n\t"
-        "subc.cc.u32 %5, %5, 0;\n\t"
-        "subc.cc.u32 %6, %6, %9;\n\t"
-        "subc.cc.u32 %7, %7, %11;\n\t"
-        "subc.u32    %8, %8, 0;\n\t"
-        "sub.cc.u32  %0, %0, %13;\n\t"
-        "subc.cc.u32 %1, %1, %14;\n\t"
-        "subc.cc.u32 %2, %2, %15;\n\t"
-        "subc.cc.u32 %3, %3, %16;\n\t"
-        "subc.cc.u32 %4, %4, 0;\n\t"
-        "subc.cc.u32 %5, %5, 0;\n\t"
-        "subc.cc.u32 %6, %6, %10;\n\t"
-        "subc.cc.u32 %7, %7, %12;\n\t"
-        "subc.u32    %8, %8, 0;"
-        : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3), "+r"(a4), "+r"(a5), "+r"(a6), "+r"(a7),
-          "+r"(a8)
-        : "r"(c[8]), "r"(c[9]), "r"(c[10]), "r"(c[11]), "r"(c[12]), "r"(c[13]), "r"(c[14]),
-          "r"(c[15]));
-    // a -= D3 = (c12, 0, c10, c9, c8, c15, c14, c13)
-    // a -= D4 = (c13, 0, c11, c10, c9, 0, c15, c14)
-    asm("sub.cc.u32  %0, %0, %14;\n\t"
-        "subc.cc.u32 %1, %1, %15;\n\t"
-        "subc.cc.u32 %2, %2, %16;\n\t"
-        "subc.cc.u32 %3, %3, %9;\n\t"
-        "subc.cc.u32 %4, %4, %10;\n\t"
-        "subc.cc.u32 %5, %5, %11;\n\t"
-        "subc.cc.u32 %6, %6, 0;\n\t"
-        "subc.cc.u32 %7, %7, %13;\n\t"
-        "subc.u32    %8, %8, 0;\n\t"
-        "sub.cc.u32  %0, %0, %15;\n\t"
-        "subc.cc.u32 %1, %1, %16;\n\t"
-        "subc.cc.u32 %2, %2, 0;\n\t"
-        "subc.cc.u32 %3, %3, %10;\n\t"
-        "subc.cc.u32 %4, %4, %11;\n\t"
-        "subc.cc.u32 %5, %5, %12;\n\t"
-        "subc.cc.u32 %6, %6, 0;\n\t"
-        "subc.cc.u32 %7, %7, %14;\n\t"
-        "subc.u32    %8, %8, 0;"
-        : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3), "+r"(a4), "+r"(a5), "+r"(a6), "+r"(a7),
-          "+r"(a8)
-        : "r"(c[8]), "r"(c[9]), "r"(c[10]), "r"(c[11]), "r"(c[12]), "r"(c[13]), "r"(c[14]),
-          "r"(c[15]));
-    // Now 0 <= a < 12 * 2^256: fold the top word t = a8 with 2^256 = K:
-    //   low + t + t 2^224 - t 2^96 - t 2^192.
-    uint32_t e1, b1;
-    asm("add.cc.u32  %0, %0, %9;\n\t"
-        "addc.cc.u32 %1, %1, 0;\n\t"
-        "addc.cc.u32 %2, %2, 0;\n\t"
-        "addc.cc.u32 %3, %3, 0;\n\t"
-        "addc.cc.u32 %4, %4, 0;\n\t"
-        "addc.cc.u32 %5, %5, 0;\n\t"
-        "addc.cc.u32 %6, %6, 0;\n\t"
-        "addc.cc.u32 %7, %7, %9;\n\t"
+        "addc.cc.u32 %7, %7, %15;\n\t"
         "addc.u32    %8, 0, 0;"
-        : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3), "+r"(a4), "+r"(a5), "+r"(a6), "+r"(a7),
-          "=r"(e1)
-        : "r"(a8));
-    asm("sub.cc.u32  %3, %3, %9;\n\t"
-        "subc.cc.u32 %4, %4, 0;\n\t"
-        "subc.cc.u32 %5, %5, 0;\n\t"
-        "subc.cc.u32 %6, %6, %9;\n\t"
-        "subc.cc.u32 %7, %7, 0;\n\t"
-        "subc.u32    %8, 0, 0;"
-        : "+r"(a0), "+r"(a1), "+r"(a2), "+r"(a3), "+r"(a4), "+r"(a5), "+r"(a6), "+r"(a7),
-          "=r"(b1)
-        : "r"(a8));
-    // The folded value is non-negative and below 2^256 + 11 * 2^224, so the
-    // net top word e1 + b1 (b1 is 0 or -1) is 0 or 1; it is 1 only when the
-    // value reached 2^256 (probability below 2^-27), handled on a branch.
-    r.v[0] = a0; r.v[1] = a1; r.v[2] = a2; r.v[3] = a3;
-    r.v[4] = a4; r.v[5] = a5; r.v[6] = a6; r.v[7] = a7;
-    if (e1 + b1) fe_add_K_masked(r, 0xffffffffu);
+        : "+r"(t[3]), "+r"(t[4]), "+r"(t[5]), "+r"(t[6]), "+r"(t[7]), "+r"(t[8]), "+r"(t[9]), "+r"(t[10]),
+          "=r"(c)
+        : "r"(t[0]), "r"(t[1]), "r"(t[2]), "r"(D1), "r"(D2), "r"(D3), "r"(D4));
+    // Words 3..5: the same, with the carry c (word 11) joining D2; D stays
+    // below 2^160 with it.  New carry c into word 14.
+    asm("add.cc.u32  %1, %7, 0xffffffff;\n\t"
+        "addc.cc.u32 %1, %6, %4;\n\t"
+        "addc.cc.u32 %2, %5, 0;\n\t"
+        "addc.u32    %3, %6, 0;\n\t"
+        "sub.cc.u32  %0, %5, %4;\n\t"
+        "subc.cc.u32 %1, %1, %5;\n\t"
+        "subc.cc.u32 %2, %2, %6;\n\t"
+        "subc.u32    %3, %3, 0;"
+        : "=&r"(D1), "=&r"(D2), "=&r"(D3), "=&r"(D4)
+        : "r"(t[3]), "r"(t[4]), "r"(t[5]), "r"(c));
+    asm("add.cc.u32  %0, %0, %9;\n\t"
+        "addc.cc.u32 %1, %1, %10;\n\t"
+        "addc.cc.u32 %2, %2, %11;\n\t"
+        "addc.cc.u32 %3, %3, %9;\n\t"
+        "addc.cc.u32 %4, %4, %12;\n\t"
+        "addc.cc.u32 %5, %5, %13;\n\t"
+        "addc.cc.u32 %6, %6, %14;\n\t"
+        "addc.cc.u32 %7, %7, %15;\n\t"
+        "addc.u32    %8, 0, 0;"
+        : "+r"(t[6]), "+r"(t[7]), "+r"(t[8]), "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12]), "+r"(t[13]),
+          "=r"(c)
+        : "r"(t[3]), "r"(t[4]), "r"(t[5]), "r"(D1), "r"(D2), "r"(D3), "r"(D4));
+    // Words 6, 7: D = (q0, D1, D2, D3) with the carry c (word 14) added to D2,
+    // then words 9..15 += (q0, q1, 0, q0, D1, D2, D3), carry c.
+    asm("sub.cc.u32  %0, %4, %3;\n\t"
+        "subc.cc.u32 %1, %3, %4;\n\t"
+        "subc.u32    %2, %4, 0;\n\t"
+        "add.cc.u32  %1, %1, %5;\n\t"
+        "addc.u32    %2, %2, 0;"
+        : "=&r"(D1), "=&r"(D2), "=&r"(D3)
+        : "r"(t[6]), "r"(t[7]), "r"(c));
+    asm("add.cc.u32  %0, %0, %8;\n\t"
+        "addc.cc.u32 %1, %1, %9;\n\t"
+        "addc.cc.u32 %2, %2, 0;\n\t"
+        "addc.cc.u32 %3, %3, %8;\n\t"
+        "addc.cc.u32 %4, %4, %10;\n\t"
+        "addc.cc.u32 %5, %5, %11;\n\t"
+        "addc.cc.u32 %6, %6, %12;\n\t"
+        "addc.u32    %7, 0, 0;"
+        : "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12]), "+r"(t[13]), "+r"(t[14]), "+r"(t[15]), "=r"(c)
+        : "r"(t[6]), "r"(t[7]), "r"(D1), "r"(D2), "r"(D3));
+    // The value (t + q p) / R is below 2^256 + p: on a carry subtract p once
+    // (add K and drop the carry).
+#pragma unroll
+    for (int i = 0; i < 8; i++) r.v[i] = t[8 + i];
+    fe_add_K_masked(r, 0u - c);
 }
 
 // Rows of fused wide multiply-adds.  A 64-bit product a_j b_i lands on words
@@ -496,6 +442,22 @@ static __device__ __noinline__ fe fsqr(fe a) {
     return r;
 }
 
+// Standard residue -> Montgomery domain and back.
+__device__ __forceinline__ void fe_to_mont(fe& r, const fe& a) {
+    fe r2;
+    fe_set_R2(r2);
+    r = fmul(a, r2);
+}
+__device__ __forceinline__ void fe_from_mont(fe& r, const fe& a) {
+    uint32_t t[16];
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        t[i] = a.v[i];
+        t[8 + i] = 0;
+    }
+    fe_reduce(r, t);
+}
+
 // x <- x 2^-k mod p for canonical x and 1 <= k <= 31.  Since p = -1 mod
 // 2^32, x + (x mod 2^k) p is a multiple of 2^k, below 2^k p, so the shifted
 // sum is canonical again.
@@ -517,8 +479,10 @@ __device__ __forceinline__ void fe_div_pow2(fe& x, unsigned k) {
     for (int j = 0; j < 8; j++) x.v[j] = __funnelshift_r(t[j], t[j + 1], k);
 }
 
-// r = a^-1 mod p for a != 0 mod p (0 gives 0), a weakly reduced; r is
-// canonical.  Binary extended Euclid: with u = a, v = p, x1 = 1, x2 = 0 the
+// r = a^-1 in the Montgomery domain (a holds x R, r gets x^-1 R) for a != 0
+// mod p (0 gives 0), a weakly reduced.  Binary extended Euclid on the held
+// value, whose inverse x^-1 R^-1 a multiplication by R^3 brings to x^-1 R:
+// with u = a, v = p, x1 = 1, x2 = 0 the
 // invariants x1 a = u and x2 a = v (mod p) hold throughout; factors of two
 // leave u (or v) together with the same power of two from x1 (or x2), and
 // the smaller of two odd u, v is subtracted from the larger (their
@@ -536,7 +500,8 @@ static __device__ __noinline__ void fe_inv(fe& r, const fe& a) {
     v.v[3] = v.v[4] = v.v[5] = 0u;
     v.v[6] = 1u;
     v.v[7] = 0xffffffffu;
-    fe_one(x1);
+    fe_zero(x1);
+    x1.v[0] = 1u;
     fe_zero(x2);
     // Each step removes a factor of two or shrinks u + v: the bound is never
     // reached for a != 0 mod p.
@@ -601,7 +566,9 @@ static __device__ __noinline__ void fe_inv(fe& r, const fe& a) {
             fe_canon(x2, x2);
         }
     }
-    r = x1;
+    fe r3;
+    fe_set_R3(r3);
+    r = fmul(x1, r3);
 }
 
 // r = a b - c d (mod p) with a single reduction: the two 512-bit products

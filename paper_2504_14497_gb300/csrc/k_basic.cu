@@ -42,9 +42,11 @@ __global__ void __launch_bounds__(128) comb_build_kernel(aff base, uint4* __rest
     for (int i = 0; i < 8; i++) s[i] = 0;
     s[win >> 2] = (uint32_t)v << (8 * (win & 3));
     jac R[1];
+    aff_to_mont(base);
     jac_mul_u256(R[0], base, s);
     aff out[1];
     warp_normalize_regs<1>(out, R);
+    aff_from_mont(out[0]);
     store_aff(tab, COMB_POINTS, idx, out[0]);
 }
 
@@ -73,9 +75,11 @@ __global__ void __launch_bounds__(128) comb_build_cached_kernel(aff base, const 
     for (int i = 0; i < 8; i++) s[i] = 0;
     s[win >> 2] = (uint32_t)v << (8 * (win & 3));
     jac R[1];
+    aff_to_mont(base);
     jac_mul_u256(R[0], base, s);
     aff out[1];
     warp_normalize_regs<1>(out, R);
+    aff_from_mont(out[0]);
     store_aff(tab, COMB_POINTS, idx, out[0]);
 }
 
@@ -94,8 +98,49 @@ __global__ void comb_tag_kernel(aff base, uint32_t* __restrict__ hdr) {
     if (i == 0) hdr[0] = KEY_TAG;
 }
 
-// Enc(b) = (rG, rH + bG): 32 window lookups per base point.
-__global__ void __launch_bounds__(128) encrypt_kernel(const uint4* __restrict__ gtab,
+// Normalise E sums of comb entries (jacz with the factor R) held in each
+// thread's registers to canonical standard affine coordinates; infinity
+// becomes (0, 0).  1 / (ZZ ZZZ) gives both 1 / ZZ and 1 / ZZZ; one inversion
+// per 128-thread block (all threads must call).
+template <int E>
+__device__ __forceinline__ void block_normalize_jacz(aff out[E], const jacz P[E]) {
+    fe pref[E], prod[E], acc;
+    fe_one(acc);
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+        prod[e] = fmul(P[e].ZZ, P[e].ZZZ);
+        if (fe_is_zero(prod[e])) fe_one(prod[e]);
+        acc = fmul(acc, prod[e]);
+        pref[e] = acc;
+    }
+    fe inv = block4_inverse(acc);
+#pragma unroll
+    for (int e = E - 1; e >= 0; e--) {
+        const fe i5 = e > 0 ? fmul(inv, pref[e - 1]) : inv;
+        inv = fmul(inv, prod[e]);
+        if (fe_is_zero(P[e].ZZ)) {
+            fe_zero(out[e].x);
+            fe_zero(out[e].y);
+        } else {
+            // 1 / (ZZ R) and 1 / (ZZZ R): the products are standard residues.
+            out[e].x = fmul(P[e].X, fmul(i5, P[e].ZZZ));
+            out[e].y = fmul(P[e].Y, fmul(i5, P[e].ZZ));
+            fe_canon(out[e].x, out[e].x);
+            fe_canon(out[e].y, out[e].y);
+        }
+    }
+}
+
+// Blocks per SM the register allocation must allow: 262144 encryptions took
+// 2.28, 2.11, 2.04 and 2.03 ms at 3, 4, 5 and 6 blocks.
+#ifndef PCMM_ENCRYPT_MINBLOCKS
+#define PCMM_ENCRYPT_MINBLOCKS 6
+#endif
+
+// Enc(b) = (rG, rH + bG): 32 window lookups per base point, added into
+// (X, Y, Z^2, Z^3) accumulators (8M + 2S each, and the standard comb entries
+// need no conversion).
+__global__ void __launch_bounds__(128, PCMM_ENCRYPT_MINBLOCKS) encrypt_kernel(const uint4* __restrict__ gtab,
                                                       const uint4* __restrict__ htab,
                                                       const uint8_t* __restrict__ msg,
                                                       const uint4* __restrict__ r, size_t count,
@@ -105,26 +150,26 @@ __global__ void __launch_bounds__(128) encrypt_kernel(const uint4* __restrict__ 
     const size_t ii = valid ? i : 0;
     fe rr;
     fe_from_quads(rr, r[ii], r[count + ii]);
-    jac P[2];
-    jac_set_inf(P[0]);
-    jac_set_inf(P[1]);
+    jacz P[2];
+    jacz_set_inf(P[0]);
+    jacz_set_inf(P[1]);
     aff T;
     for (int win = 0; win < COMB_WINDOWS; win++) {
         const uint32_t v = (rr.v[win >> 2] >> (8 * (win & 3))) & 0xffu;
         if (v) {
             load_aff(T, gtab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
-            jac_madd(P[0], T);
+            jacz_madd_t<0, true>(P[0], T);
             load_aff(T, htab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
-            jac_madd(P[1], T);
+            jacz_madd_t<0, true>(P[1], T);
         }
     }
     const uint32_t b = msg[ii];
     if (b) {
         load_aff(T, gtab, COMB_POINTS, b);
-        jac_madd(P[1], T);
+        jacz_madd_t<0, true>(P[1], T);
     }
     aff out[2];
-    warp_normalize_regs<2>(out, P);
+    block_normalize_jacz<2>(out, P);
     if (valid) {
         store_aff(ct, count, i, out[0]);
         store_aff(ct + 4 * count, count, i, out[1]);
@@ -132,7 +177,7 @@ __global__ void __launch_bounds__(128) encrypt_kernel(const uint4* __restrict__ 
 }
 
 // s G for count scalars (key generation: H = x G), one thread per scalar.
-__global__ void __launch_bounds__(128) base_mul_kernel(const uint4* __restrict__ gtab,
+__global__ void __launch_bounds__(128, PCMM_ENCRYPT_MINBLOCKS) base_mul_kernel(const uint4* __restrict__ gtab,
                                                        const uint4* __restrict__ sc, size_t count,
                                                        uint4* __restrict__ out) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -140,18 +185,18 @@ __global__ void __launch_bounds__(128) base_mul_kernel(const uint4* __restrict__
     const size_t ii = valid ? i : 0;
     fe s;
     fe_from_quads(s, sc[ii], sc[count + ii]);
-    jac P[1];
-    jac_set_inf(P[0]);
+    jacz P[1];
+    jacz_set_inf(P[0]);
     aff T;
     for (int win = 0; win < COMB_WINDOWS; win++) {
         const uint32_t v = (s.v[win >> 2] >> (8 * (win & 3))) & 0xffu;
         if (v) {
             load_aff(T, gtab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
-            jac_madd(P[0], T);
+            jacz_madd_t<0, true>(P[0], T);
         }
     }
     aff o[1];
-    warp_normalize_regs<1>(o, P);
+    block_normalize_jacz<1>(o, P);
     if (valid) store_aff(out, count, i, o[0]);
 }
 
@@ -163,33 +208,29 @@ __global__ void __launch_bounds__(128) base_mul_kernel(const uint4* __restrict__
 // shuffles, across the block's four warps).
 // The prefix products wait in the output's x words, which the
 // backward pass overwrites point by point after reading them.
+// X, Y and Z are standard residues throughout: the products of Z's form the
+// same group with R as its identity, and scaling the inverse once by 1 / R
+// makes each Z^-1 the one whose products with X and Y are standard again.
 __global__ void __launch_bounds__(128) normalize_kernel(const uint4* __restrict__ in, size_t count,
                                                         uint4* __restrict__ out, int G) {
     const unsigned lane = threadIdx.x & 31u;
     const size_t T = (size_t)gridDim.x * blockDim.x;
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    fe acc;
-    fe_one(acc);
-    bool ones = true;
+    // A block whose Z's are all 1 or 0 (sums of at most one table entry) only
+    // copies.  Every thread of the (128-thread) block reaches the vote, with
+    // or without ciphertexts.
+    bool plain = true;
     for (int g = 0; g < G; g++) {
         const size_t i = (size_t)g * T + t;
         if (i >= count) break;
 #pragma unroll
         for (int c = 0; c < 2; c++) {
             const uint4* b = in + (size_t)c * 6 * count;
-            fe z;
-            fe_from_quads(z, b[4 * count + i], b[5 * count + i]);
-            ones &= fe_is_one(z);
-            if (fe_is_zero(z)) fe_one(z);
-            acc = fmul(acc, z);
-            uint4* o = out + (size_t)c * 4 * count;
-            o[i] = fe_lo(acc);
-            o[count + i] = fe_hi(acc);
+            const uint4 lo = b[4 * count + i], hi = b[5 * count + i];
+            plain &= (lo.x <= 1u) & ((lo.y | lo.z | lo.w | hi.x | hi.y | hi.z | hi.w) == 0u);
         }
     }
-    // Every thread of the (128-thread) block reaches this point, with or
-    // without ciphertexts, so the block votes and shares one inversion.
-    if (group_all(ones, true)) {
+    if (group_all(plain, true)) {
         for (int g = 0; g < G; g++) {
             const size_t i = (size_t)g * T + t;
             if (i >= count) break;
@@ -200,13 +241,35 @@ __global__ void __launch_bounds__(128) normalize_kernel(const uint4* __restrict_
                 aff A;
                 fe_canon(A.x, P.X);
                 fe_canon(A.y, P.Y);
+                if (P.Z.v[0] == 0u) {
+                    fe_zero(A.x);
+                    fe_zero(A.y);
+                }
                 store_aff(out + (size_t)c * 4 * count, count, i, A);
             }
         }
         return;
     }
+    fe acc;
+    fe_one(acc);
+    for (int g = 0; g < G; g++) {
+        const size_t i = (size_t)g * T + t;
+        if (i >= count) break;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const uint4* b = in + (size_t)c * 6 * count;
+            fe z;
+            fe_from_quads(z, b[4 * count + i], b[5 * count + i]);
+            if (fe_is_zero(z)) fe_one(z);
+            acc = fmul(acc, z);
+            uint4* o = out + (size_t)c * 4 * count;
+            o[i] = fe_lo(acc);
+            o[count + i] = fe_hi(acc);
+        }
+    }
     fe inv;
     group_inverse(inv, acc, true);
+    fe_from_mont(inv, inv);
     for (int g = G - 1; g >= 0; g--) {
         const size_t i = (size_t)g * T + t;
         if (i >= count) continue;
@@ -235,6 +298,8 @@ __global__ void __launch_bounds__(128) normalize_kernel(const uint4* __restrict_
                 fe_zero(A.y);
             } else {
                 jac_to_aff_with_zinv(A, P, zinv);
+                fe_canon(A.x, A.x);
+                fe_canon(A.y, A.y);
             }
             store_aff(out + (size_t)c * 4 * count, count, i, A);
         }
@@ -249,6 +314,10 @@ __global__ void __launch_bounds__(128) test_field_kernel(int op, const uint4* __
     fe x, y, r;
     load_fe(x, a, count, i);
     if (op <= 2) load_fe(y, b, count, i);
+    if (op >= 2 && op <= 4) {
+        fe_to_mont(x, x);
+        if (op == 2) fe_to_mont(y, y);
+    }
     switch (op) {
         case 0: fe_add(r, x, y); break;
         case 1: fe_sub(r, x, y); break;
@@ -257,6 +326,7 @@ __global__ void __launch_bounds__(128) test_field_kernel(int op, const uint4* __
         case 4: fe_inv(r, x); break;
         default: r = x; break;
     }
+    if (op >= 2 && op <= 4) fe_from_mont(r, r);
     fe_canon(r, r);
     store_fe(out, count, i, r);
 }
@@ -272,23 +342,28 @@ __global__ void __launch_bounds__(128) test_point_kernel(int op, const uint4* __
     if (op == 3) {
         aff A;
         load_aff(A, P, count, ii);
+        aff_to_mont(A);
         jac_mul_small(R[0], A, ks[ii]);
     } else {
         load_jac(R[0], P, count, ii);
+        jac_to_mont(R[0]);
         if (op == 0) {
             jac_dbl(R[0]);
         } else if (op == 1) {
             aff B;
             load_aff(B, Q, count, ii);
+            aff_to_mont(B);
             jac_madd(R[0], B);
         } else {
             jac B;
             load_jac(B, Q, count, ii);
+            jac_to_mont(B);
             jac_add(R[0], B);
         }
     }
     aff o[1];
     warp_normalize_regs<1>(o, R);
+    aff_from_mont(o[0]);
     if (valid) store_aff(out, count, i, o[0]);
 }
 

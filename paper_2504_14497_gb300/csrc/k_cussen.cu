@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(128, PCMM_GATHER_MINBLOCKS) gather_kernel(Gath
     gather_item<false>(a, P, gw);
 }
 
-// Adds the parts partial sums of every output point (and, after the first
+// Adds the parts partial sums (Montgomery domain) of every output point (and, after the first
 // pass, the accumulated value) into ctC: one thread per point.
 __global__ void __launch_bounds__(128) combine_kernel(const uint4* __restrict__ partial, int parts,
                                                       uint4* __restrict__ ctC, size_t ml, bool first) {
@@ -87,13 +87,18 @@ __global__ void __launch_bounds__(128) combine_kernel(const uint4* __restrict__ 
     const size_t c = t / ml, idx = t % ml;
     uint4* Cc = ctC + c * 6 * ml;
     jac acc;
-    if (first) jac_set_inf(acc);
-    else load_jac(acc, Cc, ml, idx);
+    if (first) {
+        jac_set_inf(acc);
+    } else {
+        load_jac(acc, Cc, ml, idx);
+        jac_to_mont(acc);
+    }
     for (int p = 0; p < parts; p++) {
         jac Q;
         load_jac(Q, partial + (size_t)p * 12 * ml + c * 6 * ml, ml, idx);
         jac_add(acc, Q);
     }
+    jac_from_mont(acc);
     store_jac(Cc, ml, idx, acc);
 }
 

@@ -47,8 +47,8 @@ __device__ __forceinline__ void fe_neg(fe& r, const fe& a) {
     r = t;
 }
 
-// Normalise E Jacobian points held in each thread's registers to canonical
-// affine coordinates with one field inversion per 128-thread block
+// Normalise E Jacobian points held in each thread's registers to affine
+// coordinates with one field inversion per 128-thread block
 // (infinity becomes (0, 0)).  All 128 threads of the block must call.
 template <int E>
 __device__ __forceinline__ void block_normalize_regs(aff out[E], const jac P[E]) {
@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(128) bsgs_build_kernel(const uint4* __restrict
     comb_mul_u64(R[0], gtab, valid ? j : 1u, 3);
     aff A[1];
     block_normalize_regs<1>(A, R);   // every thread of the block reaches this
+    aff_from_mont(A[0]);
     if (!valid) return;
     const unsigned long long val = ((unsigned long long)A[0].x.v[1] << 32) | (unsigned long long)(j + 1);
     uint32_t h = A[0].x.v[0] & mask;
@@ -144,8 +145,11 @@ static __device__ __noinline__ void start_point(aff& M, aff& negS, jac R, const 
 // sets *j.
 static __device__ __noinline__ bool baby_lookup(const aff& M, const uint4* __restrict__ gtab, uint32_t mask,
                                                 const unsigned long long* __restrict__ slots, uint32_t* jout) {
-    const uint32_t tag = M.x.v[1];
-    uint32_t h = M.x.v[0] & mask;
+    fe x;                               // canonical standard x, as in the table
+    fe_from_mont(x, M.x);
+    fe_canon(x, x);
+    const uint32_t tag = x.v[1];
+    uint32_t h = x.v[0] & mask;
     for (uint32_t probe = 0; probe <= mask; probe++) {
         const unsigned long long e = slots[h];
         if (e == 0ull) return false;
@@ -188,6 +192,7 @@ __global__ void __launch_bounds__(128, PCMM_DECRYPT_MINBLOCKS) decrypt_kernel(
     const size_t ii = valid ? i : 0;
     aff C1;
     load_aff(C1, ct, count, ii);
+    aff_to_mont(C1);
     aff odd[4];
     odd_multiples(odd, C1);
     jac R;
@@ -203,6 +208,7 @@ __global__ void __launch_bounds__(128, PCMM_DECRYPT_MINBLOCKS) decrypt_kernel(
     }
     aff C2, M, negS;
     load_aff(C2, ct + 4 * count, count, ii);
+    aff_to_mont(C2);
     start_point(M, negS, R, C2, gtab, s);
 
     const unsigned long long gmax = (unsigned long long)mmax / s;

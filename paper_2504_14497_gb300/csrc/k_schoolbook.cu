@@ -39,9 +39,11 @@ __global__ void __launch_bounds__(128) schoolbook_kernel(const TA* __restrict__ 
         const uint32_t a = A[(size_t)i * n + k] & amask;
         if (a == 0u) continue;
         load_aff(P, Bc, nl, (size_t)k * l + jj);
+        aff_to_mont(P);
         jac_mul_small(term, P, a);
         jac_add(acc, term);
     }
+    jac_from_mont(acc);
     if (j < l) store_jac(ctC + (size_t)c * 6 * ml, ml, (size_t)i * l + j, acc);
 }
 

@@ -83,9 +83,12 @@ __device__ __forceinline__ void aff_negate(aff& Q) {
 // position (k, j) of its top-left quadrant, the seven children's
 // ciphertexts, both points: copies B11 (child 2) and B22 (child 5), and
 // B11 + B22, B12 - B22, B21 - B11, B11 + B12, B21 + B22 (children 1, 3, 4,
-// 6, 7) by complete mixed additions, normalised to canonical affine two
+// 6, 7) by complete mixed additions, normalised to affine two
 // points per lane at a time (one warp inversion per 64 points).  Parent and
 // child arrays are quad-planar with np_count and nc_count ciphertexts.
+// The top level (TOP) reads the input's standard coordinates; the levels
+// below hold Montgomery-domain ones.
+template <bool TOP>
 __global__ void __launch_bounds__(128) strassen_csum_kernel(const uint4* __restrict__ B, int np, int lp,
                                                             long long nodes, uint4* __restrict__ T) {
     const int nh = np / 2, lh = lp / 2;
@@ -105,8 +108,10 @@ __global__ void __launch_bounds__(128) strassen_csum_kernel(const uint4* __restr
     for (int c = 0; c < 2; c++) {
         aff x;
         load_aff(x, B + (size_t)c * 4 * Np, Np, i11);
+        if (TOP) aff_to_mont(x);
         if (valid) store_aff(T + (size_t)c * 4 * Nc, Nc, o + 1 * cs, x);
         load_aff(x, B + (size_t)c * 4 * Np, Np, i22);
+        if (TOP) aff_to_mont(x);
         if (valid) store_aff(T + (size_t)c * 4 * Nc, Nc, o + 4 * cs, x);
     }
     const size_t sx[5] = {i11, i12, i21, i11, i21};
@@ -121,6 +126,10 @@ __global__ void __launch_bounds__(128) strassen_csum_kernel(const uint4* __restr
             aff x, y;
             load_aff(x, B + (size_t)c * 4 * Np, Np, sx[u]);
             load_aff(y, B + (size_t)c * 4 * Np, Np, sy[u]);
+            if (TOP) {
+                aff_to_mont(x);
+                aff_to_mont(y);
+            }
             if (neg[u]) aff_negate(y);
             jac_from_aff(R[c], x);
             jac_madd(R[c], y);
@@ -172,6 +181,7 @@ __global__ void __launch_bounds__(128) strassen_leaf_kernel(const TA* __restrict
         }
         if (a == 0) continue;
         load_aff(P, Tc, NT, ((size_t)q * nd + k) * ld_ + jj);
+        if (TOP) aff_to_mont(P);        // A's own product reads the input
         jac_mul_small(term, P, (uint32_t)(a < 0 ? -a : a));
         if (a < 0) {
             fe z;
@@ -180,6 +190,7 @@ __global__ void __launch_bounds__(128) strassen_leaf_kernel(const TA* __restrict
         }
         jac_add(acc, term);
     }
+    if (TOP) jac_from_mont(acc);        // and writes the output
     if (j < ld_) store_jac(M + (size_t)c * 6 * NM, NM, ((size_t)q * md + i) * ld_ + j, acc);
 }
 
@@ -187,6 +198,9 @@ __global__ void __launch_bounds__(128) strassen_leaf_kernel(const TA* __restrict
 // quadrant by quadrant (C11 = M1 + M4 - M5 + M7, C12 = M3 + M5,
 // C21 = M2 + M4, C22 = M1 - M2 + M3 + M6) by complete Jacobian additions;
 // one thread per (parent q, position (i, j) of a quadrant, component c).
+// The children's products are in the Montgomery domain, the top level's own
+// (TOP) is the output in standard coordinates.
+template <bool TOP>
 __global__ void __launch_bounds__(128) strassen_combine_kernel(const uint4* __restrict__ M, int mc, int lc,
                                                                long long nodes, uint4* __restrict__ C) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -218,6 +232,7 @@ __global__ void __launch_bounds__(128) strassen_combine_kernel(const uint4* __re
             jac_add(acc, x);
         }
         const size_t out = ((size_t)q * 2 * mc + (size_t)qi[u] * mc + i) * (2 * (size_t)lc) + (size_t)qj[u] * lc + j;
+        if (TOP) jac_from_mont(acc);
         store_jac(Cc, NC, out, acc);
     }
 }
@@ -299,7 +314,10 @@ pcmm_status strassen_run(const StrassenLayout& L, const TA* A, int w, const uint
                 (const TS*)(base + L.offP[t]), L.m[t], L.n[t], pn, amask, S, status);
         PCMM_CUDA_CHECK_LAUNCH();
         const long long cthreads = pn * (L.n[t] / 2) * (L.l[t] / 2);
-        strassen_csum_kernel<<<blocks_for(cthreads), 128, 0, st>>>(B, L.n[t], L.l[t], pn, T);
+        if (t == 0)
+            strassen_csum_kernel<true><<<blocks_for(cthreads), 128, 0, st>>>(B, L.n[t], L.l[t], pn, T);
+        else
+            strassen_csum_kernel<false><<<blocks_for(cthreads), 128, 0, st>>>(B, L.n[t], L.l[t], pn, T);
         PCMM_CUDA_CHECK_LAUNCH();
     }
     // Leaves.
@@ -324,7 +342,12 @@ pcmm_status strassen_run(const StrassenLayout& L, const TA* A, int w, const uint
         uint4* C = t == 0 ? (uint4*)ctC : (uint4*)(base + L.offM[t]);
         const int mc = L.m[t + 1], lc = L.l[t + 1];
         ProfScope ps(KID_STRASSEN_COMBINE, st);
-        strassen_combine_kernel<<<blocks_for(L.nodes[t] * mc * lc * 2), 128, 0, st>>>(M, mc, lc, L.nodes[t], C);
+        if (t == 0)
+            strassen_combine_kernel<true><<<blocks_for(L.nodes[t] * mc * lc * 2), 128, 0, st>>>(M, mc, lc,
+                                                                                              L.nodes[t], C);
+        else
+            strassen_combine_kernel<false><<<blocks_for(L.nodes[t] * mc * lc * 2), 128, 0, st>>>(M, mc, lc,
+                                                                                               L.nodes[t], C);
         PCMM_CUDA_CHECK_LAUNCH();
     }
     return PCMM_OK;
