@@ -280,6 +280,46 @@ static __device__ __noinline__ fe block4_inverse(fe t) {
     return fmul(inv, sex);
 }
 
+// The inverses of 128 non-zero values, one per thread of a 128-thread block,
+// in place in shared memory (low quads sm[0..127], high quads sm[128..255]),
+// by one warp: each lane folds four of the values, the lanes fold theirs by
+// a butterfly of which every lane keeps its partners' products, one field
+// inversion, and the same way back: 19 multiplications and an inversion of
+// one warp while the other blocks of the SM have the pipes. Call with one
+// whole warp, between two block barriers.
+static __device__ __noinline__ void fold_inverse128(uint4* sm) {
+    const unsigned lane = threadIdx.x & 31u;
+    fe t[4], sib[5];
+#pragma unroll
+    for (int w = 0; w < 4; w++) fe_from_quads(t[w], sm[32 * w + lane], sm[128 + 32 * w + lane]);
+    const fe p1 = fmul(t[0], t[1]);
+    const fe p2 = fmul(p1, t[2]);
+    fe cur = fmul(p2, t[3]);
+#pragma unroll
+    for (int k = 0; k < 5; k++) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) sib[k].v[i] = __shfl_xor_sync(0xffffffffu, cur.v[i], 1 << k);
+        cur = fmul(cur, sib[k]);
+    }
+    fe inv = warp_uniform_inv(cur);
+#pragma unroll
+    for (int k = 4; k >= 0; k--) inv = fmul(inv, sib[k]);
+    fe r = fmul(inv, p2);
+    sm[96 + lane] = fe_lo(r);
+    sm[128 + 96 + lane] = fe_hi(r);
+    inv = fmul(inv, t[3]);
+    r = fmul(inv, p1);
+    sm[64 + lane] = fe_lo(r);
+    sm[128 + 64 + lane] = fe_hi(r);
+    inv = fmul(inv, t[2]);
+    r = fmul(inv, t[0]);
+    sm[32 + lane] = fe_lo(r);
+    sm[128 + 32 + lane] = fe_hi(r);
+    r = fmul(inv, t[1]);
+    sm[lane] = fe_lo(r);
+    sm[128 + lane] = fe_hi(r);
+}
+
 // t^-1 per lane: block4_inverse when `shared` (then all 128 threads of the
 // block must call), warp_inverse otherwise.
 __device__ __forceinline__ void group_inverse(fe& tinv, const fe& t, bool shared) {

@@ -429,6 +429,9 @@ struct TableArgs {
     uint4* table;          // affine, quad-planar, table_points points
     size_t table_points;
     bool bshare;           // the 4 warps of each block share one strip's plan: share inversions
+    // Digit build (table_block): digits per column, digits of all columns,
+    // digits of the low half and the bits of both halves.
+    int dpc, nd, ns, hl, hh;
 };
 
 __device__ __forceinline__ void lp_store_aff(uint4* base, int e, unsigned lane, const aff& Q) {
@@ -904,6 +907,475 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
         else lp_load_aff(R, part, e, lane);
         store_table_mont(e, R);
     }
+}
+
+// ---------------------------------------------------------------------------
+// Table build by digits.
+//
+// A strip code of w k bits is cut into digits of at most four bits, none
+// across two columns, and the digits into a low and a high half. Then
+//   1. the multiples of every digit's point: chains of mixed additions, one
+//      inversion for all digits of the same place;
+//   2. both halves' tables, digit by digit: E[v 2^o + g] = E[v 2^o] + E[g];
+//   3. the strip's entries: code = v 2^hl + u gives L[u] + H[v], one affine
+//      addition per distinct code.
+// Within a round of 2 and in 3 the additions are independent, so their slopes
+// share one inversion of the block: 5M + 1S an entry. The chains of prefix
+// sums over the sorted values (table_item) are serial, and cost 12M + 2S an
+// entry with its normalisation. The values of a column (k = 1) come from its
+// compressed levels, prefix sums of integers here.
+//
+// Points are standard residues from the digits' tables on: with the inverse
+// of a product a b / R a slope comes out in the Montgomery domain, its square
+// is reduced twice, and its product with x1 - x3 is standard again.
+
+// How a pair of points is added when their x's are equal or one of them is
+// infinity.
+enum : int { PAIR_ADD = 0, PAIR_SECOND = 1, PAIR_FIRST = 2, PAIR_DOUBLE = 3, PAIR_CANCEL = 4 };
+
+static __device__ __noinline__ void table_item_call(const TableArgs& a, const PlanPtrs& P, long long item,
+                                                    uint4* scratch) {
+    table_item(a, P, item, scratch);
+}
+
+static __device__ __noinline__ int special_pair(const aff& A, const aff& B, const fe& dx) {
+    if (aff_is_inf(B)) return PAIR_FIRST;
+    if (aff_is_inf(A)) return PAIR_SECOND;
+    if (!fe_is_zero(dx)) return PAIR_ADD;
+    return fe_equal(A.y, B.y) ? PAIR_DOUBLE : PAIR_CANCEL;
+}
+
+// 3 x^2 - 3 for a standard residue x.
+static __device__ __noinline__ fe tangent_num(const fe& x) {
+    fe one, t;
+    fe_zero(one);
+    one.v[0] = 1u;
+    fe_to_mont(t, fsqr(x));          // x^2
+    fe_sub(t, t, one);
+    fe r;
+    fe_add(r, t, t);
+    fe_add(r, r, t);
+    return r;
+}
+
+__device__ __forceinline__ bool words345_zero(const fe& a) { return (a.v[3] | a.v[4] | a.v[5]) == 0u; }
+
+// The sums of pair(i) for i < cnt, each handed to put(i, sum): pair sets the
+// two lane-planar affine entries and returns false where there is nothing to
+// add. pref: cnt field elements of lane-planar scratch. All 128 threads of
+// the block call; cnt may differ from warp to warp. `turn` names the warp
+// that inverts.
+template <class Pair, class Put>
+__device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4* pref, uint4* sm, unsigned turn) {
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
+    const unsigned all = 0xffffffffu;
+    // Forward: the prefix products of the differences of x.
+    fe run;
+    fe_one(run);
+#pragma unroll 1
+    for (int i = 0; i < cnt; i++) {
+        const uint4 *pa, *pb;
+        if (!pair(i, pa, pb)) continue;
+        aff A, B;
+        fe_from_quads(A.x, pa[0], pa[32]);
+        fe_from_quads(B.x, pb[0], pb[32]);
+        fe dx;
+        fe_sub(dx, B.x, A.x);
+        // Words 3..5 are zero in 0 and in p: no zero passes this test.
+        const bool sp = words345_zero(dx) || words345_zero(A.x) || words345_zero(B.x);
+        if (__any_sync(all, sp)) {
+            if (sp) {
+                fe_from_quads(A.y, pa[64], pa[96]);
+                fe_from_quads(B.y, pb[64], pb[96]);
+                const int kind = special_pair(A, B, dx);
+                if (kind == PAIR_DOUBLE) fe_add(dx, A.y, A.y);
+                else if (kind != PAIR_ADD) fe_one(dx);
+            }
+        }
+        lp_store_fe(pref, i, lane, run);
+        fe_mul(run, run, dx);
+    }
+    sm[tid] = fe_lo(run);
+    sm[128 + tid] = fe_hi(run);
+    __syncthreads();
+    if (warp == (turn & 3u)) fold_inverse128(sm);
+    __syncthreads();
+    fe inv;
+    fe_from_quads(inv, sm[tid], sm[128 + tid]);
+    // Backward: each difference's inverse, the slope and the sum.
+#pragma unroll 1
+    for (int i = cnt - 1; i >= 0; i--) {
+        const uint4 *pa, *pb;
+        if (!pair(i, pa, pb)) continue;
+        aff A, B, S;
+        fe pr, lam, t;
+        lp_load_fe(pr, pref, i, lane);
+        lp_load_aff(A, pa, 0, 0);
+        lp_load_aff(B, pb, 0, 0);
+        fe dx, dy;
+        fe_sub(dx, B.x, A.x);
+        fe_sub(dy, B.y, A.y);
+        int kind = PAIR_ADD;
+        const bool sp = words345_zero(dx) || words345_zero(A.x) || words345_zero(B.x);
+        const bool anysp = __any_sync(all, sp);
+        if (anysp && sp) {
+            kind = special_pair(A, B, dx);
+            if (kind == PAIR_DOUBLE) {
+                fe_add(dx, A.y, A.y);
+                dy = tangent_num(A.x);
+            } else if (kind != PAIR_ADD) {
+                fe_one(dx);
+            }
+        }
+        fe_mul(lam, inv, pr);
+        fe_mul(inv, inv, dx);
+        fe_mul(lam, dy, lam);
+        t = fe_sqr_std(lam);
+        fe_sub(t, t, A.x);
+        fe_sub(S.x, t, B.x);
+        fe_sub(t, A.x, S.x);
+        fe_mul(t, lam, t);
+        fe_sub(S.y, t, A.y);
+        fe_canon(S.x, S.x);
+        fe_canon(S.y, S.y);
+        if (anysp) {
+            if (kind == PAIR_FIRST) S = A;
+            if (kind == PAIR_SECOND) S = B;
+            if (kind == PAIR_CANCEL) {
+                fe_zero(S.x);
+                fe_zero(S.y);
+            }
+        }
+        put(i, S);
+    }
+}
+
+// Bits of digit d: four, or what is left of its column.
+__device__ __forceinline__ int digit_bits(const TableArgs& a, int d) {
+    const int r = a.w - 4 * (d % a.dpc);
+    return r < 4 ? r : 4;
+}
+
+// Scratch of the digit build, in uint4 per warp: the values of the level
+// lists, the digits' chains (6 + 2 quads an entry), the next places' base
+// points, both halves' tables and the prefix products.
+struct DigitScratch {
+    size_t vals, chain, rat, base, half, pref, total;
+};
+__host__ __device__ inline DigitScratch digit_scratch(int w, int k, int dpc, int hl, int hh, int n1max, int l2max,
+                                                      int emax) {
+    DigitScratch D;
+    size_t off = 0;
+    D.vals = off;
+    off += (size_t)((n1max + 2 * l2max) * 2 + 15) / 16 + 1;
+    const int place = w < 4 ? w : 4;
+    const size_t chain = (size_t)k * (1 << place);
+    D.chain = off;
+    off += chain * 192;
+    D.rat = off;
+    off += chain * 64;
+    D.base = off;
+    off += (size_t)(dpc > 1 ? k : 0) * 128;
+    D.half = off;
+    off += ((size_t)(1 << hl) + (size_t)(1 << hh)) * 128;
+    D.pref = off;
+    size_t np = (size_t)1 << (hl > hh ? hl : hh);
+    np = 2 * np > (size_t)emax ? 2 * np : (size_t)emax;
+    off += (np > (size_t)k ? np : (size_t)k) * 64;
+    D.total = off;
+    return D;
+}
+
+// The values of column col's level 1, in lists of 16-bit words at buf:
+// level N's values, and each level below as prefix sums over its tracking
+// pointers. One warp.
+__device__ __forceinline__ const uint16_t* column_values(const PlanPtrs& P, int col, const int* lens, uint16_t* buf) {
+    const unsigned lane = threadIdx.x & 31u;
+    const uint16_t* cur = P.col_vN + (size_t)col * P.l2max;
+    for (int lev = NLEV - 1; lev >= 1; lev--) {
+        const uint16_t* ptr = col_level_ptr(P, col, lev);
+        uint16_t* out = lev == 1 ? buf + 2 * P.l2max : buf + (lev & 1) * P.l2max;
+        uint32_t carry = 0;
+        for (int b = 0; b < lens[lev - 1]; b += 32) {
+            const int e = b + (int)lane;
+            uint32_t x = e < lens[lev - 1] ? cur[ptr[e]] : 0u;
+#pragma unroll
+            for (int k = 1; k < 32; k <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, x, k);
+                if ((int)lane >= k) x += o;
+            }
+            x += carry;
+            if (e < lens[lev - 1]) out[e] = (uint16_t)x;
+            carry = __shfl_sync(0xffffffffu, x, 31);
+        }
+        __syncwarp();
+        cur = out;
+    }
+    return cur;
+}
+
+// Table of one warp item by digits. All 128 threads of the block call (valid:
+// the warp has an item); sm: 256 uint4 of shared memory. Returns false, for
+// the whole block, when a chain met infinity (an input at infinity): nothing
+// the caller reads has been written then, and table_item builds the tables.
+__device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
+                                            uint4* scratch, uint4* sm) {
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
+    const int s_local = valid ? (int)(item / (2 * a.njb)) : 0;
+    const int rem = valid ? (int)(item % (2 * a.njb)) : 0;
+    const int c = rem / a.njb, jb = rem % a.njb;
+    const int s = a.s0 + s_local;
+    const int c0 = s * a.k;
+    const int kw = !valid ? 0 : (c0 + a.k <= a.n) ? a.k : a.n - c0;
+    const int j = jb * 32 + (int)lane;
+    const int jj = j < a.l ? j : a.l - 1;
+    const size_t nl = (size_t)a.n * a.l;
+    const uint4* Bc = a.ctB + (size_t)c * 4 * nl;
+    const DigitScratch D = digit_scratch(a.w, a.k, a.dpc, a.hl, a.hh, a.n1max, a.l2max, a.emax);
+    uint4* chain = scratch + D.chain;
+    uint4* rat = scratch + D.rat;
+    uint4* base = scratch + D.base;
+    uint4* half = scratch + D.half;
+    uint4* pref = scratch + D.pref;
+    int E = valid ? P.nent[s] : 0;
+    unsigned turn = blockIdx.x;
+
+    // The strip's distinct codes.
+    const uint16_t* codes = P.codes + (size_t)s * a.emax;
+    bool bad = E > a.emax, dbad = false;
+    for (int t = 0; t < kw; t++) {
+        int lens[NLEV];
+#pragma unroll
+        for (int q = 0; q < NLEV; q++) lens[q] = P.col_len[(size_t)(c0 + t) * NLEV + q];
+        bad |= lens[0] > a.n1max;
+#pragma unroll
+        for (int q = 1; q < NLEV; q++) bad |= lens[q] > a.l2max;
+#ifdef PCMM_DEBUG_BOUNDS
+        // Each tracking pointer names an entry of the next level, each tuple
+        // component an entry of its column.
+        for (int lev = 1; lev < NLEV && !bad; lev++) {
+            const uint16_t* pl = col_level_ptr(P, c0 + t, lev);
+            for (int e = 0; e < lens[lev - 1]; e++) dbad |= pl[e] >= lens[lev];
+        }
+        for (int e = 0; a.k > 1 && e < E && !bad; e++) {
+            const uint32_t x = ((uint32_t)codes[e] >> (a.w * t)) & ((1u << a.w) - 1u);
+            if (x) dbad |= P.col_rank1[(size_t)(c0 + t) * 256 + x] >= lens[0];
+        }
+        bad |= dbad;
+#endif
+        if (a.k == 1 && !bad) {
+            bad |= E > lens[0];
+#ifdef PCMM_DEBUG_BOUNDS
+            dbad |= E != lens[0];
+            bad |= dbad;
+#endif
+            codes = column_values(P, c0, lens, (uint16_t*)(scratch + D.vals));
+        }
+    }
+    if (bad) {
+        if (lane == 0) atomicOr(P.status, dbad ? DEV_ERR_BOUNDS : DEV_ERR_PLAN);
+        E = 0;
+    }
+
+    // 1. Place by place, the digits' multiples: entry v of a digit at bit o
+    // of its half goes to half entry v 2^o (standard coordinates), and 2^4
+    // times its point (Montgomery domain) to the column's base.
+    auto half_at = [&](int dg, int& o) -> uint4* {
+        o = 0;
+        for (int x = dg < a.ns ? 0 : a.ns; x < dg; x++) o += digit_bits(a, x);
+        return half + (dg < a.ns ? (size_t)0 : (size_t)128 << a.hl);
+    };
+    bool ok = true;
+    for (int place = 0; place < a.dpc; place++) {
+        const bool more = place + 1 < a.dpc;
+        fe acc;
+        fe_one(acc);
+        for (int t = 0; t < kw; t++) {
+            const int dg = t * a.dpc + place, len = (1 << digit_bits(a, dg)) - (more ? 0 : 1);
+            aff B, S;
+            if (place == 0) {
+                load_aff(S, Bc, nl, (size_t)(c0 + t) * a.l + jj);
+                B = S;
+                aff_to_mont(B);
+            } else {
+                lp_load_aff(B, base, t, lane);
+                S = B;
+                aff_from_mont(S);
+            }
+            int o;
+            uint4* hb = half_at(dg, o);
+            lp_store_aff(hb, 1 << o, lane, S);
+            if (len < 2) continue;
+            jacz P1;
+            jacz_set_inf(P1);
+            uint4* ch = chain + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 192;
+            uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 64;
+            for (int e = 0; e < len; e++) {
+                fe r2, r3;
+                jacz_madd_ratio_t<PCMM_TABLE_INLINE>(P1, B, r2, r3, ok, e == 0);
+                uint4* b = ch + (size_t)e * 192 + lane;
+                b[0] = fe_lo(P1.X);
+                b[32] = fe_hi(P1.X);
+                b[64] = fe_lo(P1.Y);
+                b[96] = fe_hi(P1.Y);
+                b[128] = fe_lo(r3);
+                b[160] = fe_hi(r3);
+                lp_store_fe(rt, e, lane, r2);
+            }
+            // The chain's product ZZ ZZZ for the shared inversion; ZZ and ZZZ
+            // wait in slot 0, whose factors are 1.
+            uint4* b = ch + lane;
+            b[0] = fe_lo(P1.ZZ);
+            b[32] = fe_hi(P1.ZZ);
+            b[64] = fe_lo(P1.ZZZ);
+            b[96] = fe_hi(P1.ZZZ);
+            lp_store_fe(pref, t, lane, acc);
+            acc = fmul(acc, fmul(P1.ZZ, P1.ZZZ));
+        }
+        if (a.w == 1) break;                    // no chains: nothing to invert
+        if (!__syncthreads_and(ok)) return false;
+        sm[tid] = fe_lo(acc);
+        sm[128 + tid] = fe_hi(acc);
+        __syncthreads();
+        if (warp == (turn & 3u)) fold_inverse128(sm);
+        turn++;
+        __syncthreads();
+        fe inv;
+        fe_from_quads(inv, sm[tid], sm[128 + tid]);
+        for (int t = kw - 1; t >= 0; t--) {
+            const int dg = t * a.dpc + place, len = (1 << digit_bits(a, dg)) - (more ? 0 : 1);
+            if (len < 2) continue;
+            const uint4* ch = chain + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 192;
+            const uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 64;
+            fe zz, zzz, pr;
+            fe_from_quads(zz, ch[lane], ch[32 + lane]);
+            fe_from_quads(zzz, ch[64 + lane], ch[96 + lane]);
+            lp_load_fe(pr, pref, t, lane);
+            const fe i5 = fmul(inv, pr);
+            inv = fmul(inv, fmul(zz, zzz));
+            fe zi = fmul(i5, zzz), zzi = fmul(i5, zz);   // ZZ^-1 and ZZZ^-1 of the last entry
+            int o;
+            uint4* hb = half_at(dg, o);
+            for (int e = len - 1; e >= 1; e--) {
+                const bool last = more && e == len - 1;
+                if (more ? e == len - 2 : e == len - 1) {
+                    // From here on the products with X and Y are standard.
+                    fe_from_mont(zi, zi);
+                    fe_from_mont(zzi, zzi);
+                }
+                const uint4* b = ch + (size_t)e * 192 + lane;
+                fe X, Y, r2, r3;
+                fe_from_quads(X, b[0], b[32]);
+                fe_from_quads(Y, b[64], b[96]);
+                aff Q;
+                Q.x = fmul(X, zi);
+                Q.y = fmul(Y, zzi);
+                if (last) {
+                    lp_store_aff(base, t, lane, Q);
+                } else {
+                    fe_canon(Q.x, Q.x);
+                    fe_canon(Q.y, Q.y);
+                    lp_store_aff(hb, (e + 1) << o, lane, Q);
+                }
+                lp_load_fe(r2, rt, e, lane);
+                fe_from_quads(r3, b[128], b[160]);
+                zi = fmul(zi, r2);
+                zzi = fmul(zzi, r3);
+            }
+        }
+    }
+
+    // 2. The halves' tables, one more digit of each half a round.
+    const int nlow = a.ns, nhigh = a.nd - a.ns;
+    for (int r = 1; r < nlow || r < nhigh; r++) {
+        // Low half: digit r at bit oL; high half: digit ns + r at bit oH.
+        // Pair index i of a half: (v - 1) 2^o + g.
+        int o[2] = {0, 0}, n[2] = {0, 0};
+#pragma unroll
+        for (int hf = 0; hf < 2; hf++) {
+            const int dg = hf ? a.ns + r : r;
+            if (r < (hf ? nhigh : nlow) && dg / a.dpc < kw) {
+                half_at(dg, o[hf]);
+                n[hf] = ((1 << digit_bits(a, dg)) - 1) << o[hf];
+            }
+        }
+        auto pick = [&](int i, int& g, int& v, uint4*& tab) -> bool {
+            const int hf = i >= n[0];
+            if (hf) i -= n[0];
+            tab = half + (hf ? (size_t)128 << a.hl : (size_t)0);
+            const int ob = hf ? o[1] : o[0];
+            g = i & ((1 << ob) - 1);
+            v = ((i >> ob) + 1) << ob;
+            return g != 0;
+        };
+        affine_batch(
+            n[0] + n[1],
+            [&](int i, const uint4*& pa, const uint4*& pb) -> bool {
+                int g, v;
+                uint4* tab;
+                if (!pick(i, g, v, tab)) return false;
+                pa = tab + (size_t)g * 128 + lane;
+                pb = tab + (size_t)v * 128 + lane;
+                return true;
+            },
+            [&](int i, const aff& S) {
+                int g, v;
+                uint4* tab;
+                pick(i, g, v, tab);
+                lp_store_aff(tab, v + g, lane, S);
+            },
+            pref, sm, turn++);
+    }
+
+    // 3. The strip's entries.
+    const size_t tbase = (size_t)s_local * a.emax;
+    auto store_table = [&](int e, const aff& q) {
+        store_aff(a.table, a.table_points, ((tbase + e) * 2 + c) * a.lp + j, q);
+    };
+    const uint32_t lmask = (1u << a.hl) - 1u;
+    const uint4* high = half + ((size_t)128 << a.hl);
+    affine_batch(
+        E,
+        [&](int e, const uint4*& pa, const uint4*& pb) -> bool {
+            const uint32_t code = codes[e];
+            pa = half + (size_t)(code & lmask) * 128 + lane;
+            pb = high + (size_t)(code >> a.hl) * 128 + lane;
+            return (code & lmask) && (code >> a.hl);
+        },
+        store_table, pref, sm, turn);
+    for (int e = 0; e < E; e++) {
+        const uint32_t code = codes[e];
+        if ((code & lmask) && (code >> a.hl)) continue;
+        aff Q;
+        lp_load_aff(Q, code & lmask ? half + (size_t)(code & lmask) * 128 : high + (size_t)(code >> a.hl) * 128, 0, lane);
+        store_table(e, Q);
+    }
+    return true;
+}
+
+// The digits and halves of a strip code, and whether the digit build takes
+// the tables of this layout.
+inline bool digit_split(const Layout& L, TableArgs& a) {
+    a.dpc = (L.w + 3) / 4;
+    a.nd = L.k * a.dpc;
+    a.ns = a.hl = a.hh = 0;
+    if (a.nd < 2) return false;
+    auto bits = [&](int d) { const int r = L.w - 4 * (d % a.dpc); return r < 4 ? r : 4; };
+    long long best = -1;
+    int lo = 0;
+    for (int x = 1; x < a.nd; x++) {
+        lo += bits(x - 1);
+        const int hi = L.w * L.k - lo;
+        const long long size = (1LL << lo) + (1LL << hi);
+        if (best < 0 || size < best) { best = size; a.ns = x; a.hl = lo; a.hh = hi; }
+    }
+    // The halves must not outweigh the entries.  Table times (ms) by chains and
+    // by digits, 256 x 256 columns: w = 12 with 128 rows (halves 272) 4.90 and
+    // 5.38, with 256 rows 7.22 and 6.63; w = 16 with 256 rows (halves 512) 12.0
+    // and 9.96, with 512 rows 18.2 and 12.8; w = 8 with 16 rows (halves 32) 1.17
+    // and 1.11, with 128 rows 2.81 and 1.98; k = 5 at w = 1 0.54 and 0.19.
+    if (best > 2LL * L.emax) return false;
+    return digit_scratch(L.w, L.k, a.dpc, a.hl, a.hh, L.n1max, L.l2max, L.emax).total <= L.item_u4;
 }
 
 struct GatherArgs {

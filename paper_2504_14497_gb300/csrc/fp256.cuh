@@ -458,6 +458,17 @@ __device__ __forceinline__ void fe_from_mont(fe& r, const fe& a) {
     fe_reduce(r, t);
 }
 
+// The square of a, reduced twice: a^2 / R^2. Of a Montgomery-domain a it is
+// the standard residue of the square.
+__device__ __forceinline__ fe fe_sqr_std(const fe& a) {
+    uint32_t t[16];
+    sqr_wide(t, a);
+    fe r;
+    fe_reduce(r, t);
+    fe_from_mont(r, r);
+    return r;
+}
+
 // x <- x 2^-k mod p for canonical x and 1 <= k <= 31.  Since p = -1 mod
 // 2^32, x + (x mod 2^k) p is a multiple of 2^k, below 2^k p, so the shifted
 // sum is canonical again.

@@ -53,6 +53,7 @@ struct Inst {
     int nstrips, n1max, l2max, emax, lp, njb;
     int S, nchunks;
     int ctr_base;               // 2 counters per pass: tables done, gathers done
+    int digits, dpc, nd, ns, hl, hh;   // table build by digits (digit_split)
 };
 
 struct Segment {
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
     uint4* my_scratch = scratch + (size_t)warp_id * scratch_u4;
     __shared__ long long sh_t;
     __shared__ int sh_seg, sh_go;
+    __shared__ uint4 sh_inv[256];
     for (;;) {
         // The block takes BLOCK_TASKS consecutive tasks of one segment (every
         // segment starts at a multiple of BLOCK_TASKS), one per warp.  Every
@@ -139,8 +141,9 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
             // strip, follow one plan and share each inversion.
             const int ips = 2 * I.njb;
             const bool shared = (ips % BLOCK_TASKS) == 0;
-            if (real) {
+            {
                 TableArgs ta;
+                ta.dpc = I.dpc; ta.nd = I.nd; ta.ns = I.ns; ta.hl = I.hl; ta.hh = I.hh;
                 ta.ctB = I.ctB;
                 ta.bshare = shared;
                 ta.m = I.m; ta.n = I.n; ta.l = I.l; ta.w = I.w; ta.k = I.k;
@@ -150,7 +153,8 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
                 ta.item_u4 = I.item_u4;
                 ta.table = tbuf;
                 ta.table_points = I.table_points;
-                table_item(ta, I.P, item, my_scratch);
+                if (!(I.digits && table_block(ta, I.P, item, real, my_scratch, sh_inv)) && real)
+                    table_item_call(ta, I.P, item, my_scratch);
             }
         } else if (real) {
             GatherArgs ga;
@@ -253,6 +257,9 @@ pcmm_status build_layout(const pcmm_problem* probs, int count, int max_strips, i
         I.m = L.m; I.n = L.n; I.l = L.l; I.w = L.w; I.k = L.k;
         I.nstrips = L.nstrips; I.n1max = L.n1max; I.l2max = L.l2max; I.emax = L.emax;
         I.lp = L.lp; I.njb = L.njb; I.item_u4 = L.item_u4;
+        TableArgs split;
+        I.digits = digit_split(L, split);
+        I.dpc = split.dpc; I.nd = split.nd; I.ns = split.ns; I.hl = split.hl; I.hh = split.hh;
         H.scratch_u4 = std::max(H.scratch_u4, L.item_u4);
     }
     H.nctrs = ctr;

@@ -26,7 +26,10 @@
 //         level-1 chains by walking Z^-2 and Z^-3 back along the factors the
 //         chain multiplied them by; the inversion is shared by the lanes of
 //         a warp and, when the block's four warps follow one strip's plan,
-//         by the whole block.
+//         by the whole block.  Where the strip's codes outnumber the tables
+//         of their halves (most strips) the same entries are built digit by
+//         digit in affine coordinates instead (table_block), from the
+//         values that the compressed levels expand to.
 //  gather (one warp per output row i, component c and 32 output columns)
 //         C_ij += T_s[rank_s(i)] for every strip s: the "un-sort and re-insert
 //         duplicates" step of Algorithm 2 fused with the accumulation of
@@ -70,6 +73,22 @@ __global__ void __launch_bounds__(128, PCMM_TABLE_MINBLOCKS) table_kernel(TableA
     const long long nitems = (long long)a.nstrips_chunk * 2 * a.njb;
     if (item >= nitems) return;
     table_item(a, P, item, a.scratch + (size_t)item * a.item_u4);
+}
+
+// table_kernel by digits (table_block): two thirds of the multiplications and
+// hardly any spills, so it is faster than the chains and wants registers more
+// than warps. Table times of 1024 x 1024 x 256 (ms), chains and digits at 3, 4,
+// 5 and 6 blocks per SM: w = 8 21.5 / 13.9, 13.5, 14.1, 14.9; w = 4 8.3 / 6.8,
+// 6.7, 7.1, 7.3; 512 x 512 x 256, w = 16: 36.6 / 27.9, 25.5, 27.3, 30.7.
+#ifndef PCMM_DIGIT_MINBLOCKS
+#define PCMM_DIGIT_MINBLOCKS 4
+#endif
+__global__ void __launch_bounds__(128, PCMM_DIGIT_MINBLOCKS) digit_table_kernel(TableArgs a, PlanPtrs P) {
+    __shared__ uint4 sm[256];
+    const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const bool valid = item < (long long)a.nstrips_chunk * 2 * a.njb;
+    uint4* scratch = a.scratch + (valid ? (size_t)item : (size_t)0) * a.item_u4;
+    if (!table_block(a, P, item, valid, scratch, sm) && valid) table_item_call(a, P, item, scratch);
 }
 
 __global__ void __launch_bounds__(128, PCMM_GATHER_MINBLOCKS) gather_kernel(GatherArgs a, PlanPtrs P) {
@@ -175,9 +194,11 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
     uint4* scratch = (uint4*)chunk;
     uint4* table = (uint4*)(chunk + align256(S * L.items_per_strip * L.item_u4 * 16));
     const size_t ml = (size_t)L.m * L.l;
+    TableArgs split;
+    const bool digits = digit_split(L, split);
     for (int s0 = 0; s0 < L.nstrips; s0 += (int)S) {
         const int sc = (int)((size_t)(L.nstrips - s0) < S ? (size_t)(L.nstrips - s0) : S);
-        TableArgs ta;
+        TableArgs ta = split;
         ta.ctB = (const uint4*)ctB;
         ta.m = L.m; ta.n = L.n; ta.l = L.l; ta.w = L.w; ta.k = L.k;
         ta.lp = L.lp; ta.njb = L.njb; ta.n1max = L.n1max; ta.l2max = L.l2max; ta.emax = L.emax;
@@ -193,7 +214,8 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         const long long items = (long long)sc * L.items_per_strip;
         {
             ProfScope ps(KID_TABLE, st);
-            table_kernel<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(ta, P);
+            if (digits) digit_table_kernel<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(ta, P);
+            else table_kernel<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(ta, P);
         }
         PCMM_CUDA_CHECK_LAUNCH();
         GatherArgs ga;

@@ -1,0 +1,66 @@
+"""Strip tables built by digits, through whole products against the schoolbook
+path (exact): every split of a code into digits and halves, ragged last
+strips and column blocks, and pairs of points that the affine addition cannot
+take (equal and opposite columns, columns at infinity)."""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2504_14497_gb300 import inputs, pcmm
+from tests.gpu_common import P, ct_from_aos, device, encrypt_gpu
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _device_plain(A, w, dev):
+    return pcmm.plaintext16(A, dev) if w > 8 else torch.from_numpy(A).to(dev)
+
+
+def _same(A, ctB, m, l, w, k):
+    want = pcmm.normalize(pcmm.schoolbook(A, ctB, l, w), m * l)
+    ws = pcmm.workspace(m, A.shape[1], l, w, k, device=A.device)
+    got = pcmm.normalize(pcmm.cussen(A, ctB, l, w, k=k, ws=ws), m * l)
+    assert pcmm.workspace_status(ws) == 0
+    assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("w,k,m,n,l", [
+    (1, 2, 40, 5, 33), (1, 6, 300, 13, 32), (1, 16, 300, 17, 3), (2, 3, 70, 7, 65), (2, 4, 300, 9, 32),
+    (3, 2, 70, 5, 40), (3, 5, 600, 6, 32), (4, 2, 300, 3, 96), (4, 4, 700, 5, 32), (5, 1, 40, 3, 33),
+    (5, 3, 700, 4, 32), (6, 2, 400, 3, 32), (7, 1, 140, 3, 64), (8, 1, 16, 3, 1), (8, 1, 300, 2, 130),
+    (8, 2, 900, 3, 32), (9, 1, 100, 3, 33), (12, 1, 200, 2, 32), (13, 1, 300, 2, 64), (16, 1, 300, 3, 32),
+])
+def test_products(w, k, m, n, l):
+    dev = device()
+    pr = inputs.pcmm_problem(9000 + 100 * w + k, m, n, l, w)
+    _same(_device_plain(pr["A"], w, dev), encrypt_gpu(dev, pr), m, l, w, k)
+
+
+@pytest.mark.parametrize("w,k,m", [(1, 6, 64), (2, 3, 128), (4, 2, 300), (4, 4, 500), (8, 2, 700), (8, 1, 300)])
+def test_related_columns(w, k, m):
+    # Within every strip: a column, the same column, its negative, infinity.
+    dev = device()
+    n, l = 2 * k + 1, 34
+    pr = inputs.pcmm_problem(9900 + 10 * w + k, m, n, l, w)
+    ct = oracle.encrypt(oracle.keygen(pr["sk"]), pr["B"], pr["r"]).copy()     # [n, l, 2, 16]
+    for s in range(0, n, k):
+        for t in range(1, min(k, n - s)):
+            for j in range(l):
+                kind = (t + j) % 4
+                if kind == 0:
+                    ct[s + t, j] = 0
+                elif kind < 3:
+                    ct[s + t, j] = ct[s, j]
+                    for c in range(2):
+                        if kind == 2 and ct[s, j, c].any():
+                            y = oracle.words_to_int(ct[s, j, c, 8:])
+                            ct[s + t, j, c, 8:] = oracle.int_to_words((P - y) % P)
+    _same(_device_plain(pr["A"], w, dev), ct_from_aos(dev, ct), m, l, w, k)
+    # The same without infinity: no strip leaves the digit build.
+    for s in range(0, n, k):
+        for t in range(1, min(k, n - s)):
+            for j in range(l):
+                if (t + j) % 4 == 0:
+                    ct[s + t, j] = ct[s, j]
+    _same(_device_plain(pr["A"], w, dev), ct_from_aos(dev, ct), m, l, w, k)
