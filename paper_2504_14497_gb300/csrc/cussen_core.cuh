@@ -16,11 +16,12 @@ constexpr int NLEV = PCMM_N_ITER;   // compression iterations N
 
 // Which field operations the gather's mixed addition and the table build's
 // chain additions inline (build-time switches, see jacz_madd_t).  Measured
-// on GB300 (w in {8, 4}, 1024 x 1024 x 256): gather 109.3 ms per step all out
-// of line, 108.3 with the squarings inlined, 108.2 with a b - c d, 107.4-107.7
-// with both (3), 112.5-127.8 when multiplications are inlined as well.
+// on GB300 (w = 4, 1024 x 1024 x 256): gather 25.3 ms all out of line, 25.0 with
+// the squarings and a b - c d inlined (3), 23.9 all inlined (31) at four blocks
+// per SM, 24.6 at three and 25.1 at five: a call moves its operands on the pipe
+// that multiplies.
 #ifndef PCMM_GATHER_INLINE
-#define PCMM_GATHER_INLINE 3
+#define PCMM_GATHER_INLINE 31
 #endif
 #ifndef PCMM_TABLE_INLINE
 #define PCMM_TABLE_INLINE 0

@@ -30,11 +30,13 @@
 // shift by 96 bits) t / 2^96 + q (2^160 - 2^128 + 2^96 + 1): with D = q (2^64
 // - 2^32 + 1), five words from seven additions, one carry chain of eight adds
 // (q, D).  Steps of 3, 3 and 2 words clear all eight: about 54 additions and
-// no multiplications.  Measured per warp and scheduler: 104 cycles, against
+// no multiplications.  Measured per warp and scheduler: 102 cycles, against
 // 205 for the special-form (Solinas) reduction of a standard residue, whose
-// nine rearranged terms need 96 additions; a multiplication takes 323 cycles
-// inlined and 352 called (437 and 448 with the special-form reduction), a
-// squaring 270 and 280.
+// nine rearranged terms need 96 additions; a multiplication takes 330 cycles
+// inlined and 336 called (437 and 448 with the special-form reduction), a
+// squaring 262. The corrections by p and K take their words from the carry
+// itself: with general masks the multiplication took 347 cycles and a
+// subtraction 65 instead of 49.
 #pragma once
 #include <stdint.h>
 
@@ -73,45 +75,47 @@ __device__ __forceinline__ void fe_set_R3(fe& r) {
     r.v[4] = 0xfffffffcu; r.v[5] = 0x00000005u; r.v[6] = 0x00000001u; r.v[7] = 0x00000018u;
 }
 
-// r += mask & K (mask is 0 or 0xffffffff); returns the carry out.
-__device__ __forceinline__ uint32_t fe_add_K_masked(fe& r, uint32_t mask) {
-    uint32_t k0 = mask & PCMM_K0, k3 = mask, k6 = mask & PCMM_K6, c;
+// r += p & m (m is 0 or 0xffffffff) modulo 2^256; returns the carry out. With
+// words 3..5 of p zero and all others but word 6 full, m itself is the addend.
+__device__ __forceinline__ uint32_t fe_add_p_masked(fe& r, uint32_t m) {
+    uint32_t c;
     asm("add.cc.u32  %0, %0, %9;\n\t"
-        "addc.cc.u32 %1, %1, 0;\n\t"
-        "addc.cc.u32 %2, %2, 0;\n\t"
-        "addc.cc.u32 %3, %3, %10;\n\t"
-        "addc.cc.u32 %4, %4, %10;\n\t"
-        "addc.cc.u32 %5, %5, %10;\n\t"
-        "addc.cc.u32 %6, %6, %11;\n\t"
-        "addc.cc.u32 %7, %7, 0;\n\t"
+        "addc.cc.u32 %1, %1, %9;\n\t"
+        "addc.cc.u32 %2, %2, %9;\n\t"
+        "addc.cc.u32 %3, %3, 0;\n\t"
+        "addc.cc.u32 %4, %4, 0;\n\t"
+        "addc.cc.u32 %5, %5, 0;\n\t"
+        "addc.cc.u32 %6, %6, %10;\n\t"
+        "addc.cc.u32 %7, %7, %9;\n\t"
         "addc.u32    %8, 0, 0;"
         : "+r"(r.v[0]), "+r"(r.v[1]), "+r"(r.v[2]), "+r"(r.v[3]), "+r"(r.v[4]), "+r"(r.v[5]),
           "+r"(r.v[6]), "+r"(r.v[7]), "=r"(c)
-        : "r"(k0), "r"(k3), "r"(k6));
+        : "r"(m), "r"(m & 1u));
     return c;
 }
 
-// r -= mask & K; returns the borrow (1 if it wrapped).
-__device__ __forceinline__ uint32_t fe_sub_K_masked(fe& r, uint32_t mask) {
-    uint32_t k0 = mask & PCMM_K0, k3 = mask, k6 = mask & PCMM_K6, b;
+// r -= c p (c is 0 or 1) modulo 2^256; returns 0xffffffff on a borrow, else 0.
+__device__ __forceinline__ uint32_t fe_sub_p_times(fe& r, uint32_t c) {
+    const uint32_t m = 0u - c;
+    uint32_t b;
     asm("sub.cc.u32  %0, %0, %9;\n\t"
-        "subc.cc.u32 %1, %1, 0;\n\t"
-        "subc.cc.u32 %2, %2, 0;\n\t"
-        "subc.cc.u32 %3, %3, %10;\n\t"
-        "subc.cc.u32 %4, %4, %10;\n\t"
-        "subc.cc.u32 %5, %5, %10;\n\t"
-        "subc.cc.u32 %6, %6, %11;\n\t"
-        "subc.cc.u32 %7, %7, 0;\n\t"
+        "subc.cc.u32 %1, %1, %9;\n\t"
+        "subc.cc.u32 %2, %2, %9;\n\t"
+        "subc.cc.u32 %3, %3, 0;\n\t"
+        "subc.cc.u32 %4, %4, 0;\n\t"
+        "subc.cc.u32 %5, %5, 0;\n\t"
+        "subc.cc.u32 %6, %6, %10;\n\t"
+        "subc.cc.u32 %7, %7, %9;\n\t"
         "subc.u32    %8, 0, 0;"
         : "+r"(r.v[0]), "+r"(r.v[1]), "+r"(r.v[2]), "+r"(r.v[3]), "+r"(r.v[4]), "+r"(r.v[5]),
           "+r"(r.v[6]), "+r"(r.v[7]), "=r"(b)
-        : "r"(k0), "r"(k3), "r"(k6));
-    return b & 1u;
+        : "r"(m), "r"(c));
+    return b;
 }
 
-// r = a + b mod p (weak).  a + b < 2^257; a carry out of 2^256 is replaced by
-// adding K = 2^256 mod p.  A second carry (only when the first fold lands at
-// or above 2^256, probability about 2^-32) takes a branch.
+// r = a + b mod p (weak). A carry out of 2^256 is paid for by subtracting p; in
+// the rare case (about 2^-32) that this does not take the sum below 2^256, a
+// second subtraction does.
 __device__ __forceinline__ void fe_add(fe& r, const fe& a, const fe& b) {
     uint32_t c;
     asm("add.cc.u32  %0, %9, %17;\n\t"
@@ -128,13 +132,12 @@ __device__ __forceinline__ void fe_add(fe& r, const fe& a, const fe& b) {
         : "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]),
           "r"(a.v[6]), "r"(a.v[7]), "r"(b.v[0]), "r"(b.v[1]), "r"(b.v[2]), "r"(b.v[3]),
           "r"(b.v[4]), "r"(b.v[5]), "r"(b.v[6]), "r"(b.v[7]));
-    c = fe_add_K_masked(r, 0u - c);
-    if (c) fe_add_K_masked(r, 0xffffffffu);
+    c += fe_sub_p_times(r, c);           // the net top word, 0 but for the rare case
+    if (c) fe_sub_p_times(r, c);
 }
 
-// r = a - b mod p (weak).  A borrow means the register holds a - b + 2^256;
-// subtracting K turns that into a - b + p; a second borrow (only if b - a > p,
-// which needs a weakly reduced b >= p) subtracts K again on a branch.
+// r = a - b mod p (weak). A borrow is paid for by adding p; in the rare case
+// that the value stays negative (b - a > p, which needs b >= p) once more.
 __device__ __forceinline__ void fe_sub(fe& r, const fe& a, const fe& b) {
     uint32_t bw;
     asm("sub.cc.u32  %0, %9, %17;\n\t"
@@ -151,8 +154,8 @@ __device__ __forceinline__ void fe_sub(fe& r, const fe& a, const fe& b) {
         : "r"(a.v[0]), "r"(a.v[1]), "r"(a.v[2]), "r"(a.v[3]), "r"(a.v[4]), "r"(a.v[5]),
           "r"(a.v[6]), "r"(a.v[7]), "r"(b.v[0]), "r"(b.v[1]), "r"(b.v[2]), "r"(b.v[3]),
           "r"(b.v[4]), "r"(b.v[5]), "r"(b.v[6]), "r"(b.v[7]));
-    bw = fe_sub_K_masked(r, bw);
-    if (bw) fe_sub_K_masked(r, 0xffffffffu);
+    bw += fe_add_p_masked(r, bw);
+    if (bw) fe_add_p_masked(r, bw);
 }
 
 __device__ __forceinline__ void fe_dbl(fe& r, const fe& a) { fe_add(r, a, a); }
@@ -272,11 +275,22 @@ __device__ __forceinline__ void fe_reduce(fe& r, uint32_t t[16]) {
         "addc.u32    %7, 0, 0;"
         : "+r"(t[9]), "+r"(t[10]), "+r"(t[11]), "+r"(t[12]), "+r"(t[13]), "+r"(t[14]), "+r"(t[15]), "=r"(c)
         : "r"(t[6]), "r"(t[7]), "r"(D1), "r"(D2), "r"(D3));
-    // The value (t + q p) / R is below 2^256 + p: on a carry subtract p once
-    // (add K and drop the carry).
+    // The value (t + q p) / R is below 2^256 + p: on a carry add K once (and
+    // drop the carry), with c itself and -c as the words of c K.
 #pragma unroll
     for (int i = 0; i < 8; i++) r.v[i] = t[8 + i];
-    fe_add_K_masked(r, 0u - c);
+    const uint32_t n = 0u - c;
+    asm("add.cc.u32  %0, %0, %8;\n\t"
+        "addc.cc.u32 %1, %1, 0;\n\t"
+        "addc.cc.u32 %2, %2, 0;\n\t"
+        "addc.cc.u32 %3, %3, %9;\n\t"
+        "addc.cc.u32 %4, %4, %9;\n\t"
+        "addc.cc.u32 %5, %5, %9;\n\t"
+        "addc.cc.u32 %6, %6, %10;\n\t"
+        "addc.u32    %7, %7, 0;"
+        : "+r"(r.v[0]), "+r"(r.v[1]), "+r"(r.v[2]), "+r"(r.v[3]), "+r"(r.v[4]), "+r"(r.v[5]),
+          "+r"(r.v[6]), "+r"(r.v[7])
+        : "r"(c), "r"(n), "r"(n << 1));
 }
 
 // Rows of fused wide multiply-adds.  A 64-bit product a_j b_i lands on words
@@ -612,32 +626,19 @@ __device__ __forceinline__ fe fe_mulsub(const fe& a, const fe& b, const fe& c, c
           "+r"(u[15]), "=r"(bw)
         : "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
           "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]));
-    // On a borrow (bw = 0xffffffff) add p to the high half.
-    uint32_t c2;
-    asm("add.cc.u32  %0, %0, %9;\n\t"
-        "addc.cc.u32 %1, %1, %9;\n\t"
-        "addc.cc.u32 %2, %2, %9;\n\t"
-        "addc.cc.u32 %3, %3, 0;\n\t"
-        "addc.cc.u32 %4, %4, 0;\n\t"
-        "addc.cc.u32 %5, %5, 0;\n\t"
-        "addc.cc.u32 %6, %6, %10;\n\t"
-        "addc.cc.u32 %7, %7, %9;\n\t"
-        "addc.u32    %8, 0, 0;"
-        : "+r"(u[8]), "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]),
-          "+r"(u[15]), "=r"(c2)
-        : "r"(bw), "r"(bw & 1u));
-    if (bw && !c2) {  // still negative (needs c d - a b > p 2^256): add p 2^256 again
-        asm("add.cc.u32  %0, %0, 0xffffffff;\n\t"
-            "addc.cc.u32 %1, %1, 0xffffffff;\n\t"
-            "addc.cc.u32 %2, %2, 0xffffffff;\n\t"
-            "addc.cc.u32 %3, %3, 0;\n\t"
-            "addc.cc.u32 %4, %4, 0;\n\t"
-            "addc.cc.u32 %5, %5, 0;\n\t"
-            "addc.cc.u32 %6, %6, 1;\n\t"
-            "addc.u32    %7, %7, 0xffffffff;"
-            : "+r"(u[8]), "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]),
-              "+r"(u[15]));
-    }
+    // On a borrow (bw = 0xffffffff) add p to the high half, twice in the rare
+    // case (c d - a b > p 2^256) that it stays negative. As a loop, that case is
+    // a branch of its own and ends the block of instructions that the assembler
+    // schedules as one: the gather's inlined addition, whose carries overflow
+    // the predicate registers otherwise, took 25.4 ms a step with an if and
+    // 23.9 with the loop (w = 4, 1024 x 1024 x 256).
+    fe h;
+#pragma unroll
+    for (int i = 0; i < 8; i++) h.v[i] = u[8 + i];
+    bw += fe_add_p_masked(h, bw);
+    while (bw) bw += fe_add_p_masked(h, bw);
+#pragma unroll
+    for (int i = 0; i < 8; i++) u[8 + i] = h.v[i];
     fe r;
     fe_reduce(r, u);
     return r;

@@ -132,9 +132,9 @@ __device__ __forceinline__ void block_normalize_jacz(aff out[E], const jacz P[E]
 }
 
 // Blocks per SM the register allocation must allow: 262144 encryptions took
-// 2.28, 2.11, 2.04 and 2.03 ms at 3, 4, 5 and 6 blocks.
+// 1.89, 1.88, 1.92 and 1.86 ms at 4, 5, 6 and 8 blocks.
 #ifndef PCMM_ENCRYPT_MINBLOCKS
-#define PCMM_ENCRYPT_MINBLOCKS 6
+#define PCMM_ENCRYPT_MINBLOCKS 8
 #endif
 
 // Enc(b) = (rG, rH + bG): 32 window lookups per base point, added into

@@ -47,14 +47,14 @@ using namespace pcmm;
 using namespace pcmm::cussen;
 
 // Minimum resident blocks per SM requested from the compiler (its register
-// budget).  Measured on GB300: the gather is pipe-bound (5 blocks at 96
-// registers run as fast as 8); the table build waits on its scratch and
-// spill traffic, so more resident warps pay despite more spilling: table time
-// per headline step 46.3 ms at 4 blocks (128 registers), 45.1 at 5, 45.5 at
-// 6, 45.0 at 7 (72 registers), 47.3 at 8; per wide-value step 261.7, 259.3,
-// 252.7, 247.1 and 261.9 ms.  Build-time tunables.
+// budget).  Measured on GB300: the gather is pipe-bound and wants the
+// registers (w = 4, 1024 x 1024 x 256: 23.9 ms at 4 blocks, 25.1 at 5); the
+// chains of the table build wait on their scratch and spill traffic, so more
+// resident warps pay despite more spilling (at the multiplication of that
+// time, 46.3 ms a step of four widths at 4 blocks, 45.0 at 7, 47.3 at 8).
+// Build-time tunables.
 #ifndef PCMM_GATHER_MINBLOCKS
-#define PCMM_GATHER_MINBLOCKS 5
+#define PCMM_GATHER_MINBLOCKS 4
 #endif
 #ifndef PCMM_TABLE_MINBLOCKS
 #define PCMM_TABLE_MINBLOCKS 7
