@@ -930,42 +930,76 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
 // of a product a b / R a slope comes out in the Montgomery domain, its square
 // is reduced twice, and its product with x1 - x3 is standard again.
 
-// How a pair of points is added when their x's are equal or one of them is
-// infinity.
-enum : int { PAIR_ADD = 0, PAIR_SECOND = 1, PAIR_FIRST = 2, PAIR_DOUBLE = 3, PAIR_CANCEL = 4 };
-
 static __device__ __noinline__ void table_item_call(const TableArgs& a, const PlanPtrs& P, long long item,
                                                     uint4* scratch) {
     table_item(a, P, item, scratch);
 }
 
-static __device__ __noinline__ int special_pair(const aff& A, const aff& B, const fe& dx) {
+// Pairs whose x's are equal or of which one is at infinity. They take the
+// rare, out-of-line way: pair_factor gives the factor that the pair
+// contributes to the shared inversion (2 y for a doubling, 1 where there is
+// nothing to invert), pair_sum the sum, given the inverse of the factor.
+enum : int { PAIR_ADD = 0, PAIR_SECOND = 1, PAIR_FIRST = 2, PAIR_DOUBLE = 3, PAIR_CANCEL = 4 };
+
+__device__ __forceinline__ int pair_kind(const aff& A, const aff& B, const fe& dx) {
     if (aff_is_inf(B)) return PAIR_FIRST;
     if (aff_is_inf(A)) return PAIR_SECOND;
     if (!fe_is_zero(dx)) return PAIR_ADD;
     return fe_equal(A.y, B.y) ? PAIR_DOUBLE : PAIR_CANCEL;
 }
 
-// 3 x^2 - 3 for a standard residue x.
-static __device__ __noinline__ fe tangent_num(const fe& x) {
-    fe one, t;
-    fe_zero(one);
-    one.v[0] = 1u;
-    fe_to_mont(t, fsqr(x));          // x^2
-    fe_sub(t, t, one);
-    fe r;
-    fe_add(r, t, t);
-    fe_add(r, r, t);
-    return r;
+static __device__ __noinline__ void pair_factor(fe& dx, const aff& A, const aff& B) {
+    const int kind = pair_kind(A, B, dx);
+    if (kind == PAIR_DOUBLE) fe_add(dx, A.y, A.y);
+    else if (kind != PAIR_ADD) fe_one(dx);
+}
+
+// S = A + B for standard residues, finv = (factor)^-1 R^2.
+static __device__ __noinline__ void pair_sum(aff& S, const aff& A, const aff& B, const fe& finv) {
+    fe d, num;
+    fe_sub(d, B.x, A.x);
+    const int kind = pair_kind(A, B, d);
+    if (kind == PAIR_FIRST) {
+        S = A;
+        return;
+    }
+    if (kind == PAIR_SECOND) {
+        S = B;
+        return;
+    }
+    if (kind == PAIR_CANCEL) {
+        fe_zero(S.x);
+        fe_zero(S.y);
+        return;
+    }
+    if (kind == PAIR_DOUBLE) {           // 3 x^2 - 3
+        fe one, t;
+        fe_zero(one);
+        one.v[0] = 1u;
+        fe_to_mont(t, fsqr(A.x));
+        fe_sub(t, t, one);
+        fe_add(num, t, t);
+        fe_add(num, num, t);
+    } else {
+        fe_sub(num, B.y, A.y);
+    }
+    const fe lam = fmul(num, finv);
+    fe t = fsqr(lam);
+    fe_from_mont(t, t);
+    fe_sub(t, t, A.x);
+    fe_sub(S.x, t, B.x);
+    fe_sub(t, A.x, S.x);
+    t = fmul(lam, t);
+    fe_sub(S.y, t, A.y);
 }
 
 __device__ __forceinline__ bool words345_zero(const fe& a) { return (a.v[3] | a.v[4] | a.v[5]) == 0u; }
 
-// The sums of pair(i) for i < cnt, each handed to put(i, sum): pair sets the
-// two lane-planar affine entries and returns false where there is nothing to
-// add. pref: cnt field elements of lane-planar scratch. All 128 threads of
-// the block call; cnt may differ from warp to warp. `turn` names the warp
-// that inverts.
+// The sums of pair(i) for i < cnt, each handed to put(i, sum) in canonical
+// form: pair sets the two lane-planar canonical entries and returns false where
+// there is nothing to add. pref: cnt field elements of lane-planar scratch.
+// All 128 threads of the block call; cnt may differ from warp to warp. `turn`
+// names the warp that inverts.
 template <class Pair, class Put>
 __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4* pref, uint4* sm, unsigned turn) {
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
@@ -977,21 +1011,16 @@ __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4*
     for (int i = 0; i < cnt; i++) {
         const uint4 *pa, *pb;
         if (!pair(i, pa, pb)) continue;
-        aff A, B;
-        fe_from_quads(A.x, pa[0], pa[32]);
-        fe_from_quads(B.x, pb[0], pb[32]);
-        fe dx;
-        fe_sub(dx, B.x, A.x);
+        fe ax, bx, dx;
+        fe_from_quads(ax, pa[0], pa[32]);
+        fe_from_quads(bx, pb[0], pb[32]);
+        fe_sub_canon(dx, bx, ax);
         // Words 3..5 are zero in 0 and in p: no zero passes this test.
-        const bool sp = words345_zero(dx) || words345_zero(A.x) || words345_zero(B.x);
-        if (__any_sync(all, sp)) {
-            if (sp) {
-                fe_from_quads(A.y, pa[64], pa[96]);
-                fe_from_quads(B.y, pb[64], pb[96]);
-                const int kind = special_pair(A, B, dx);
-                if (kind == PAIR_DOUBLE) fe_add(dx, A.y, A.y);
-                else if (kind != PAIR_ADD) fe_one(dx);
-            }
+        if (__any_sync(all, words345_zero(dx) || words345_zero(ax) || words345_zero(bx))) {
+            aff A, B;
+            lp_load_aff(A, pa, 0, 0);
+            lp_load_aff(B, pb, 0, 0);
+            pair_factor(dx, A, B);
         }
         lp_store_fe(pref, i, lane, run);
         fe_mul(run, run, dx);
@@ -1009,43 +1038,33 @@ __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4*
         const uint4 *pa, *pb;
         if (!pair(i, pa, pb)) continue;
         aff A, B, S;
-        fe pr, lam, t;
+        fe pr, dinv, dx;
         lp_load_fe(pr, pref, i, lane);
         lp_load_aff(A, pa, 0, 0);
         lp_load_aff(B, pb, 0, 0);
-        fe dx, dy;
-        fe_sub(dx, B.x, A.x);
-        fe_sub(dy, B.y, A.y);
-        int kind = PAIR_ADD;
-        const bool sp = words345_zero(dx) || words345_zero(A.x) || words345_zero(B.x);
-        const bool anysp = __any_sync(all, sp);
-        if (anysp && sp) {
-            kind = special_pair(A, B, dx);
-            if (kind == PAIR_DOUBLE) {
-                fe_add(dx, A.y, A.y);
-                dy = tangent_num(A.x);
-            } else if (kind != PAIR_ADD) {
-                fe_one(dx);
-            }
-        }
-        fe_mul(lam, inv, pr);
-        fe_mul(inv, inv, dx);
-        fe_mul(lam, dy, lam);
-        t = fe_sqr_std(lam);
-        fe_sub(t, t, A.x);
-        fe_sub(S.x, t, B.x);
-        fe_sub(t, A.x, S.x);
-        fe_mul(t, lam, t);
-        fe_sub(S.y, t, A.y);
-        fe_canon(S.x, S.x);
-        fe_canon(S.y, S.y);
-        if (anysp) {
-            if (kind == PAIR_FIRST) S = A;
-            if (kind == PAIR_SECOND) S = B;
-            if (kind == PAIR_CANCEL) {
-                fe_zero(S.x);
-                fe_zero(S.y);
-            }
+        fe_sub_canon(dx, B.x, A.x);
+        const bool rare = __any_sync(all, words345_zero(dx) || words345_zero(A.x) || words345_zero(B.x));
+        if (rare) {
+            pair_factor(dx, A, B);
+            dinv = fmul(inv, pr);
+            inv = fmul(inv, dx);
+            pair_sum(S, A, B, dinv);
+            fe_canon(S.x, S.x);
+            fe_canon(S.y, S.y);
+        } else {
+            fe lam, t;
+            fe_mul(dinv, inv, pr);
+            fe_mul(inv, inv, dx);
+            fe_sub_canon(t, B.y, A.y);
+            fe_mul(lam, t, dinv);
+            t = fe_sqr_std(lam);
+            fe_sub_canon(t, t, A.x);
+            fe_sub_canon(t, t, B.x);
+            fe_canon(S.x, t);
+            fe_sub_canon(t, A.x, S.x);
+            fe_mul(t, lam, t);
+            fe_sub_canon(S.y, t, A.y);
+            fe_canon(S.y, S.y);
         }
         put(i, S);
     }
@@ -1196,6 +1215,8 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
             aff B, S;
             if (place == 0) {
                 load_aff(S, Bc, nl, (size_t)(c0 + t) * a.l + jj);
+                fe_canon(S.x, S.x);
+                fe_canon(S.y, S.y);
                 B = S;
                 aff_to_mont(B);
             } else {
