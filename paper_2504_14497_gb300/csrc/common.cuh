@@ -330,6 +330,7 @@ __device__ __forceinline__ void group_inverse(fe& tinv, const fe& t, bool shared
 // Whether x holds on every lane of the warp or, with `shared`, on every
 // thread of the block (then all threads of the block must call).
 __device__ __forceinline__ bool group_all(bool x, bool shared) {
+    __syncwarp();   // lanes may come from different branches; a block barrier wants the warp whole
     return shared ? __syncthreads_and(x) != 0 : __all_sync(0xffffffffu, x);
 }
 

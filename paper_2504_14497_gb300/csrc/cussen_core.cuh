@@ -26,6 +26,11 @@ constexpr int NLEV = PCMM_N_ITER;   // compression iterations N
 #ifndef PCMM_TABLE_INLINE
 #define PCMM_TABLE_INLINE 0
 #endif
+// The same for the digit build's chains: table of 1024 x 1024 x 256 at w = 8 12.6,
+// 12.7, 12.6 and 12.3 ms at 0, 1, 2 and 3.
+#ifndef PCMM_DIGIT_INLINE
+#define PCMM_DIGIT_INLINE 3
+#endif
 constexpr uint16_t NO_RANK = 0xFFFFu;
 constexpr int PLAN_THREADS = 256;
 
@@ -930,11 +935,6 @@ __device__ __forceinline__ void table_item(const TableArgs& a, const PlanPtrs& P
 // of a product a b / R a slope comes out in the Montgomery domain, its square
 // is reduced twice, and its product with x1 - x3 is standard again.
 
-static __device__ __noinline__ void table_item_call(const TableArgs& a, const PlanPtrs& P, long long item,
-                                                    uint4* scratch) {
-    table_item(a, P, item, scratch);
-}
-
 // Pairs whose x's are equal or of which one is at infinity. They take the
 // rare, out-of-line way: pair_factor gives the factor that the pair
 // contributes to the shared inversion (2 y for a doubling, 1 where there is
@@ -1027,6 +1027,7 @@ __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4*
     }
     sm[tid] = fe_lo(run);
     sm[128 + tid] = fe_hi(run);
+    __syncwarp();
     __syncthreads();
     if (warp == (turn & 3u)) fold_inverse128(sm);
     __syncthreads();
@@ -1070,6 +1071,37 @@ __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4*
     }
 }
 
+// The generator (Montgomery domain): it stands in for a point at infinity in
+// the digits' chains, whose multiples the lane then stores as infinity.
+__device__ __forceinline__ void aff_generator(aff& G) {
+    const uint32_t x[8] = {0x18a9143cu, 0x79e730d4u, 0x5fedb601u, 0x75ba95fcu,
+                           0x77622510u, 0x79fb732bu, 0xa53755c6u, 0x18905f76u};
+    const uint32_t y[8] = {0xce95560au, 0xddf25357u, 0xba19e45cu, 0x8b4ab8e4u,
+                           0xdd21f325u, 0xd2e88688u, 0x25885d85u, 0x8571ff18u};
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        G.x.v[i] = x[i];
+        G.y.v[i] = y[i];
+    }
+}
+
+// v B in affine coordinates for a lane whose chain met infinity, which takes a
+// point of order 16 or less and so an input off the curve.
+static __device__ __noinline__ aff small_multiple(const aff& B, uint32_t v) {
+    jac J;
+    jac_mul_small(J, B, v);
+    aff Q;
+    if (jac_is_inf(J)) {
+        fe_zero(Q.x);
+        fe_zero(Q.y);
+        return Q;
+    }
+    fe zi;
+    fe_inv(zi, J.Z);
+    jac_to_aff_with_zinv(Q, J, zi);
+    return Q;
+}
+
 // Bits of digit d: four, or what is left of its column.
 __device__ __forceinline__ int digit_bits(const TableArgs& a, int d) {
     const int r = a.w - 4 * (d % a.dpc);
@@ -1077,10 +1109,11 @@ __device__ __forceinline__ int digit_bits(const TableArgs& a, int d) {
 }
 
 // Scratch of the digit build, in uint4 per warp: the values of the level
-// lists, the digits' chains (6 + 2 quads an entry), the next places' base
-// points, both halves' tables and the prefix products.
+// lists, the factors of the digits' chains (4 quads an entry; X and Y wait in
+// the half's entry), the next places' base points, both halves' tables and
+// the prefix products.
 struct DigitScratch {
-    size_t vals, chain, rat, base, half, pref, total;
+    size_t vals, rat, base, half, pref, total;
 };
 __host__ __device__ inline DigitScratch digit_scratch(int w, int k, int dpc, int hl, int hh, int n1max, int l2max,
                                                       int emax) {
@@ -1088,19 +1121,18 @@ __host__ __device__ inline DigitScratch digit_scratch(int w, int k, int dpc, int
     size_t off = 0;
     D.vals = off;
     off += (size_t)((n1max + 2 * l2max) * 2 + 15) / 16 + 1;
-    const int place = w < 4 ? w : 4;
-    const size_t chain = (size_t)k * (1 << place);
-    D.chain = off;
-    off += chain * 192;
     D.rat = off;
-    off += chain * 64;
+    off += (size_t)k * (1 << (w < 4 ? w : 4)) * 128;
     D.base = off;
     off += (size_t)(dpc > 1 ? k : 0) * 128;
     D.half = off;
     off += ((size_t)(1 << hl) + (size_t)(1 << hh)) * 128;
     D.pref = off;
-    size_t np = (size_t)1 << (hl > hh ? hl : hh);
-    np = 2 * np > (size_t)emax ? 2 * np : (size_t)emax;
+    size_t np = 0;                       // a single digit has no pairs to add
+    if (k * dpc > 1) {
+        np = (size_t)2 << (hl > hh ? hl : hh);
+        if (np < (size_t)emax) np = emax;
+    }
     off += (np > (size_t)k ? np : (size_t)k) * 64;
     D.total = off;
     return D;
@@ -1135,10 +1167,8 @@ __device__ __forceinline__ const uint16_t* column_values(const PlanPtrs& P, int 
 }
 
 // Table of one warp item by digits. All 128 threads of the block call (valid:
-// the warp has an item); sm: 256 uint4 of shared memory. Returns false, for
-// the whole block, when a chain met infinity (an input at infinity): nothing
-// the caller reads has been written then, and table_item builds the tables.
-__device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
+// the warp has an item); sm: 256 uint4 of shared memory.
+__device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
                                             uint4* scratch, uint4* sm) {
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
     const int s_local = valid ? (int)(item / (2 * a.njb)) : 0;
@@ -1152,7 +1182,6 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
     const size_t nl = (size_t)a.n * a.l;
     const uint4* Bc = a.ctB + (size_t)c * 4 * nl;
     const DigitScratch D = digit_scratch(a.w, a.k, a.dpc, a.hl, a.hh, a.n1max, a.l2max, a.emax);
-    uint4* chain = scratch + D.chain;
     uint4* rat = scratch + D.rat;
     uint4* base = scratch + D.base;
     uint4* half = scratch + D.half;
@@ -1205,9 +1234,10 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
         for (int x = dg < a.ns ? 0 : a.ns; x < dg; x++) o += digit_bits(a, x);
         return half + (dg < a.ns ? (size_t)0 : (size_t)128 << a.hl);
     };
-    bool ok = true;
+    uint32_t atinf = 0;          // columns (by t) whose point is infinity in this lane
     for (int place = 0; place < a.dpc; place++) {
         const bool more = place + 1 < a.dpc;
+        uint32_t failed = 0;     // columns whose chain met infinity in this lane
         fe acc;
         fe_one(acc);
         for (int t = 0; t < kw; t++) {
@@ -1217,45 +1247,64 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
                 load_aff(S, Bc, nl, (size_t)(c0 + t) * a.l + jj);
                 fe_canon(S.x, S.x);
                 fe_canon(S.y, S.y);
+                if (aff_is_inf(S)) atinf |= 1u << t;
                 B = S;
                 aff_to_mont(B);
             } else {
                 lp_load_aff(B, base, t, lane);
+                if (aff_is_inf(B)) atinf |= 1u << t;
                 S = B;
                 aff_from_mont(S);
+            }
+            if ((atinf >> t) & 1u) {
+                fe_zero(S.x);
+                fe_zero(S.y);
+                aff_generator(B);
             }
             int o;
             uint4* hb = half_at(dg, o);
             lp_store_aff(hb, 1 << o, lane, S);
             if (len < 2) continue;
             jacz P1;
-            jacz_set_inf(P1);
-            uint4* ch = chain + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 192;
-            uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 64;
-            for (int e = 0; e < len; e++) {
+            P1.X = B.x;
+            P1.Y = B.y;
+            fe_one(P1.ZZ);
+            fe_one(P1.ZZZ);
+            bool ok = true;
+            uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 128;
+            // Entry e is (e + 1) times the point: X and Y to its place, ZZ's and
+            // ZZZ's factors to slot e.  The first step is a doubling.
+#pragma unroll 1
+            for (int e = 1; e < len; e++) {
+                uint4* xy = (more && e == len - 1 ? base + (size_t)t * 128 : hb + ((size_t)(e + 1) << o) * 128) + lane;
+                uint4* f = rt + (size_t)e * 128 + lane;
                 fe r2, r3;
-                jacz_madd_ratio_t<PCMM_TABLE_INLINE>(P1, B, r2, r3, ok, e == 0);
-                uint4* b = ch + (size_t)e * 192 + lane;
-                b[0] = fe_lo(P1.X);
-                b[32] = fe_hi(P1.X);
-                b[64] = fe_lo(P1.Y);
-                b[96] = fe_hi(P1.Y);
-                b[128] = fe_lo(r3);
-                b[160] = fe_hi(r3);
-                lp_store_fe(rt, e, lane, r2);
+                jacz_madd_ratio_t<PCMM_DIGIT_INLINE>(P1, B, r2, r3, ok, false);
+                xy[0] = fe_lo(P1.X);
+                xy[32] = fe_hi(P1.X);
+                xy[64] = fe_lo(P1.Y);
+                xy[96] = fe_hi(P1.Y);
+                f[0] = fe_lo(r2);
+                f[32] = fe_hi(r2);
+                f[64] = fe_lo(r3);
+                f[96] = fe_hi(r3);
             }
             // The chain's product ZZ ZZZ for the shared inversion; ZZ and ZZZ
-            // wait in slot 0, whose factors are 1.
-            uint4* b = ch + lane;
-            b[0] = fe_lo(P1.ZZ);
-            b[32] = fe_hi(P1.ZZ);
-            b[64] = fe_lo(P1.ZZZ);
-            b[96] = fe_hi(P1.ZZZ);
+            // wait in slot 0, whose factors would be 1.
+            aff zz;
+            zz.x = P1.ZZ;
+            zz.y = P1.ZZZ;
+            if (!ok) {
+                failed |= 1u << t;
+                fe_one(zz.x);
+                fe_one(zz.y);
+            }
+            lp_store_aff(rt, 0, lane, zz);
             lp_store_fe(pref, t, lane, acc);
-            acc = fmul(acc, fmul(P1.ZZ, P1.ZZZ));
+            acc = fmul(acc, fmul(zz.x, zz.y));
         }
         if (a.w == 1) break;                    // no chains: nothing to invert
-        if (!__syncthreads_and(ok)) return false;
+        __syncwarp();
         sm[tid] = fe_lo(acc);
         sm[128 + tid] = fe_hi(acc);
         __syncthreads();
@@ -1267,15 +1316,14 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
         for (int t = kw - 1; t >= 0; t--) {
             const int dg = t * a.dpc + place, len = (1 << digit_bits(a, dg)) - (more ? 0 : 1);
             if (len < 2) continue;
-            const uint4* ch = chain + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 192;
-            const uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 64;
-            fe zz, zzz, pr;
-            fe_from_quads(zz, ch[lane], ch[32 + lane]);
-            fe_from_quads(zzz, ch[64 + lane], ch[96 + lane]);
+            const uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 128;
+            aff zz;
+            fe pr;
+            lp_load_aff(zz, rt, 0, lane);
             lp_load_fe(pr, pref, t, lane);
             const fe i5 = fmul(inv, pr);
-            inv = fmul(inv, fmul(zz, zzz));
-            fe zi = fmul(i5, zzz), zzi = fmul(i5, zz);   // ZZ^-1 and ZZZ^-1 of the last entry
+            inv = fmul(inv, fmul(zz.x, zz.y));
+            fe zi = fmul(i5, zz.y), zzi = fmul(i5, zz.x);   // ZZ^-1 and ZZZ^-1 of the last entry
             int o;
             uint4* hb = half_at(dg, o);
             for (int e = len - 1; e >= 1; e--) {
@@ -1285,24 +1333,34 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
                     fe_from_mont(zi, zi);
                     fe_from_mont(zzi, zzi);
                 }
-                const uint4* b = ch + (size_t)e * 192 + lane;
-                fe X, Y, r2, r3;
-                fe_from_quads(X, b[0], b[32]);
-                fe_from_quads(Y, b[64], b[96]);
-                aff Q;
-                Q.x = fmul(X, zi);
-                Q.y = fmul(Y, zzi);
+                aff Q, r;
+                if (last) lp_load_aff(Q, base, t, lane);
+                else lp_load_aff(Q, hb, (e + 1) << o, lane);
+                Q.x = fmul(Q.x, zi);
+                Q.y = fmul(Q.y, zzi);
+                if (failed) {
+                    if ((failed >> t) & 1u) {
+                        aff B;
+                        lp_load_aff(B, hb, 1 << o, lane);
+                        aff_to_mont(B);
+                        Q = small_multiple(B, (uint32_t)(e + 1));
+                        if (!last) aff_from_mont(Q);
+                    }
+                }
                 if (last) {
                     lp_store_aff(base, t, lane, Q);
                 } else {
                     fe_canon(Q.x, Q.x);
                     fe_canon(Q.y, Q.y);
+                    if ((atinf >> t) & 1u) {
+                        fe_zero(Q.x);
+                        fe_zero(Q.y);
+                    }
                     lp_store_aff(hb, (e + 1) << o, lane, Q);
                 }
-                lp_load_fe(r2, rt, e, lane);
-                fe_from_quads(r3, b[128], b[160]);
-                zi = fmul(zi, r2);
-                zzi = fmul(zzi, r3);
+                lp_load_aff(r, rt, e, lane);
+                zi = fmul(zi, r.x);
+                zzi = fmul(zzi, r.y);
             }
         }
     }
@@ -1356,7 +1414,7 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
     };
     const uint32_t lmask = (1u << a.hl) - 1u;
     const uint4* high = half + ((size_t)128 << a.hl);
-    affine_batch(
+    if (a.nd > 1) affine_batch(
         E,
         [&](int e, const uint4*& pa, const uint4*& pb) -> bool {
             const uint32_t code = codes[e];
@@ -1372,7 +1430,6 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
         lp_load_aff(Q, code & lmask ? half + (size_t)(code & lmask) * 128 : high + (size_t)(code >> a.hl) * 128, 0, lane);
         store_table(e, Q);
     }
-    return true;
 }
 
 // The digits and halves of a strip code, and whether the digit build takes
@@ -1380,10 +1437,11 @@ __device__ __forceinline__ bool table_block(const TableArgs& a, const PlanPtrs& 
 inline bool digit_split(const Layout& L, TableArgs& a) {
     a.dpc = (L.w + 3) / 4;
     a.nd = L.k * a.dpc;
-    a.ns = a.hl = a.hh = 0;
-    if (a.nd < 2) return false;
+    a.ns = 1;
+    a.hl = L.w;
+    a.hh = 0;
     auto bits = [&](int d) { const int r = L.w - 4 * (d % a.dpc); return r < 4 ? r : 4; };
-    long long best = -1;
+    long long best = a.nd == 1 ? 1LL << L.w : -1;
     int lo = 0;
     for (int x = 1; x < a.nd; x++) {
         lo += bits(x - 1);
@@ -1391,7 +1449,9 @@ inline bool digit_split(const Layout& L, TableArgs& a) {
         const long long size = (1LL << lo) + (1LL << hi);
         if (best < 0 || size < best) { best = size; a.ns = x; a.hl = lo; a.hh = hi; }
     }
-    // The halves must not outweigh the entries.  Table times (ms) by chains and
+    // The halves must not outweigh the entries (with one digit, its multiples
+    // are the entries: 10 x 128 x 1 at w = 4 takes 135 us by chains and 118 us by
+    // digits).  Table times (ms) by chains and
     // by digits, 256 x 256 columns: w = 12 with 128 rows (halves 272) 4.90 and
     // 5.38, with 256 rows 7.22 and 6.63; w = 16 with 256 rows (halves 512) 12.0
     // and 9.96, with 512 rows 18.2 and 12.8; w = 8 with 16 rows (halves 32) 1.17

@@ -153,8 +153,8 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
                 ta.item_u4 = I.item_u4;
                 ta.table = tbuf;
                 ta.table_points = I.table_points;
-                if (!(I.digits && table_block(ta, I.P, item, real, my_scratch, sh_inv)) && real)
-                    table_item_call(ta, I.P, item, my_scratch);
+                if (I.digits) table_block(ta, I.P, item, real, my_scratch, sh_inv);
+                else if (real) table_item(ta, I.P, item, my_scratch);
             }
         } else if (real) {
             GatherArgs ga;
@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
             gather_item<true>(ga, I.P, item);
         }
         __threadfence();
+        __syncwarp();
         __syncthreads();
         if (threadIdx.x == 0) {
             const long long left = sg.count - (t0 - sg.start);

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(128, PCMM_DIGIT_MINBLOCKS) digit_table_kernel(
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const bool valid = item < (long long)a.nstrips_chunk * 2 * a.njb;
     uint4* scratch = a.scratch + (valid ? (size_t)item : (size_t)0) * a.item_u4;
-    if (!table_block(a, P, item, valid, scratch, sm) && valid) table_item_call(a, P, item, scratch);
+    table_block(a, P, item, valid, scratch, sm);
 }
 
 __global__ void __launch_bounds__(128, PCMM_GATHER_MINBLOCKS) gather_kernel(GatherArgs a, PlanPtrs P) {
@@ -119,6 +119,76 @@ __global__ void __launch_bounds__(128) combine_kernel(const uint4* __restrict__ 
     }
     jac_from_mont(acc);
     store_jac(Cc, ml, idx, acc);
+}
+
+// combine_kernel for few outputs, where its chain of additions would be the
+// time: G lanes (a power of two, at least parts) load a part each and add
+// them as a tree, log2 G additions instead of parts.
+__global__ void __launch_bounds__(128) combine_tree_kernel(const uint4* __restrict__ partial, int parts, int G,
+                                                           uint4* __restrict__ ctC, size_t ml, bool first) {
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = (int)(t % G);
+    const bool valid = t / G < 2 * ml;
+    const size_t o = valid ? t / G : 0;
+    const size_t c = o / ml, idx = o % ml;
+    uint4* Cc = ctC + c * 6 * ml;
+    jac acc;
+    if (p < parts) load_jac(acc, partial + (size_t)p * 12 * ml + c * 6 * ml, ml, idx);
+    else jac_set_inf(acc);
+    for (int d = G / 2; d >= 1; d >>= 1) {
+        jac Q;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            Q.X.v[i] = __shfl_down_sync(0xffffffffu, acc.X.v[i], d);
+            Q.Y.v[i] = __shfl_down_sync(0xffffffffu, acc.Y.v[i], d);
+            Q.Z.v[i] = __shfl_down_sync(0xffffffffu, acc.Z.v[i], d);
+        }
+        if (p < d) jac_add(acc, Q);
+        __syncwarp();
+    }
+    if (!valid || p) return;
+    if (!first) {
+        jac prev;
+        load_jac(prev, Cc, ml, idx);
+        jac_to_mont(prev);
+        jac_add(acc, prev);
+    }
+    jac_from_mont(acc);
+    store_jac(Cc, ml, idx, acc);
+}
+
+// Gather of a product of one strip: every output is its row's table entry (Z
+// = 1) or infinity, a copy bound by memory. One warp per row, component and
+// 32 columns. At 512 x 1 x 16384 (w = 4) it takes 241 us, where gather_kernel at
+// its 128 registers keeps too few loads in flight (514 us).
+__global__ void __launch_bounds__(128) gather_copy_kernel(GatherArgs a, PlanPtrs P) {
+    const unsigned lane = threadIdx.x & 31u;
+    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (gw >= (long long)a.m * 2 * a.njb) return;
+    const int i = (int)(gw % a.m), rem = (int)(gw / a.m);
+    const int c = rem / a.njb, jb = rem % a.njb;
+    const int j = jb * 32 + (int)lane;
+    if (j >= a.l) return;
+    const size_t ml = (size_t)a.m * a.l;
+    aff T;
+    fe_zero(T.x);
+    fe_zero(T.y);
+    const uint16_t code = P.rank[(size_t)a.s0 * a.m + i];
+    if (code != NO_RANK) {
+#ifdef PCMM_DEBUG_BOUNDS
+        if (code >= P.nent[a.s0]) {   // a rank past the strip's table
+            atomicOr(P.status, DEV_ERR_BOUNDS);
+            return;
+        }
+#endif
+        load_aff(T, a.table, a.table_points, ((size_t)code * 2 + c) * a.lp + j);
+    }
+    jac out;
+    out.X = T.x;
+    out.Y = T.y;
+    fe_zero(out.Z);
+    out.Z.v[0] = aff_is_inf(T) ? 0u : 1u;
+    store_jac(a.ctC + (size_t)c * 6 * ml, ml, (size_t)i * a.l + j, out);
 }
 
 }  // namespace
@@ -168,15 +238,24 @@ pcmm_status launch_plan(const Layout& L, const TA* A, const PlanPtrs& P, cudaStr
 // Warps per output for the gather of a pass of S strips: when the outputs
 // alone give fewer than GATHER_WARPS_TARGET warps (about four waves of the
 // gather on 152 SMs), each output's strips are split into up to 32 parts of
-// at least 16 strips, and combine_kernel adds the partial sums (one full
-// addition per part against at least 16 mixed additions).
+// at least part_strips strips, and a combine kernel adds the partial sums
+// (one full addition per part against at least part_strips mixed additions).
+// Parts go down to 4 strips while all of them still leave the 608 schedulers
+// with two warps each at most: such a gather takes as long as one part's
+// chain, and the tree that adds the parts is short (10 x 128 x 1 at w = 4: 51 +
+// 41 us with 8 parts of 16 strips added in a row, 22 + 29 us with 32 of 4).
 const long long GATHER_WARPS_TARGET = 12288;
+const long long SCHEDULERS = 608;
+
+int part_strips(const Layout& L, size_t S) {
+    return (long long)L.m * 2 * L.njb * (long long)(S / 4) <= 2 * SCHEDULERS ? 4 : 16;
+}
 
 int gather_parts(const Layout& L, size_t S) {
     const long long warps = (long long)L.m * 2 * L.njb;
     if (warps >= GATHER_WARPS_TARGET) return 1;
     long long parts = (GATHER_WARPS_TARGET + warps - 1) / warps;
-    const long long by_strips = (long long)S / 16;
+    const long long by_strips = (long long)S / part_strips(L, S);
     if (parts > by_strips) parts = by_strips;
     if (parts > 32) parts = 32;
     return parts < 1 ? 1 : (int)parts;
@@ -226,19 +305,28 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         ga.table_points = ta.table_points;
         ga.ctC = (uint4*)ctC;
         // A short last chunk may take fewer parts than the buffer holds.
-        const int pc = parts > 1 ? (sc / 16 < parts ? (sc / 16 > 1 ? sc / 16 : 1) : parts) : 1;
+        int pc = sc / part_strips(L, S);
+        pc = pc < 1 ? 1 : pc < parts ? pc : parts;
         ga.parts = pc;
         ga.partial = (uint4*)partial;
         const long long warps = (long long)L.m * 2 * L.njb * pc;
         {
             ProfScope ps(KID_GATHER, st);
-            gather_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(ga, P);
+            if (ga.first && sc == 1) gather_copy_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(ga, P);
+            else gather_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(ga, P);
         }
         PCMM_CUDA_CHECK_LAUNCH();
         if (pc > 1) {
             ProfScope ps(KID_COMBINE, st);
-            combine_kernel<<<(unsigned)((2 * ml + 127) / 128), 128, 0, st>>>((const uint4*)partial, pc,
-                                                                           (uint4*)ctC, ml, s0 == 0);
+            int G = 2;
+            while (G < pc) G *= 2;
+            const size_t lanes = 2 * ml * G;
+            if (lanes <= (size_t)SCHEDULERS * 32)
+                combine_tree_kernel<<<(unsigned)((lanes + 127) / 128), 128, 0, st>>>((const uint4*)partial, pc, G,
+                                                                                    (uint4*)ctC, ml, s0 == 0);
+            else
+                combine_kernel<<<(unsigned)((2 * ml + 127) / 128), 128, 0, st>>>((const uint4*)partial, pc,
+                                                                                (uint4*)ctC, ml, s0 == 0);
         }
         PCMM_CUDA_CHECK_LAUNCH();
     }
