@@ -31,6 +31,10 @@ constexpr int NLEV = PCMM_N_ITER;   // compression iterations N
 #ifndef PCMM_DIGIT_INLINE
 #define PCMM_DIGIT_INLINE 3
 #endif
+// And for the build with signed pairs: 10.8, 10.7, 10.5 and 10.7 ms.
+#ifndef PCMM_SIGNED_INLINE
+#define PCMM_SIGNED_INLINE 2
+#endif
 constexpr uint16_t NO_RANK = 0xFFFFu;
 constexpr int PLAN_THREADS = 256;
 
@@ -438,6 +442,7 @@ struct TableArgs {
     // Digit build (table_block): digits per column, digits of all columns,
     // digits of the low half and the bits of both halves.
     int dpc, nd, ns, hl, hh;
+    bool sgn;              // some of the digits make signed pairs (signed_pair)
 };
 
 __device__ __forceinline__ void lp_store_aff(uint4* base, int e, unsigned lane, const aff& Q) {
@@ -945,13 +950,16 @@ __device__ __forceinline__ int pair_kind(const aff& A, const aff& B, const fe& d
     if (aff_is_inf(B)) return PAIR_FIRST;
     if (aff_is_inf(A)) return PAIR_SECOND;
     if (!fe_is_zero(dx)) return PAIR_ADD;
-    return fe_equal(A.y, B.y) ? PAIR_DOUBLE : PAIR_CANCEL;
+    return fe_equal(A.y, B.y) && !fe_is_zero(A.y) ? PAIR_DOUBLE : PAIR_CANCEL;
 }
 
+// The same factor serves A + B and A - B: one of them doubles where the other
+// cancels.
 static __device__ __noinline__ void pair_factor(fe& dx, const aff& A, const aff& B) {
     const int kind = pair_kind(A, B, dx);
-    if (kind == PAIR_DOUBLE) fe_add(dx, A.y, A.y);
-    else if (kind != PAIR_ADD) fe_one(dx);
+    if (kind == PAIR_ADD) return;
+    fe_one(dx);
+    if (kind >= PAIR_DOUBLE && !fe_is_zero(A.y)) fe_add(dx, A.y, A.y);
 }
 
 // S = A + B for standard residues, finv = (factor)^-1 R^2.
@@ -995,12 +1003,23 @@ static __device__ __noinline__ void pair_sum(aff& S, const aff& A, const aff& B,
 
 __device__ __forceinline__ bool words345_zero(const fe& a) { return (a.v[3] | a.v[4] | a.v[5]) == 0u; }
 
-// The sums of pair(i) for i < cnt, each handed to put(i, sum) in canonical
-// form: pair sets the two lane-planar canonical entries and returns false where
-// there is nothing to add. pref: cnt field elements of lane-planar scratch.
-// All 128 threads of the block call; cnt may differ from warp to warp. `turn`
-// names the warp that inverts.
-template <class Pair, class Put>
+// With both signs the multiplications are called: inlined, two copies of the
+// sum outgrow the instruction cache (w = 8 below 11.1 against 10.5 ms).
+template <bool BOTH>
+__device__ __forceinline__ fe batch_mul(const fe& a, const fe& b) {
+    if (BOTH) return fmul(a, b);
+    fe r;
+    fe_mul(r, a, b);
+    return r;
+}
+
+// A + B (bit 0 of pair(i, A, B)) and, for BOTH, A - B (bit 1) for i < cnt, each handed to
+// put(i, 0 or 1, sum) in canonical form: pair sets the two lane-planar canonical
+// entries and returns 0 where there is nothing to add. Both signs share the
+// difference of x and its inverse: 7M + 2S instead of 10M + 2S. pref: cnt field
+// elements of lane-planar scratch. All 128 threads of the block call; cnt may
+// differ from warp to warp. `turn` names the warp that inverts.
+template <bool BOTH, class Pair, class Put>
 __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4* pref, uint4* sm, unsigned turn) {
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
     const unsigned all = 0xffffffffu;
@@ -1037,8 +1056,9 @@ __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4*
 #pragma unroll 1
     for (int i = cnt - 1; i >= 0; i--) {
         const uint4 *pa, *pb;
-        if (!pair(i, pa, pb)) continue;
-        aff A, B, S;
+        const unsigned want = pair(i, pa, pb);
+        if (!want) continue;
+        aff A, B;
         fe pr, dinv, dx;
         lp_load_fe(pr, pref, i, lane);
         lp_load_aff(A, pa, 0, 0);
@@ -1049,25 +1069,49 @@ __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4*
             pair_factor(dx, A, B);
             dinv = fmul(inv, pr);
             inv = fmul(inv, dx);
-            pair_sum(S, A, B, dinv);
-            fe_canon(S.x, S.x);
-            fe_canon(S.y, S.y);
-        } else {
+            for (int sign = 0; sign < (BOTH ? 2 : 1); sign++) {
+                aff S;
+                if (sign) {
+                    fe_zero(S.y);
+                    fe_sub_canon(B.y, S.y, B.y);
+                }
+                if (BOTH && !((want >> sign) & 1u)) continue;
+                pair_sum(S, A, B, dinv);
+                fe_canon(S.x, S.x);
+                fe_canon(S.y, S.y);
+                put(i, sign, S);
+            }
+            continue;
+        }
+        dinv = batch_mul<BOTH>(inv, pr);
+        inv = batch_mul<BOTH>(inv, dx);
+        auto finish = [&](int sign) {
+            aff S;
             fe lam, t;
-            fe_mul(dinv, inv, pr);
-            fe_mul(inv, inv, dx);
             fe_sub_canon(t, B.y, A.y);
-            fe_mul(lam, t, dinv);
-            t = fe_sqr_std(lam);
+            lam = batch_mul<BOTH>(t, dinv);
+            if (BOTH) {
+                t = fsqr(lam);
+                fe_from_mont(t, t);
+            } else {
+                t = fe_sqr_std(lam);
+            }
             fe_sub_canon(t, t, A.x);
             fe_sub_canon(t, t, B.x);
             fe_canon(S.x, t);
             fe_sub_canon(t, A.x, S.x);
-            fe_mul(t, lam, t);
+            t = batch_mul<BOTH>(lam, t);
             fe_sub_canon(S.y, t, A.y);
             fe_canon(S.y, S.y);
+            put(i, sign, S);
+        };
+        if (!BOTH || (want & 1u)) finish(0);
+        if (BOTH && (want & 2u)) {
+            fe zero;
+            fe_zero(zero);
+            fe_sub_canon(B.y, zero, B.y);
+            finish(1);
         }
-        put(i, S);
     }
 }
 
@@ -1103,10 +1147,28 @@ static __device__ __noinline__ aff small_multiple(const aff& B, uint32_t v) {
 }
 
 // Bits of digit d: four, or what is left of its column.
-__device__ __forceinline__ int digit_bits(const TableArgs& a, int d) {
+__host__ __device__ inline int digit_bits(const TableArgs& a, int d) {
     const int r = a.w - 4 * (d % a.dpc);
     return r < 4 ? r : 4;
 }
+
+// Signed pairs: where a digit d and the next one d + 1 belong to one column and
+// come first in their half (or are the only two), an entry 16 v + u of theirs is
+// 16 v + u for u <= 8 and 16 (v + 1) - (16 - u) above, so that one factor of the
+// shared inversion serves two entries (affine_batch) and the multiples 9..15 of
+// the lower digit's point are not needed. It takes one more multiple of the
+// upper digit's, 2^bits, which waits in row 0 of the other half (no code 0 is
+// ever read). With one bit in the upper digit there is nothing to share. Table
+// times without and with signed pairs (ms): 1024 x 1024 x 256 at w = 8 12.6 and
+// 10.5, with one value in ten not zero 7.0 and 6.5; 512 x 512 x 256 at w = 16
+// 24.0 and 22.2.
+__host__ __device__ inline bool signed_pair(const TableArgs& a, int d, int end) {
+    return d + 1 < end && d % a.dpc + 1 < a.dpc && digit_bits(a, d + 1) >= 2;
+}
+
+// Shared memory of the digit build, in uint4 per block: the shared inversion,
+// and for each warp the entry of every code and the list of pairs.
+constexpr int DIGIT_SHARED_U4 = 256 + 4 * 48;
 
 // Scratch of the digit build, in uint4 per warp: the values of the level
 // lists, the factors of the digits' chains (4 quads an entry; X and Y wait in
@@ -1166,8 +1228,10 @@ __device__ __forceinline__ const uint16_t* column_values(const PlanPtrs& P, int 
     return cur;
 }
 
-// Table of one warp item by digits. All 128 threads of the block call (valid:
-// the warp has an item); sm: 256 uint4 of shared memory.
+// Table of one warp item by digits, SIGNED where some digits make signed pairs
+// (a separate copy for the others, which it would slow by 2-4%). All 128 threads of the block call (valid:
+// the warp has an item); sm: DIGIT_SHARED_U4 uint4 of shared memory.
+template <bool SIGNED>
 __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
                                             uint4* scratch, uint4* sm) {
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
@@ -1186,6 +1250,13 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     uint4* base = scratch + D.base;
     uint4* half = scratch + D.half;
     uint4* pref = scratch + D.pref;
+    uint4* high = half + ((size_t)128 << a.hl);
+    // Signed pairs of each half's first two digits, and of the only two.
+    const bool two = SIGNED && a.nd == 2 && signed_pair(a, 0, 2);
+    const bool sp[2] = {two || (SIGNED && signed_pair(a, 0, a.ns)), SIGNED && signed_pair(a, a.ns, a.nd)};
+    const int second[2] = {1, a.ns + 1};
+    auto lower = [&](int dg) { return (sp[0] && dg == 0) || (sp[1] && dg == a.ns); };
+    auto upper = [&](int dg) { return (sp[0] && dg == second[0]) || (sp[1] && dg == second[1]); };
     int E = valid ? P.nent[s] : 0;
     unsigned turn = blockIdx.x;
 
@@ -1228,11 +1299,25 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
 
     // 1. Place by place, the digits' multiples: entry v of a digit at bit o
     // of its half goes to half entry v 2^o (standard coordinates), and 2^4
-    // times its point (Montgomery domain) to the column's base.
+    // times its point (Montgomery domain) to the column's base. Of the lower
+    // digit of a signed pair 1..8 and 16 are made, of the upper one 1..2^bits.
     auto half_at = [&](int dg, int& o) -> uint4* {
         o = 0;
         for (int x = dg < a.ns ? 0 : a.ns; x < dg; x++) o += digit_bits(a, x);
-        return half + (dg < a.ns ? (size_t)0 : (size_t)128 << a.hl);
+        return dg < a.ns ? half : high;
+    };
+    // Steps of a digit's chain, and the row of its entry e.
+    auto chain_len = [&](int dg, bool more) -> int {
+        if (lower(dg)) return 9;
+        return (1 << digit_bits(a, dg)) - (more || upper(dg) ? 0 : 1);
+    };
+    auto spare = [&](int dg) -> uint4* { return dg < a.ns ? high : half; };
+    auto chain_row = [&](int dg, int t, int e, int len, bool more, uint4* hb, int o) -> uint4* {
+        if (e == len - 1) {
+            if (more) return base + (size_t)t * 128;
+            if (upper(dg)) return spare(dg);
+        }
+        return hb + ((size_t)(e + 1) << o) * 128;
     };
     uint32_t atinf = 0;          // columns (by t) whose point is infinity in this lane
     for (int place = 0; place < a.dpc; place++) {
@@ -1241,7 +1326,7 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
         fe acc;
         fe_one(acc);
         for (int t = 0; t < kw; t++) {
-            const int dg = t * a.dpc + place, len = (1 << digit_bits(a, dg)) - (more ? 0 : 1);
+            const int dg = t * a.dpc + place, len = chain_len(dg, more);
             aff B, S;
             if (place == 0) {
                 load_aff(S, Bc, nl, (size_t)(c0 + t) * a.l + jj);
@@ -1276,10 +1361,15 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             // ZZZ's factors to slot e.  The first step is a doubling.
 #pragma unroll 1
             for (int e = 1; e < len; e++) {
-                uint4* xy = (more && e == len - 1 ? base + (size_t)t * 128 : hb + ((size_t)(e + 1) << o) * 128) + lane;
+                uint4* xy = chain_row(dg, t, e, len, more, hb, o) + lane;
                 uint4* f = rt + (size_t)e * 128 + lane;
                 fe r2, r3;
-                jacz_madd_ratio_t<PCMM_DIGIT_INLINE>(P1, B, r2, r3, ok, false);
+                if (SIGNED && e == 8 && lower(dg)) {
+                    jacz_dbl_ratio(P1, r2, r3);
+                    if (fe_is_zero(P1.ZZ)) ok = false;
+                } else {
+                    jacz_madd_ratio_t<SIGNED ? PCMM_SIGNED_INLINE : PCMM_DIGIT_INLINE>(P1, B, r2, r3, ok, false);
+                }
                 xy[0] = fe_lo(P1.X);
                 xy[32] = fe_hi(P1.X);
                 xy[64] = fe_lo(P1.Y);
@@ -1314,7 +1404,7 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
         fe inv;
         fe_from_quads(inv, sm[tid], sm[128 + tid]);
         for (int t = kw - 1; t >= 0; t--) {
-            const int dg = t * a.dpc + place, len = (1 << digit_bits(a, dg)) - (more ? 0 : 1);
+            const int dg = t * a.dpc + place, len = chain_len(dg, more);
             if (len < 2) continue;
             const uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 128;
             aff zz;
@@ -1328,14 +1418,14 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             uint4* hb = half_at(dg, o);
             for (int e = len - 1; e >= 1; e--) {
                 const bool last = more && e == len - 1;
+                uint4* row = chain_row(dg, t, e, len, more, hb, o);
                 if (more ? e == len - 2 : e == len - 1) {
                     // From here on the products with X and Y are standard.
                     fe_from_mont(zi, zi);
                     fe_from_mont(zzi, zzi);
                 }
                 aff Q, r;
-                if (last) lp_load_aff(Q, base, t, lane);
-                else lp_load_aff(Q, hb, (e + 1) << o, lane);
+                lp_load_aff(Q, row, 0, lane);
                 Q.x = fmul(Q.x, zi);
                 Q.y = fmul(Q.y, zzi);
                 if (failed) {
@@ -1343,20 +1433,25 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
                         aff B;
                         lp_load_aff(B, hb, 1 << o, lane);
                         aff_to_mont(B);
-                        Q = small_multiple(B, (uint32_t)(e + 1));
+                        Q = small_multiple(B, last ? 16u : (uint32_t)(e + 1));
                         if (!last) aff_from_mont(Q);
                     }
                 }
                 if (last) {
-                    lp_store_aff(base, t, lane, Q);
-                } else {
+                    lp_store_aff(row, 0, lane, Q);
+                    if (upper(dg)) {
+                        aff_from_mont(Q);
+                        row = spare(dg);
+                    }
+                }
+                if (!last || upper(dg)) {
                     fe_canon(Q.x, Q.x);
                     fe_canon(Q.y, Q.y);
                     if ((atinf >> t) & 1u) {
                         fe_zero(Q.x);
                         fe_zero(Q.y);
                     }
-                    lp_store_aff(hb, (e + 1) << o, lane, Q);
+                    lp_store_aff(row, 0, lane, Q);
                 }
                 lp_load_aff(r, rt, e, lane);
                 zi = fmul(zi, r.x);
@@ -1369,42 +1464,53 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     const int nlow = a.ns, nhigh = a.nd - a.ns;
     for (int r = 1; r < nlow || r < nhigh; r++) {
         // Low half: digit r at bit oL; high half: digit ns + r at bit oH.
-        // Pair index i of a half: (v - 1) 2^o + g.
+        // Pair index i of a half: (v - 1) 2^o + g; (v - 1) 8 + (g - 1) of
+        // signed pairs.
         int o[2] = {0, 0}, n[2] = {0, 0};
 #pragma unroll
         for (int hf = 0; hf < 2; hf++) {
             const int dg = hf ? a.ns + r : r;
             if (r < (hf ? nhigh : nlow) && dg / a.dpc < kw) {
                 half_at(dg, o[hf]);
-                n[hf] = ((1 << digit_bits(a, dg)) - 1) << o[hf];
+                n[hf] = r == 1 && sp[hf] ? 8 << digit_bits(a, dg) : ((1 << digit_bits(a, dg)) - 1) << o[hf];
             }
         }
-        auto pick = [&](int i, int& g, int& v, uint4*& tab) -> bool {
+        auto pick = [&](int i, int& g, int& v, uint4*& tab, const uint4*& pa) -> unsigned {
             const int hf = i >= n[0];
+            const int cnt = hf ? n[1] : n[0];
             if (hf) i -= n[0];
-            tab = half + (hf ? (size_t)128 << a.hl : (size_t)0);
+            tab = hf ? high : half;
+            if (r == 1 && (hf ? sp[1] : sp[0])) {
+                const int top = cnt >> 3;
+                g = (i & 7) + 1;
+                v = (i >> 3) + 1;
+                pa = v == top ? (hf ? half : high) : tab + (size_t)v * (16 * 128);
+                const unsigned want = (v < top ? 1u : 0u) | (g < 8 ? 2u : 0u);
+                v *= 16;
+                return want;
+            }
             const int ob = hf ? o[1] : o[0];
             g = i & ((1 << ob) - 1);
             v = ((i >> ob) + 1) << ob;
+            pa = tab + (size_t)v * 128;
             return g != 0;
         };
-        affine_batch(
-            n[0] + n[1],
-            [&](int i, const uint4*& pa, const uint4*& pb) -> bool {
-                int g, v;
-                uint4* tab;
-                if (!pick(i, g, v, tab)) return false;
-                pa = tab + (size_t)g * 128 + lane;
-                pb = tab + (size_t)v * 128 + lane;
-                return true;
-            },
-            [&](int i, const aff& S) {
-                int g, v;
-                uint4* tab;
-                pick(i, g, v, tab);
-                lp_store_aff(tab, v + g, lane, S);
-            },
-            pref, sm, turn++);
+        auto pair = [&](int i, const uint4*& pa, const uint4*& pb) -> unsigned {
+            int g, v;
+            uint4* tab;
+            const unsigned want = pick(i, g, v, tab, pa);
+            pa += lane;
+            pb = tab + (size_t)g * 128 + lane;
+            return want;
+        };
+        auto put = [&](int i, int minus, const aff& S) {
+            int g, v;
+            uint4* tab;
+            const uint4* pa;
+            pick(i, g, v, tab, pa);
+            lp_store_aff(tab, minus ? v - g : v + g, lane, S);
+        };
+        affine_batch<SIGNED>(n[0] + n[1], pair, put, pref, sm, turn++);
     }
 
     // 3. The strip's entries.
@@ -1413,21 +1519,57 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
         store_aff(a.table, a.table_points, ((tbase + e) * 2 + c) * a.lp + j, q);
     };
     const uint32_t lmask = (1u << a.hl) - 1u;
-    const uint4* high = half + ((size_t)128 << a.hl);
-    if (a.nd > 1) affine_batch(
-        E,
-        [&](int e, const uint4*& pa, const uint4*& pb) -> bool {
-            const uint32_t code = codes[e];
-            pa = half + (size_t)(code & lmask) * 128 + lane;
-            pb = high + (size_t)(code >> a.hl) * 128 + lane;
-            return (code & lmask) && (code >> a.hl);
-        },
-        store_table, pref, sm, turn);
+    if (two) {
+        // The entry of each code, then the pairs that hold one: v, g and the
+        // entries of 16 v + g and 16 v - g (255: none).
+        uint8_t* rank = (uint8_t*)(sm + 256 + warp * 48);
+        uint32_t* list = (uint32_t*)(rank + 256);
+        ((uint2*)rank)[lane] = make_uint2(0xffffffffu, 0xffffffffu);
+        __syncwarp();
+        for (int e = lane; e < E; e += 32) rank[codes[e] & 255] = (uint8_t)e;
+        __syncwarp();
+        const int top = 1 << a.hh;
+        int cnt = 0;
+        for (int b = 0; b < top * 8; b += 32) {
+            const int i = b + (int)lane, v = (i >> 3) + 1, g = (i & 7) + 1;
+            const uint32_t plus = v < top ? rank[(16 * v + g) & 255] : 255u;
+            const uint32_t minus = g < 8 ? rank[(16 * v - g) & 255] : 255u;
+            const bool any = (plus & minus) != 255u;
+            const unsigned mask = __ballot_sync(0xffffffffu, any);
+            if (any) list[cnt + __popc(mask & ((1u << lane) - 1u))] = (uint32_t)v | (uint32_t)g << 8 | plus << 16 | minus << 24;
+            cnt += __popc(mask);
+        }
+        __syncwarp();
+        affine_batch<true>(
+            cnt,
+            [&](int i, const uint4*& pa, const uint4*& pb) -> unsigned {
+                const uint32_t x = list[i];
+                const int v = x & 255;
+                pa = (v == top ? half : high + (size_t)v * 128) + lane;
+                pb = half + (size_t)((x >> 8) & 255u) * 128 + lane;
+                return (((x >> 16) & 255u) != 255u ? 1u : 0u) | ((x >> 24) != 255u ? 2u : 0u);
+            },
+            [&](int i, int minus, const aff& S) {
+                store_table((int)(minus ? list[i] >> 24 : (list[i] >> 16) & 255u), S);
+            },
+            pref, sm, turn);
+    } else if (a.nd > 1) {
+        affine_batch<false>(
+            E,
+            [&](int e, const uint4*& pa, const uint4*& pb) -> unsigned {
+                const uint32_t code = codes[e];
+                pa = half + (size_t)(code & lmask) * 128 + lane;
+                pb = high + (size_t)(code >> a.hl) * 128 + lane;
+                return (code & lmask) && (code >> a.hl);
+            },
+            [&](int e, int, const aff& S) { store_table(e, S); },
+            pref, sm, turn);
+    }
     for (int e = 0; e < E; e++) {
-        const uint32_t code = codes[e];
-        if ((code & lmask) && (code >> a.hl)) continue;
+        const uint32_t code = codes[e], u = code & lmask;
+        if (u && ((code >> a.hl) || (two && u > 8))) continue;
         aff Q;
-        lp_load_aff(Q, code & lmask ? half + (size_t)(code & lmask) * 128 : high + (size_t)(code >> a.hl) * 128, 0, lane);
+        lp_load_aff(Q, u ? half + (size_t)u * 128 : high + (size_t)(code >> a.hl) * 128, 0, lane);
         store_table(e, Q);
     }
 }
@@ -1456,6 +1598,8 @@ inline bool digit_split(const Layout& L, TableArgs& a) {
     // 5.38, with 256 rows 7.22 and 6.63; w = 16 with 256 rows (halves 512) 12.0
     // and 9.96, with 512 rows 18.2 and 12.8; w = 8 with 16 rows (halves 32) 1.17
     // and 1.11, with 128 rows 2.81 and 1.98; k = 5 at w = 1 0.54 and 0.19.
+    a.w = L.w;
+    a.sgn = (a.nd == 2 && signed_pair(a, 0, 2)) || signed_pair(a, 0, a.ns) || signed_pair(a, a.ns, a.nd);
     if (best > 2LL * L.emax) return false;
     return digit_scratch(L.w, L.k, a.dpc, a.hl, a.hh, L.n1max, L.l2max, L.emax).total <= L.item_u4;
 }

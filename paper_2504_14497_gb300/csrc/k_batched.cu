@@ -73,6 +73,14 @@ __global__ void __launch_bounds__(PLAN_THREADS) batched_plan_kernel(const Inst* 
     plan_strip(I.A, I.m, I.n, I.w, I.k, I.P, is.y);
 }
 
+// The digit build as a function of its own: inlined beside the gather it was
+// slower (twelve uneven products 50.2 against 48.9 ms), and with one copy for
+// signed pairs and one without as well (50.4).
+static __device__ __noinline__ void digit_item(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
+                                               uint4* scratch, uint4* sm) {
+    table_block<true>(a, P, item, valid, scratch, sm);
+}
+
 // Resident blocks per SM requested from the compiler: 4 (128 registers, some
 // spilled) measured 1256.9 ms for the 64-instance batch against 1497.9 ms
 // uncapped (168 registers, 3 blocks) and 1262.7 ms at 5 blocks.
@@ -89,7 +97,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
     uint4* my_scratch = scratch + (size_t)warp_id * scratch_u4;
     __shared__ long long sh_t;
     __shared__ int sh_seg, sh_go;
-    __shared__ uint4 sh_inv[256];
+    __shared__ uint4 sh_inv[DIGIT_SHARED_U4];
     for (;;) {
         // The block takes BLOCK_TASKS consecutive tasks of one segment (every
         // segment starts at a multiple of BLOCK_TASKS), one per warp.  Every
@@ -153,7 +161,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
                 ta.item_u4 = I.item_u4;
                 ta.table = tbuf;
                 ta.table_points = I.table_points;
-                if (I.digits) table_block(ta, I.P, item, real, my_scratch, sh_inv);
+                if (I.digits) digit_item(ta, I.P, item, real, my_scratch, sh_inv);
                 else if (real) table_item(ta, I.P, item, my_scratch);
             }
         } else if (real) {

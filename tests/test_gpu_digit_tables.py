@@ -64,3 +64,60 @@ def test_related_columns(w, k, m):
                 if (t + j) % 4 == 0:
                     ct[s + t, j] = ct[s, j]
     _same(_device_plain(pr["A"], w, dev), ct_from_aos(dev, ct), m, l, w, k)
+
+
+@pytest.mark.parametrize("w,k,m,n,l", [
+    (6, 1, 40, 3, 33), (6, 1, 300, 2, 1), (6, 2, 900, 3, 40), (7, 1, 20, 2, 32), (7, 2, 400, 3, 33), (8, 1, 17, 3, 33),
+    (8, 1, 120, 2, 64), (8, 1, 1500, 2, 32), (8, 2, 600, 5, 20), (10, 1, 300, 2, 33), (11, 1, 300, 3, 32),
+    (12, 1, 400, 2, 40), (14, 1, 300, 2, 32), (15, 1, 400, 2, 3), (16, 1, 900, 2, 40),
+])
+def test_signed_pairs(w, k, m, n, l):
+    # Values around the multiples of 16, where an entry is the sum or the
+    # difference of a pair, besides random ones.
+    dev = device()
+    pr = inputs.pcmm_problem(9300 + 100 * w + k, m, n, l, w)
+    A = pr["A"].copy()
+    near = (np.arange(m * n).reshape(m, n) * 16 + np.resize([0, 1, 7, 8, 9, 15], (m, n))) % (1 << w)
+    A[::2] = near[::2]
+    _same(_device_plain(A, w, dev), encrypt_gpu(dev, pr), m, l, w, k)
+
+
+def _small_order():
+    """Points of orders 2, 3 and 4, each on the curve y^2 = x^3 - 3 x + b' of
+    its own b', on which the same formulas add."""
+    root = lambda a: pow(a, (P + 1) // 4, P)
+    square = lambda a: a and pow(a, (P - 1) // 2, P) == 1
+    pts = [(5, 0)]
+    x = 2
+    while True:          # 3 x^4 - 18 x^2 + 12 b x - 9 = 0: order 3
+        b = (9 - 3 * x**4 + 18 * x * x) * pow(12 * x, -1, P) % P
+        y2 = (x**3 - 3 * x + b) % P
+        if square(y2):
+            pts.append((x, root(y2)))
+            break
+        x += 1
+    x2 = 2
+    while True:          # twice the point is (x2, 0): (x - x2)^2 = 3 x2^2 - 3
+        b = (3 * x2 - x2**3) % P
+        if square((3 * x2 * x2 - 3) % P):
+            x = (x2 + root((3 * x2 * x2 - 3) % P)) % P
+            y2 = (x**3 - 3 * x + b) % P
+            if square(y2):
+                pts.append((x, root(y2)))
+                break
+        x2 += 1
+    return pts
+
+
+@pytest.mark.parametrize("w", [4, 6, 8, 12, 16])
+def test_points_of_small_order_keep_to_their_lane(w):
+    # Such a column is no ciphertext; its neighbours in the shared inversion are.
+    dev = device()
+    m, l = 300, 34
+    pr = inputs.pcmm_problem(9700 + w, m, 1, l, w)
+    ct = oracle.encrypt(oracle.keygen(pr["sk"]), pr["B"], pr["r"]).copy()
+    for i, (x, y) in enumerate(_small_order()):
+        for j in (i, 20 + i):
+            ct[0, j, j % 2, :8] = oracle.int_to_words(x)
+            ct[0, j, j % 2, 8:] = oracle.int_to_words(y)
+    _same(_device_plain(pr["A"], w, dev), ct_from_aos(dev, ct), m, l, w, 1)
