@@ -35,6 +35,10 @@ constexpr int NLEV = PCMM_N_ITER;   // compression iterations N
 #ifndef PCMM_SIGNED_INLINE
 #define PCMM_SIGNED_INLINE 2
 #endif
+// Of two columns' digits (w = 4): 5.4, -, 5.3 and 5.4 ms.
+#ifndef PCMM_CROSS_INLINE
+#define PCMM_CROSS_INLINE 2
+#endif
 constexpr uint16_t NO_RANK = 0xFFFFu;
 constexpr int PLAN_THREADS = 256;
 
@@ -442,7 +446,7 @@ struct TableArgs {
     // Digit build (table_block): digits per column, digits of all columns,
     // digits of the low half and the bits of both halves.
     int dpc, nd, ns, hl, hh;
-    bool sgn;              // some of the digits make signed pairs (signed_pair)
+    int pairs;             // signed pairs: 0 none, 1 of one column's digits, 2 of two columns
 };
 
 __device__ __forceinline__ void lp_store_aff(uint4* base, int e, unsigned lane, const aff& Q) {
@@ -1146,24 +1150,46 @@ static __device__ __noinline__ aff small_multiple(const aff& B, uint32_t v) {
     return Q;
 }
 
+// 8 A + v B for a lane whose chain over two columns met infinity.
+static __device__ __noinline__ aff small_sum(const aff& A, const aff& B, uint32_t v) {
+    jac J, K;
+    jac_mul_small(J, A, 8u);
+    jac_mul_small(K, B, v);
+    jac_add(J, K);
+    aff Q;
+    if (jac_is_inf(J)) {
+        fe_zero(Q.x);
+        fe_zero(Q.y);
+        return Q;
+    }
+    fe zi;
+    fe_inv(zi, J.Z);
+    jac_to_aff_with_zinv(Q, J, zi);
+    return Q;
+}
+
 // Bits of digit d: four, or what is left of its column.
 __host__ __device__ inline int digit_bits(const TableArgs& a, int d) {
     const int r = a.w - 4 * (d % a.dpc);
     return r < 4 ? r : 4;
 }
 
-// Signed pairs: where a digit d and the next one d + 1 belong to one column and
-// come first in their half (or are the only two), an entry 16 v + u of theirs is
-// 16 v + u for u <= 8 and 16 (v + 1) - (16 - u) above, so that one factor of the
-// shared inversion serves two entries (affine_batch) and the multiples 9..15 of
-// the lower digit's point are not needed. It takes one more multiple of the
-// upper digit's, 2^bits, which waits in row 0 of the other half (no code 0 is
-// ever read). With one bit in the upper digit there is nothing to share. Table
-// times without and with signed pairs (ms): 1024 x 1024 x 256 at w = 8 12.6 and
-// 10.5, with one value in ten not zero 7.0 and 6.5; 512 x 512 x 256 at w = 16
-// 24.0 and 22.2.
+// Signed pairs: two digits d and d + 1 that come first in their half (or are
+// the only two), so that one factor of the shared inversion serves two of their
+// entries (affine_batch), and the multiples 9..15 of the lower digit's point are
+// not needed.
+//  - Digits of one column: an entry 16 v + u is 16 v + u for u <= 8 and
+//    16 (v + 1) - (16 - u) above. It takes one more multiple of the upper digit's
+//    point, 2^bits, which waits in row 0 of the other half (no code 0 is ever
+//    read). With one bit in the upper digit there is nothing to share.
+//  - Columns of four bits: v P1 + u P0 is (v P1 + 8 P0) + (u - 8) P0, and the
+//    upper digit's chain goes on from 8 P0 where the lower one's ends.
+// Table times without and with signed pairs (ms): 1024 x 1024 x 256 at w = 8 12.6
+// and 10.5, with one value in ten not zero 7.0 and 6.5, at w = 4 6.2 and 5.3; 512
+// x 512 x 256 at w = 16 24.0 and 22.2.
 __host__ __device__ inline bool signed_pair(const TableArgs& a, int d, int end) {
-    return d + 1 < end && d % a.dpc + 1 < a.dpc && digit_bits(a, d + 1) >= 2;
+    if (d + 1 >= end) return false;
+    return a.dpc == 1 ? a.w == 4 : d % a.dpc + 1 < a.dpc && digit_bits(a, d + 1) >= 2;
 }
 
 // Shared memory of the digit build, in uint4 per block: the shared inversion,
@@ -1228,12 +1254,16 @@ __device__ __forceinline__ const uint16_t* column_values(const PlanPtrs& P, int 
     return cur;
 }
 
-// Table of one warp item by digits, SIGNED where some digits make signed pairs
-// (a separate copy for the others, which it would slow by 2-4%). All 128 threads of the block call (valid:
+// Table of one warp item by digits; PAIRS: no signed pairs, pairs of one column's
+// digits or of two columns (a.pairs). One copy for all would slow each by 2-5%. All 128 threads of the block call (valid:
 // the warp has an item); sm: DIGIT_SHARED_U4 uint4 of shared memory.
-template <bool SIGNED>
+template <int PAIRS>
 __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
                                             uint4* scratch, uint4* sm) {
+    constexpr bool SIGNED = PAIRS != 0;
+    // Read rather than known from PAIRS: the compiler then made 5.3 ms (w = 4) of
+    // what took 5.5.
+    const bool cross = PAIRS == 2 && a.dpc == 1;   // of two columns
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
     const int s_local = valid ? (int)(item / (2 * a.njb)) : 0;
     const int rem = valid ? (int)(item % (2 * a.njb)) : 0;
@@ -1252,8 +1282,9 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     uint4* pref = scratch + D.pref;
     uint4* high = half + ((size_t)128 << a.hl);
     // Signed pairs of each half's first two digits, and of the only two.
-    const bool two = SIGNED && a.nd == 2 && signed_pair(a, 0, 2);
-    const bool sp[2] = {two || (SIGNED && signed_pair(a, 0, a.ns)), SIGNED && signed_pair(a, a.ns, a.nd)};
+    const bool pairs = SIGNED && (a.dpc == 1) == cross;
+    const bool two = pairs && a.nd == 2 && signed_pair(a, 0, 2);
+    const bool sp[2] = {two || (pairs && signed_pair(a, 0, a.ns)), pairs && signed_pair(a, a.ns, a.nd)};
     const int second[2] = {1, a.ns + 1};
     auto lower = [&](int dg) { return (sp[0] && dg == 0) || (sp[1] && dg == a.ns); };
     auto upper = [&](int dg) { return (sp[0] && dg == second[0]) || (sp[1] && dg == second[1]); };
@@ -1300,7 +1331,8 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     // 1. Place by place, the digits' multiples: entry v of a digit at bit o
     // of its half goes to half entry v 2^o (standard coordinates), and 2^4
     // times its point (Montgomery domain) to the column's base. Of the lower
-    // digit of a signed pair 1..8 and 16 are made, of the upper one 1..2^bits.
+    // digit of a signed pair 1..8 and 16 are made, of the upper one 1..2^bits;
+    // across two columns 1..8 and the sums 8 P0 + v P1, in one chain.
     auto half_at = [&](int dg, int& o) -> uint4* {
         o = 0;
         for (int x = dg < a.ns ? 0 : a.ns; x < dg; x++) o += digit_bits(a, x);
@@ -1308,11 +1340,12 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     };
     // Steps of a digit's chain, and the row of its entry e.
     auto chain_len = [&](int dg, bool more) -> int {
-        if (lower(dg)) return 9;
+        if (lower(dg)) return cross ? 8 : 9;
         return (1 << digit_bits(a, dg)) - (more || upper(dg) ? 0 : 1);
     };
     auto spare = [&](int dg) -> uint4* { return dg < a.ns ? high : half; };
     auto chain_row = [&](int dg, int t, int e, int len, bool more, uint4* hb, int o) -> uint4* {
+        if (cross && upper(dg)) return hb + (((size_t)e << o) + (two ? 0 : 8)) * 128;
         if (e == len - 1) {
             if (more) return base + (size_t)t * 128;
             if (upper(dg)) return spare(dg);
@@ -1325,6 +1358,8 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
         uint32_t failed = 0;     // columns whose chain met infinity in this lane
         fe acc;
         fe_one(acc);
+        jacz P1;
+        bool ok = true;
         for (int t = 0; t < kw; t++) {
             const int dg = t * a.dpc + place, len = chain_len(dg, more);
             aff B, S;
@@ -1350,12 +1385,14 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             uint4* hb = half_at(dg, o);
             lp_store_aff(hb, 1 << o, lane, S);
             if (len < 2) continue;
-            jacz P1;
-            P1.X = B.x;
-            P1.Y = B.y;
-            fe_one(P1.ZZ);
-            fe_one(P1.ZZZ);
-            bool ok = true;
+            const bool goes_on = cross && upper(dg);
+            if (!goes_on) {
+                P1.X = B.x;
+                P1.Y = B.y;
+                fe_one(P1.ZZ);
+                fe_one(P1.ZZZ);
+                ok = true;
+            }
             uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 128;
             // Entry e is (e + 1) times the point: X and Y to its place, ZZ's and
             // ZZZ's factors to slot e.  The first step is a doubling.
@@ -1368,7 +1405,16 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
                     jacz_dbl_ratio(P1, r2, r3);
                     if (fe_is_zero(P1.ZZ)) ok = false;
                 } else {
-                    jacz_madd_ratio_t<SIGNED ? PCMM_SIGNED_INLINE : PCMM_DIGIT_INLINE>(P1, B, r2, r3, ok, false);
+                    jacz_madd_ratio_t<PAIRS == 2 ? PCMM_CROSS_INLINE : PAIRS == 1 ? PCMM_SIGNED_INLINE : PCMM_DIGIT_INLINE>(P1, B, r2, r3, ok, false);
+                }
+                if (goes_on && e == 1 && ((atinf >> (t - 1)) & 1u)) {
+                    // Nothing to go on from: the upper column's own multiples.
+                    P1.X = B.x;
+                    P1.Y = B.y;
+                    fe_one(P1.ZZ);
+                    fe_one(P1.ZZZ);
+                    fe_one(r2);
+                    fe_one(r3);
                 }
                 xy[0] = fe_lo(P1.X);
                 xy[32] = fe_hi(P1.X);
@@ -1379,13 +1425,14 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
                 f[64] = fe_lo(r3);
                 f[96] = fe_hi(r3);
             }
+            if (cross && lower(dg) && t + 1 < kw) continue;
             // The chain's product ZZ ZZZ for the shared inversion; ZZ and ZZZ
             // wait in slot 0, whose factors would be 1.
             aff zz;
             zz.x = P1.ZZ;
             zz.y = P1.ZZZ;
             if (!ok) {
-                failed |= 1u << t;
+                failed |= (goes_on ? 3u << (t - 1) : 1u << t);
                 fe_one(zz.x);
                 fe_one(zz.y);
             }
@@ -1403,23 +1450,28 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
         __syncthreads();
         fe inv;
         fe_from_quads(inv, sm[tid], sm[128 + tid]);
+        fe zi, zzi;                             // ZZ^-1 and ZZZ^-1 of the entry
         for (int t = kw - 1; t >= 0; t--) {
             const int dg = t * a.dpc + place, len = chain_len(dg, more);
             if (len < 2) continue;
             const uint4* rt = rat + (size_t)t * (size_t)(1 << (a.w < 4 ? a.w : 4)) * 128;
-            aff zz;
-            fe pr;
-            lp_load_aff(zz, rt, 0, lane);
-            lp_load_fe(pr, pref, t, lane);
-            const fe i5 = fmul(inv, pr);
-            inv = fmul(inv, fmul(zz.x, zz.y));
-            fe zi = fmul(i5, zz.y), zzi = fmul(i5, zz.x);   // ZZ^-1 and ZZZ^-1 of the last entry
+            const bool began = cross && lower(dg) && t + 1 < kw;   // the upper digit went on from here
+            if (!began) {
+                aff zz;
+                fe pr;
+                lp_load_aff(zz, rt, 0, lane);
+                lp_load_fe(pr, pref, t, lane);
+                const fe i5 = fmul(inv, pr);
+                inv = fmul(inv, fmul(zz.x, zz.y));
+                zi = fmul(i5, zz.y);
+                zzi = fmul(i5, zz.x);
+            }
             int o;
             uint4* hb = half_at(dg, o);
             for (int e = len - 1; e >= 1; e--) {
                 const bool last = more && e == len - 1;
                 uint4* row = chain_row(dg, t, e, len, more, hb, o);
-                if (more ? e == len - 2 : e == len - 1) {
+                if (!began && (more ? e == len - 2 : e == len - 1)) {
                     // From here on the products with X and Y are standard.
                     fe_from_mont(zi, zi);
                     fe_from_mont(zzi, zzi);
@@ -1433,7 +1485,18 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
                         aff B;
                         lp_load_aff(B, hb, 1 << o, lane);
                         aff_to_mont(B);
-                        Q = small_multiple(B, last ? 16u : (uint32_t)(e + 1));
+                        if (cross && upper(dg)) {
+                            aff A;
+                            int ol;
+                            uint4* lb = half_at(dg - 1, ol);
+                            lp_load_aff(A, lb, 1 << ol, lane);
+                            aff_to_mont(A);
+                            load_aff(B, Bc, nl, (size_t)(c0 + t) * a.l + jj);
+                            aff_to_mont(B);
+                            Q = small_sum(A, B, (uint32_t)e);
+                        } else {
+                            Q = small_multiple(B, last ? 16u : (uint32_t)(e + 1));
+                        }
                         if (!last) aff_from_mont(Q);
                     }
                 }
@@ -1457,6 +1520,14 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
                 zi = fmul(zi, r.x);
                 zzi = fmul(zzi, r.y);
             }
+            if (began && ((atinf >> (t + 1)) & 1u)) {
+                // v infinity + 8 P0.
+                aff Q;
+                lp_load_aff(Q, hb, 8 << o, lane);
+                int ou;
+                uint4* ub = half_at(dg + 1, ou);
+                for (int v = 1; v < 16; v++) lp_store_aff(chain_row(dg + 1, t + 1, v, 16, more, ub, ou), 0, lane, Q);
+            }
         }
     }
 
@@ -1465,7 +1536,8 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     for (int r = 1; r < nlow || r < nhigh; r++) {
         // Low half: digit r at bit oL; high half: digit ns + r at bit oH.
         // Pair index i of a half: (v - 1) 2^o + g; (v - 1) 8 + (g - 1) of
-        // signed pairs.
+        // signed pairs, v 8 + (g - 1) across two columns (of which the upper
+        // one may be missing: v = 0).
         int o[2] = {0, 0}, n[2] = {0, 0};
 #pragma unroll
         for (int hf = 0; hf < 2; hf++) {
@@ -1473,6 +1545,8 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             if (r < (hf ? nhigh : nlow) && dg / a.dpc < kw) {
                 half_at(dg, o[hf]);
                 n[hf] = r == 1 && sp[hf] ? 8 << digit_bits(a, dg) : ((1 << digit_bits(a, dg)) - 1) << o[hf];
+            } else if (cross && r == 1 && sp[hf] && dg - 1 < kw) {
+                n[hf] = 8;
             }
         }
         auto pick = [&](int i, int& g, int& v, uint4*& tab, const uint4*& pa) -> unsigned {
@@ -1483,6 +1557,11 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             if (r == 1 && (hf ? sp[1] : sp[0])) {
                 const int top = cnt >> 3;
                 g = (i & 7) + 1;
+                if (cross) {
+                    v = (i >> 3) * 16 + 8;
+                    pa = tab + (size_t)v * 128;
+                    return (g < 8 ? 1u : 0u) | (v > 8 ? 2u : 0u);
+                }
                 v = (i >> 3) + 1;
                 pa = v == top ? (hf ? half : high) : tab + (size_t)v * (16 * 128);
                 const unsigned want = (v < top ? 1u : 0u) | (g < 8 ? 2u : 0u);
@@ -1521,7 +1600,8 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     const uint32_t lmask = (1u << a.hl) - 1u;
     if (two) {
         // The entry of each code, then the pairs that hold one: v, g and the
-        // entries of 16 v + g and 16 v - g (255: none).
+        // entries of z + g and z - g (255: none), z = 16 v, or 16 v + 8 across two
+        // columns.
         uint8_t* rank = (uint8_t*)(sm + 256 + warp * 48);
         uint32_t* list = (uint32_t*)(rank + 256);
         ((uint2*)rank)[lane] = make_uint2(0xffffffffu, 0xffffffffu);
@@ -1531,9 +1611,10 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
         const int top = 1 << a.hh;
         int cnt = 0;
         for (int b = 0; b < top * 8; b += 32) {
-            const int i = b + (int)lane, v = (i >> 3) + 1, g = (i & 7) + 1;
-            const uint32_t plus = v < top ? rank[(16 * v + g) & 255] : 255u;
-            const uint32_t minus = g < 8 ? rank[(16 * v - g) & 255] : 255u;
+            const int i = b + (int)lane, v = (i >> 3) + (cross ? 0 : 1), g = (i & 7) + 1;
+            const int z = 16 * v + (cross ? 8 : 0);
+            const uint32_t plus = (cross ? g < 8 : v < top) ? rank[(z + g) & 255] : 255u;
+            const uint32_t minus = (cross ? v > 0 : g < 8) ? rank[(z - g) & 255] : 255u;
             const bool any = (plus & minus) != 255u;
             const unsigned mask = __ballot_sync(0xffffffffu, any);
             if (any) list[cnt + __popc(mask & ((1u << lane) - 1u))] = (uint32_t)v | (uint32_t)g << 8 | plus << 16 | minus << 24;
@@ -1545,7 +1626,7 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             [&](int i, const uint4*& pa, const uint4*& pb) -> unsigned {
                 const uint32_t x = list[i];
                 const int v = x & 255;
-                pa = (v == top ? half : high + (size_t)v * 128) + lane;
+                pa = (v == top ? half : cross && v == 0 ? half + 8 * 128 : high + (size_t)v * 128) + lane;
                 pb = half + (size_t)((x >> 8) & 255u) * 128 + lane;
                 return (((x >> 16) & 255u) != 255u ? 1u : 0u) | ((x >> 24) != 255u ? 2u : 0u);
             },
@@ -1567,9 +1648,9 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     }
     for (int e = 0; e < E; e++) {
         const uint32_t code = codes[e], u = code & lmask;
-        if (u && ((code >> a.hl) || (two && u > 8))) continue;
+        if (two && cross ? (code >> a.hl ? u != 8 : u > 8) : u && ((code >> a.hl) || (two && u > 8))) continue;
         aff Q;
-        lp_load_aff(Q, u ? half + (size_t)u * 128 : high + (size_t)(code >> a.hl) * 128, 0, lane);
+        lp_load_aff(Q, u && !(two && cross && (code >> a.hl)) ? half + (size_t)u * 128 : high + (size_t)(code >> a.hl) * 128, 0, lane);
         store_table(e, Q);
     }
 }
@@ -1599,7 +1680,8 @@ inline bool digit_split(const Layout& L, TableArgs& a) {
     // and 9.96, with 512 rows 18.2 and 12.8; w = 8 with 16 rows (halves 32) 1.17
     // and 1.11, with 128 rows 2.81 and 1.98; k = 5 at w = 1 0.54 and 0.19.
     a.w = L.w;
-    a.sgn = (a.nd == 2 && signed_pair(a, 0, 2)) || signed_pair(a, 0, a.ns) || signed_pair(a, a.ns, a.nd);
+    const bool any = (a.nd == 2 && signed_pair(a, 0, 2)) || signed_pair(a, 0, a.ns) || signed_pair(a, a.ns, a.nd);
+    a.pairs = !any ? 0 : a.dpc > 1 ? 1 : 2;
     if (best > 2LL * L.emax) return false;
     return digit_scratch(L.w, L.k, a.dpc, a.hl, a.hh, L.n1max, L.l2max, L.emax).total <= L.item_u4;
 }

@@ -83,13 +83,13 @@ __global__ void __launch_bounds__(128, PCMM_TABLE_MINBLOCKS) table_kernel(TableA
 #ifndef PCMM_DIGIT_MINBLOCKS
 #define PCMM_DIGIT_MINBLOCKS 4
 #endif
-template <bool SIGNED>
+template <int PAIRS>
 __global__ void __launch_bounds__(128, PCMM_DIGIT_MINBLOCKS) digit_table_kernel(TableArgs a, PlanPtrs P) {
     __shared__ uint4 sm[DIGIT_SHARED_U4];
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const bool valid = item < (long long)a.nstrips_chunk * 2 * a.njb;
     uint4* scratch = a.scratch + (valid ? (size_t)item : (size_t)0) * a.item_u4;
-    table_block<SIGNED>(a, P, item, valid, scratch, sm);
+    table_block<PAIRS>(a, P, item, valid, scratch, sm);
 }
 
 __global__ void __launch_bounds__(128, PCMM_GATHER_MINBLOCKS) gather_kernel(GatherArgs a, PlanPtrs P) {
@@ -294,9 +294,11 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         const long long items = (long long)sc * L.items_per_strip;
         {
             ProfScope ps(KID_TABLE, st);
-            if (digits && split.sgn) digit_table_kernel<true><<<(unsigned)((items + 3) / 4), 128, 0, st>>>(ta, P);
-            else if (digits) digit_table_kernel<false><<<(unsigned)((items + 3) / 4), 128, 0, st>>>(ta, P);
-            else table_kernel<<<(unsigned)((items + 3) / 4), 128, 0, st>>>(ta, P);
+            const unsigned blocks = (unsigned)((items + 3) / 4);
+            if (!digits) table_kernel<<<blocks, 128, 0, st>>>(ta, P);
+            else if (split.pairs == 0) digit_table_kernel<0><<<blocks, 128, 0, st>>>(ta, P);
+            else if (split.pairs == 1) digit_table_kernel<1><<<blocks, 128, 0, st>>>(ta, P);
+            else digit_table_kernel<2><<<blocks, 128, 0, st>>>(ta, P);
         }
         PCMM_CUDA_CHECK_LAUNCH();
         GatherArgs ga;

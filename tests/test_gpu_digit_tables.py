@@ -121,3 +121,54 @@ def test_points_of_small_order_keep_to_their_lane(w):
             ct[0, j, j % 2, :8] = oracle.int_to_words(x)
             ct[0, j, j % 2, 8:] = oracle.int_to_words(y)
     _same(_device_plain(pr["A"], w, dev), ct_from_aos(dev, ct), m, l, w, 1)
+
+
+def _add(p, q):
+    if p is None or q is None:
+        return p or q
+    if p[0] == q[0]:
+        if (p[1] + q[1]) % P == 0:
+            return None
+        s = (3 * p[0] * p[0] - 3) * pow(2 * p[1], -1, P) % P
+    else:
+        s = (q[1] - p[1]) * pow(q[0] - p[0], -1, P) % P
+    x = (s * s - p[0] - q[0]) % P
+    return x, (s * (p[0] - x) - p[1]) % P
+
+
+def _times(k, p):
+    if k < 0:
+        p, k = (p[0], (P - p[1]) % P), -k
+    r = None
+    while k:
+        if k & 1:
+            r = _add(r, p)
+        p, k = _add(p, p), k >> 1
+    return r
+
+
+@pytest.mark.parametrize("k,m,n,l", [(2, 300, 5, 33), (2, 20, 2, 70), (3, 600, 4, 34), (3, 900, 5, 20), (4, 700, 9, 33),
+                                     (4, 600, 6, 34)])
+def test_signed_pairs_of_two_columns(k, m, n, l):
+    # Beside random lanes, upper columns that are 0, 8, -8, -4, -2, -1, 1, 2 or 16
+    # times the lower one (8 P0 + v P1 doubles or cancels), and lower columns, and
+    # both, at infinity.
+    dev = device()
+    pr = inputs.pcmm_problem(9400 + 10 * k + m, m, n, l, 4)
+    ct = oracle.encrypt(oracle.keygen(pr["sk"]), pr["B"], pr["r"]).copy()
+    scale = [0, 8, -8, -4, -2, -1, 1, 2, 16]
+    for col in range(1, n):
+        for j in range(l):
+            kind = (3 * col + j) % 15
+            for c in range(2):
+                if kind < len(scale):
+                    base = ct[col - 1, j, c]
+                    q = None
+                    if base.any():
+                        q = _times(scale[kind], (oracle.words_to_int(base[:8]), oracle.words_to_int(base[8:])))
+                    ct[col, j, c, :8] = oracle.int_to_words(q[0]) if q else 0
+                    ct[col, j, c, 8:] = oracle.int_to_words(q[1]) if q else 0
+                if kind in (0, 10):
+                    ct[col - 1, j, c] = 0
+    _same(_device_plain(pr["A"], 4, dev), ct_from_aos(dev, ct), m, l, 4, k)
+    _same(_device_plain(pr["A"], 4, dev), encrypt_gpu(dev, pr), m, l, 4, k)
