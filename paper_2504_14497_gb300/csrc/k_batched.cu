@@ -50,7 +50,7 @@ struct Inst {
     size_t table_points;        // points per buffer (S strips)
     size_t item_u4;
     int m, n, l, w, k;
-    int nstrips, n1max, l2max, emax, lp, njb;
+    int nstrips, n1max, l2max, emax, lp, span, nq;
     int S, nchunks;
     int ctr_base;               // 2 counters per pass: tables done, gathers done
     int digits, dpc, nd, ns, hl, hh;   // table build by digits (digit_split)
@@ -120,10 +120,10 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
                 int* tdone = ctrs + I.ctr_base + 2 * sg.chunk;
                 const int sc = min(I.S, I.nstrips - sg.chunk * I.S);
                 if (sg.type == TASK_TABLE) {
-                    if (sg.chunk >= 2) go = wait_at_least(tdone - 4 + 1, I.m * 2 * I.njb, &hdr->status);
+                    if (sg.chunk >= 2) go = wait_at_least(tdone - 4 + 1, I.m * I.nq, &hdr->status);
                 } else {
-                    go = wait_at_least(tdone, sc * 2 * I.njb, &hdr->status);
-                    if (go && sg.chunk > 0) go = wait_at_least(tdone - 2 + 1, I.m * 2 * I.njb, &hdr->status);
+                    go = wait_at_least(tdone, sc * I.nq, &hdr->status);
+                    if (go && sg.chunk > 0) go = wait_at_least(tdone - 2 + 1, I.m * I.nq, &hdr->status);
                 }
             }
             sh_t = t0;
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
             // A strip's items come in multiples of BLOCK_TASKS exactly when
             // its item count is one; then the block's four items belong to one
             // strip, follow one plan and share each inversion.
-            const int ips = 2 * I.njb;
+            const int ips = I.nq;
             const bool shared = (ips % BLOCK_TASKS) == 0;
             {
                 TableArgs ta;
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
                 ta.ctB = I.ctB;
                 ta.bshare = shared;
                 ta.m = I.m; ta.n = I.n; ta.l = I.l; ta.w = I.w; ta.k = I.k;
-                ta.lp = I.lp; ta.njb = I.njb; ta.n1max = I.n1max; ta.l2max = I.l2max; ta.emax = I.emax;
+                ta.lp = I.lp; ta.span = I.span; ta.nq = I.nq; ta.n1max = I.n1max; ta.l2max = I.l2max; ta.emax = I.emax;
                 ta.s0 = s0; ta.nstrips_chunk = sc;
                 ta.scratch = my_scratch;
                 ta.item_u4 = I.item_u4;
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
             }
         } else if (real) {
             GatherArgs ga;
-            ga.m = I.m; ga.l = I.l; ga.lp = I.lp; ga.njb = I.njb; ga.emax = I.emax;
+            ga.m = I.m; ga.l = I.l; ga.lp = I.lp; ga.span = I.span; ga.nq = I.nq; ga.emax = I.emax;
             ga.parts = 1; ga.partial = nullptr;
             ga.s0 = s0; ga.nstrips_chunk = sc;
             ga.first = (sg.chunk == 0);
@@ -265,7 +265,7 @@ pcmm_status build_layout(const pcmm_problem* probs, int count, int max_strips, i
         ctr += 2 * I.nchunks;
         I.m = L.m; I.n = L.n; I.l = L.l; I.w = L.w; I.k = L.k;
         I.nstrips = L.nstrips; I.n1max = L.n1max; I.l2max = L.l2max; I.emax = L.emax;
-        I.lp = L.lp; I.njb = L.njb; I.item_u4 = L.item_u4;
+        I.lp = L.lp; I.span = lane_span(L.l); I.nq = lane_blocks(L.l); I.item_u4 = L.item_u4;
         TableArgs split;
         I.digits = digit_split(L, split);
         I.dpc = split.dpc; I.nd = split.nd; I.ns = split.ns; I.hl = split.hl; I.hh = split.hh;
@@ -294,7 +294,7 @@ pcmm_status build_layout(const pcmm_problem* probs, int count, int max_strips, i
                 sg.type = ph == 0 ? TASK_TABLE : TASK_GATHER;
                 sg.inst = i;
                 sg.chunk = r;
-                sg.count = ph == 0 ? sc * 2 * I.njb : I.m * 2 * I.njb;
+                sg.count = ph == 0 ? sc * I.nq : I.m * I.nq;
                 H.segs.push_back(sg);
                 // Segments start at multiples of BLOCK_TASKS: a block's tasks
                 // never straddle two segments (padding tasks do nothing).

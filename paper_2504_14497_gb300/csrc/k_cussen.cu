@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_kernel(const TA* __restrict
 
 __global__ void __launch_bounds__(128, PCMM_TABLE_MINBLOCKS) table_kernel(TableArgs a, PlanPtrs P) {
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nitems = (long long)a.nstrips_chunk * 2 * a.njb;
+    const long long nitems = (long long)a.nstrips_chunk * a.nq;
     if (item >= nitems) return;
     table_item(a, P, item, a.scratch + (size_t)item * a.item_u4);
 }
@@ -87,14 +87,14 @@ template <int PAIRS>
 __global__ void __launch_bounds__(128, PCMM_DIGIT_MINBLOCKS) digit_table_kernel(TableArgs a, PlanPtrs P) {
     __shared__ uint4 sm[DIGIT_SHARED_U4];
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const bool valid = item < (long long)a.nstrips_chunk * 2 * a.njb;
+    const bool valid = item < (long long)a.nstrips_chunk * a.nq;
     uint4* scratch = a.scratch + (valid ? (size_t)item : (size_t)0) * a.item_u4;
     table_block<PAIRS>(a, P, item, valid, scratch, sm);
 }
 
 __global__ void __launch_bounds__(128, PCMM_GATHER_MINBLOCKS) gather_kernel(GatherArgs a, PlanPtrs P) {
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= (long long)a.m * 2 * a.njb * a.parts) return;
+    if (gw >= (long long)a.m * a.nq * a.parts) return;
     gather_item<false>(a, P, gw);
 }
 
@@ -163,13 +163,11 @@ __global__ void __launch_bounds__(128) combine_tree_kernel(const uint4* __restri
 // 32 columns. At 512 x 1 x 16384 (w = 4) it takes 241 us, where gather_kernel at
 // its 128 registers keeps too few loads in flight (514 us).
 __global__ void __launch_bounds__(128) gather_copy_kernel(GatherArgs a, PlanPtrs P) {
-    const unsigned lane = threadIdx.x & 31u;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= (long long)a.m * 2 * a.njb) return;
-    const int i = (int)(gw % a.m), rem = (int)(gw / a.m);
-    const int c = rem / a.njb, jb = rem % a.njb;
-    const int j = jb * 32 + (int)lane;
-    if (j >= a.l) return;
+    if (gw >= (long long)a.m * a.nq) return;
+    const int i = (int)(gw % a.m);
+    int c, j;
+    if (!lane_chain((int)(gw / a.m), a.span, a.l, c, j)) return;
     const size_t ml = (size_t)a.m * a.l;
     aff T;
     fe_zero(T.x);
@@ -281,7 +279,7 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         TableArgs ta = split;
         ta.ctB = (const uint4*)ctB;
         ta.m = L.m; ta.n = L.n; ta.l = L.l; ta.w = L.w; ta.k = L.k;
-        ta.lp = L.lp; ta.njb = L.njb; ta.n1max = L.n1max; ta.l2max = L.l2max; ta.emax = L.emax;
+        ta.lp = L.lp; ta.span = lane_span(L.l); ta.nq = lane_blocks(L.l); ta.n1max = L.n1max; ta.l2max = L.l2max; ta.emax = L.emax;
         ta.s0 = s0; ta.nstrips_chunk = sc;
         ta.scratch = scratch;
         ta.item_u4 = L.item_u4;
@@ -290,8 +288,8 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         // Four consecutive items (one 128-thread block) belong to one strip
         // exactly when a strip has a multiple of 4 items; then every block is
         // full and its warps follow the same plan, and share inversions.
-        ta.bshare = (L.items_per_strip % 4) == 0;
-        const long long items = (long long)sc * L.items_per_strip;
+        ta.bshare = (ta.nq % 4) == 0;
+        const long long items = (long long)sc * ta.nq;
         {
             ProfScope ps(KID_TABLE, st);
             const unsigned blocks = (unsigned)((items + 3) / 4);
@@ -302,7 +300,7 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         }
         PCMM_CUDA_CHECK_LAUNCH();
         GatherArgs ga;
-        ga.m = L.m; ga.l = L.l; ga.lp = L.lp; ga.njb = L.njb; ga.emax = L.emax;
+        ga.m = L.m; ga.l = L.l; ga.lp = L.lp; ga.span = ta.span; ga.nq = ta.nq; ga.emax = L.emax;
         ga.s0 = s0; ga.nstrips_chunk = sc;
         ga.first = (s0 == 0);
         ga.table = table;
@@ -313,7 +311,7 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         pc = pc < 1 ? 1 : pc < parts ? pc : parts;
         ga.parts = pc;
         ga.partial = (uint4*)partial;
-        const long long warps = (long long)L.m * 2 * L.njb * pc;
+        const long long warps = (long long)L.m * ga.nq * pc;
         {
             ProfScope ps(KID_GATHER, st);
             if (ga.first && sc == 1) gather_copy_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(ga, P);

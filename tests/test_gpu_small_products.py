@@ -74,3 +74,27 @@ def test_infinity_beside_points(w, k, m, l):
     if w <= 8:
         for out in pcmm.cussen_batched([(A, ctB, l, w, k)] * 3):
             assert torch.equal(pcmm.normalize(out, m * l), want)
+
+
+@pytest.mark.parametrize("l", [1, 15, 16, 17, 31, 32, 33, 47, 48, 49, 63, 64, 65, 97])
+@pytest.mark.parametrize("m,n,w,k", [(60, 1, 4, 1), (9, 40, 4, 1), (300, 5, 8, 1), (40, 4, 12, 1), (300, 5, 4, 2),
+                                     (300, 9, 2, 4)])
+def test_columns_that_fill_no_block(m, n, w, k, l):
+    # Both components' chains in blocks of 32, packed where that saves one:
+    # copies, parts, tables by digits and by chains, several passes, batched.
+    pr = inputs.pcmm_problem(7600 + 100 * l + n, m, n, l, w)
+    if w > 8:
+        dev = device()
+        A = pcmm.plaintext16(pr["A"], dev)
+        ctB = encrypt_gpu(dev, pr)
+        want = pcmm.normalize(pcmm.schoolbook(A, ctB, l, w), m * l)
+        assert torch.equal(pcmm.normalize(pcmm.cussen(A, ctB, l, w, k=k), m * l), want)
+        return
+    _check(pr, m, n, l, w, k)
+    _check(pr, m, n, l, w, k, ws=pcmm.cussen_workspace_bytes_for(m, n, l, w, k, 2))
+    dev = device()
+    A = torch.from_numpy(pr["A"]).to(dev)
+    ctB = encrypt_gpu(dev, pr)
+    want = pcmm.normalize(pcmm.schoolbook(A, ctB, l, w), m * l)
+    for out in pcmm.cussen_batched([(A, ctB, l, w, k)] * 2):
+        assert torch.equal(pcmm.normalize(out, m * l), want)
