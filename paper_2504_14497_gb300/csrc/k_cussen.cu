@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_kernel(const TA* __restrict
     plan_strip(A, m, n, w, k, P, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(128, PCMM_TABLE_MINBLOCKS) table_kernel(TableArgs a, PlanPtrs P) {
+template <int BLOCKS>
+__global__ void __launch_bounds__(128, BLOCKS) table_kernel(TableArgs a, PlanPtrs P) {
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nitems = (long long)a.nstrips_chunk * a.nq;
     if (item >= nitems) return;
@@ -83,8 +84,14 @@ __global__ void __launch_bounds__(128, PCMM_TABLE_MINBLOCKS) table_kernel(TableA
 #ifndef PCMM_DIGIT_MINBLOCKS
 #define PCMM_DIGIT_MINBLOCKS 4
 #endif
-template <int PAIRS>
-__global__ void __launch_bounds__(128, PCMM_DIGIT_MINBLOCKS) digit_table_kernel(TableArgs a, PlanPtrs P) {
+// Up to two blocks per SM the tables are bound by the latency of one warp per
+// scheduler or two, and are built by copies of the kernels that the register file
+// holds twice per SM (no spills). Table of 10 x 128 x 1 (w = 4) 119 -> 104 us, 512 x
+// 1 x 16384 158 -> 141 us, by chains (10 x 160 x 15, w = 7) 243 -> 211 us; with up to four
+// blocks per SM the copies lose (256 x 784 x 64 1.01 -> 1.35 ms).
+constexpr unsigned FEW_BLOCKS = 2 * 152;
+template <int PAIRS, int BLOCKS>
+__global__ void __launch_bounds__(128, BLOCKS) digit_table_kernel(TableArgs a, PlanPtrs P) {
     __shared__ uint4 sm[DIGIT_SHARED_U4];
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const bool valid = item < (long long)a.nstrips_chunk * a.nq;
@@ -293,10 +300,19 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         {
             ProfScope ps(KID_TABLE, st);
             const unsigned blocks = (unsigned)((items + 3) / 4);
-            if (!digits) table_kernel<<<blocks, 128, 0, st>>>(ta, P);
-            else if (split.pairs == 0) digit_table_kernel<0><<<blocks, 128, 0, st>>>(ta, P);
-            else if (split.pairs == 1) digit_table_kernel<1><<<blocks, 128, 0, st>>>(ta, P);
-            else digit_table_kernel<2><<<blocks, 128, 0, st>>>(ta, P);
+            const int kind = digits ? 1 + split.pairs : 0;
+            auto* kernel = table_kernel<PCMM_TABLE_MINBLOCKS>;
+            if (blocks <= FEW_BLOCKS) {
+                if (kind == 0) kernel = table_kernel<1>;
+                else if (kind == 1) kernel = digit_table_kernel<0, 1>;
+                else if (kind == 2) kernel = digit_table_kernel<1, 1>;
+                else kernel = digit_table_kernel<2, 1>;
+            } else if (kind) {
+                if (kind == 1) kernel = digit_table_kernel<0, PCMM_DIGIT_MINBLOCKS>;
+                else if (kind == 2) kernel = digit_table_kernel<1, PCMM_DIGIT_MINBLOCKS>;
+                else kernel = digit_table_kernel<2, PCMM_DIGIT_MINBLOCKS>;
+            }
+            kernel<<<blocks, 128, 0, st>>>(ta, P);
         }
         PCMM_CUDA_CHECK_LAUNCH();
         GatherArgs ga;

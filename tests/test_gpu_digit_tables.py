@@ -82,6 +82,15 @@ def test_signed_pairs(w, k, m, n, l):
     _same(_device_plain(A, w, dev), encrypt_gpu(dev, pr), m, l, w, k)
 
 
+@pytest.mark.parametrize("w,k,m", [(8, 1, 20), (8, 1, 400), (4, 2, 40), (4, 1, 20), (2, 3, 70), (12, 1, 16), (16, 1, 300)])
+def test_many_blocks(w, k, m):
+    # More than two blocks per SM: the kernels with the smaller register share.
+    dev = device()
+    n, l = 125 * k, 160
+    pr = inputs.pcmm_problem(9500 + 10 * w + k, m, n, l, w)
+    _same(_device_plain(pr["A"], w, dev), encrypt_gpu(dev, pr), m, l, w, k)
+
+
 def _small_order():
     """Points of orders 2, 3 and 4, each on the curve y^2 = x^3 - 3 x + b' of
     its own b', on which the same formulas add."""
