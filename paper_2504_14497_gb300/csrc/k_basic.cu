@@ -132,52 +132,77 @@ __device__ __forceinline__ void block_normalize_jacz(aff out[E], const jacz P[E]
 }
 
 // Blocks per SM the register allocation must allow: 262144 encryptions took
-// 1.89, 1.88, 1.92 and 1.86 ms at 4, 5, 6 and 8 blocks.
+// 1.75, 1.89 and 1.87 ms at 4, 5 and 6 blocks with the addition inlined (1.84
+// with the multiplications called, 1.82 and 1.83 with everything called at 6 and 8).
 #ifndef PCMM_ENCRYPT_MINBLOCKS
-#define PCMM_ENCRYPT_MINBLOCKS 8
+#define PCMM_ENCRYPT_MINBLOCKS 4
 #endif
 
-// Enc(b) = (rG, rH + bG): 32 window lookups per base point, added into
-// (X, Y, Z^2, Z^3) accumulators (8M + 2S each, and the standard comb entries
-// need no conversion).
-__global__ void __launch_bounds__(128, PCMM_ENCRYPT_MINBLOCKS) encrypt_kernel(const uint4* __restrict__ gtab,
-                                                      const uint4* __restrict__ htab,
-                                                      const uint8_t* __restrict__ msg,
-                                                      const uint4* __restrict__ r, size_t count,
-                                                      uint4* __restrict__ ct) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Enc(b) = (rG, rH + bG): 32 window lookups per base point, added into an
+// (X, Y, Z^2, Z^3) accumulator (8M + 2S each, and the standard comb entries
+// need no conversion). G threads (a power of two) take one component
+// (blockIdx.y) of a ciphertext, every G-th window each, and add their sums as a
+// tree.
+template <int G, int INL, int BLOCKS>
+__global__ void __launch_bounds__(128, BLOCKS) encrypt_kernel(const uint4* __restrict__ gtab,
+                                                              const uint4* __restrict__ htab,
+                                                              const uint8_t* __restrict__ msg,
+                                                              const uint4* __restrict__ r, size_t count,
+                                                              uint4* __restrict__ ct) {
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t i = t / G;
+    const int part = (int)(t % G), c = blockIdx.y;
     const bool valid = i < count;
     const size_t ii = valid ? i : 0;
-    fe rr;
-    fe_from_quads(rr, r[ii], r[count + ii]);
-    jacz P[2];
+    const uint4* tab = c ? htab : gtab;
+    jacz P[1];
     jacz_set_inf(P[0]);
-    jacz_set_inf(P[1]);
     aff T;
-    for (int win = 0; win < COMB_WINDOWS; win++) {
-        const uint32_t v = (rr.v[win >> 2] >> (8 * (win & 3))) & 0xffu;
+#pragma unroll 1
+    for (int win = part; win < COMB_WINDOWS; win += G) {
+        const uint32_t word = ((const uint32_t*)(r + (size_t)(win >> 4) * count + ii))[(win >> 2) & 3];
+        const uint32_t v = (word >> (8 * (win & 3))) & 0xffu;
         if (v) {
-            load_aff(T, gtab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
-            jacz_madd_t<0, true>(P[0], T);
-            load_aff(T, htab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
-            jacz_madd_t<0, true>(P[1], T);
+            load_aff(T, tab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
+            jacz_madd_t<INL, true>(P[0], T);
         }
     }
-    const uint32_t b = msg[ii];
+    const uint32_t b = c && part == G - 1 ? msg[ii] : 0u;
     if (b) {
         load_aff(T, gtab, COMB_POINTS, b);
-        jacz_madd_t<0, true>(P[1], T);
+        jacz_madd_t<0, true>(P[0], T);
     }
-    aff out[2];
-    block_normalize_jacz<2>(out, P);
-    if (valid) {
-        store_aff(ct, count, i, out[0]);
-        store_aff(ct + 4 * count, count, i, out[1]);
+    if (G > 1) {
+        __syncwarp();
+        jac S;
+        jacz_drop_R(P[0]);
+        jac_from_jacz(S, P[0]);
+        for (int d = G / 2; d >= 1; d >>= 1) {
+            jac Q;
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                Q.X.v[k] = __shfl_down_sync(0xffffffffu, S.X.v[k], d);
+                Q.Y.v[k] = __shfl_down_sync(0xffffffffu, S.Y.v[k], d);
+                Q.Z.v[k] = __shfl_down_sync(0xffffffffu, S.Z.v[k], d);
+            }
+            if (part < d) jac_add(S, Q);
+            __syncwarp();
+        }
+        if (part == 0) {
+            jacz_from_jac(P[0], S);
+            jacz_add_R(P[0]);
+        } else {
+            jacz_set_inf(P[0]);
+        }
+        __syncwarp();
     }
+    aff out[1];
+    block_normalize_jacz<1>(out, P);
+    if (valid && part == 0) store_aff(ct + (size_t)c * 4 * count, count, i, out[0]);
 }
 
 // s G for count scalars (key generation: H = x G), one thread per scalar.
-__global__ void __launch_bounds__(128, PCMM_ENCRYPT_MINBLOCKS) base_mul_kernel(const uint4* __restrict__ gtab,
+__global__ void __launch_bounds__(128, 8) base_mul_kernel(const uint4* __restrict__ gtab,
                                                        const uint4* __restrict__ sc, size_t count,
                                                        uint4* __restrict__ out) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -469,8 +494,16 @@ static pcmm_status launch_encrypt(const void* keytable, const uint8_t* msg, cons
     uint4* gtab = nullptr;
     if (cudaGetSymbolAddress((void**)&gtab, g_comb_G) != cudaSuccess) return PCMM_ECUDA;
     ProfScope ps(KID_ENCRYPT, st);
-    encrypt_kernel<<<grid_for(count, 128), 128, 0, st>>>(gtab, (const uint4*)keytable, msg, (const uint4*)r,
-                                                         count, (uint4*)ct);
+    // One thread a component from three warps per scheduler on; below, the
+    // windows' serial additions are the time, and threads up to one or two warps
+    // per scheduler share them. Time (us) with both components in one thread, and
+    // with 1, 2 and 8 threads each: 1 ciphertext 282 / -, 78, 57; 1000 282 / -, 82,
+    // 60; 4000 284 / 119, 83, 139; 10000 285 / 163, 145, 270; 30000 389 / 280, 332, -.
+    const int G = count <= 1216 ? 8 : count <= 9728 ? 2 : 1;
+    auto* kernel = G == 8 ? encrypt_kernel<8, 31, 2> : G == 2 ? encrypt_kernel<2, 31, 2>
+                                                              : encrypt_kernel<1, 31, PCMM_ENCRYPT_MINBLOCKS>;
+    kernel<<<dim3(grid_for(count * G, 128), 2), 128, 0, st>>>(gtab, (const uint4*)keytable, msg, (const uint4*)r,
+                                                              count, (uint4*)ct);
     PCMM_CUDA_CHECK_LAUNCH();
     return PCMM_OK;
 }
