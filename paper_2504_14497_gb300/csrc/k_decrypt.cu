@@ -181,14 +181,18 @@ static __device__ __noinline__ void giant_step(aff& M, const aff& Q) {
 // Blocks per SM the register allocation must allow (the scalar
 // multiplication is a serial chain per thread: occupancy hides its latency).
 // What the doublings inline (jac_dbl_t): 65536 decryptions took 2.54, 2.49, 2.52,
-// 2.48, 2.45, 2.51 and 2.48 ms at 0, 1, 2, 3, 4, 5 and 7.
+// 2.48, 2.45, 2.51 and 2.48 ms at 0, 1, 2, 3, 4, 5 and 7. Up to three blocks per
+// SM everything inlined is faster, the more so the fewer warps hide a chain's
+// latency: 72 take 0.92 ms at 4 and 0.85 at 7, 40000 1.72 and 1.66.
 #ifndef PCMM_DECRYPT_INLINE
 #define PCMM_DECRYPT_INLINE 4
 #endif
+constexpr size_t DECRYPT_FEW = 3 * 152 * 128;
 #ifndef PCMM_DECRYPT_MINBLOCKS
 #define PCMM_DECRYPT_MINBLOCKS 4
 #endif
 
+template <int INL>
 __global__ void __launch_bounds__(128, PCMM_DECRYPT_MINBLOCKS) decrypt_kernel(
         const uint4* __restrict__ gtab, Naf naf, const uint4* __restrict__ ct, size_t count, long long mmax,
         uint32_t s, uint32_t mask, const unsigned long long* __restrict__ slots, long long* __restrict__ out) {
@@ -203,7 +207,7 @@ __global__ void __launch_bounds__(128, PCMM_DECRYPT_MINBLOCKS) decrypt_kernel(
     jac R;
     jac_set_inf(R);
     for (int b = naf.len - 1; b >= 0; b--) {
-        jac_dbl_t<PCMM_DECRYPT_INLINE>(R);
+        jac_dbl_t<INL>(R);
         const int d = naf.d[b];
         if (d) {
             aff T = odd[(d < 0 ? -d : d) >> 1];
@@ -340,7 +344,8 @@ extern "C" pcmm_status pcmm_decrypt(const uint32_t* sk_host, const uint32_t* ct,
     Naf naf;
     naf4(sk_host, naf);
     ProfScope ps(KID_DECRYPT, (cudaStream_t)stream);
-    decrypt_kernel<<<grid_for(count, 128), 128, 0, (cudaStream_t)stream>>>(
+    auto* kernel = count <= DECRYPT_FEW ? decrypt_kernel<7> : decrypt_kernel<PCMM_DECRYPT_INLINE>;
+    kernel<<<grid_for(count, 128), 128, 0, (cudaStream_t)stream>>>(
         gtab, naf, (const uint4*)ct, count, (long long)mmax, baby, slot_count(baby) - 1,
         (const unsigned long long*)table, (long long*)out);
     PCMM_CUDA_CHECK_LAUNCH();

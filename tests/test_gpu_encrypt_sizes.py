@@ -53,3 +53,16 @@ def test_empty_windows(pad):
     assert not got[0].any()          # nonce 0, message 0 (the oracle refuses this nonce): infinity twice
     want = oracle.encrypt(oracle.keygen(sk), msg[1:k].reshape(1, k - 1), r[1:k].reshape(1, k - 1, 8))
     assert (got[1:k] == want.reshape(k - 1, 2, 16)).all()
+
+
+@pytest.mark.parametrize("count", [58368, 58369])
+def test_decryption_where_its_kernel_changes(count):
+    dev = device()
+    rng = np.random.default_rng(count)
+    r = rng.integers(0, 2**32, size=(count, 8), dtype=np.uint64).astype(np.uint32)
+    r[:, 7] >>= 1
+    msg = rng.integers(0, 256, size=count, dtype=np.uint8)
+    sk, H = _key()
+    steps = pcmm.BabySteps.for_range(255, device=dev)
+    out = pcmm.decrypt(sk, _encrypt(dev, H, msg, r), count, 255, steps)
+    assert (out.cpu().numpy() == msg.astype(np.int64)).all()
