@@ -1691,17 +1691,16 @@ inline bool digit_split(const Layout& L, TableArgs& a) {
         const long long size = (1LL << lo) + (1LL << hi);
         if (best < 0 || size < best) { best = size; a.ns = x; a.hl = lo; a.hh = hi; }
     }
-    // The halves must not outweigh the entries (with one digit, its multiples
-    // are the entries: 10 x 128 x 1 at w = 4 takes 135 us by chains and 118 us by
-    // digits).  Table times (ms) by chains and
-    // by digits, 256 x 256 columns: w = 12 with 128 rows (halves 272) 4.90 and
-    // 5.38, with 256 rows 7.22 and 6.63; w = 16 with 256 rows (halves 512) 12.0
-    // and 9.96, with 512 rows 18.2 and 12.8; w = 8 with 16 rows (halves 32) 1.17
-    // and 1.11, with 128 rows 2.81 and 1.98; k = 5 at w = 1 0.54 and 0.19.
+    // The digit build takes every layout whose scratch holds its halves: up to
+    // about 3.5 half entries for each entry of the strip. Table times (ms) by chains
+    // and by digits, 256 columns of 256: w = 16 with 160 rows (halves 512) 8.99 and
+    // 7.46, w = 12 with 128 rows (halves 272) 4.90 and 4.64, with 96 rows 4.21 and
+    // 4.34; 200 x 64 at w = 14 with 100 rows (halves 320) 1.81 and 1.55; 256 x 64 at w
+    // = 8 with 12 rows (halves 32) 0.332 and 0.289; one digit, 128 x 1 at w = 4 with
+    // 10 rows 135 and 118 us.
     a.w = L.w;
     const bool any = (a.nd == 2 && signed_pair(a, 0, 2)) || signed_pair(a, 0, a.ns) || signed_pair(a, a.ns, a.nd);
     a.pairs = !any ? 0 : a.dpc > 1 ? 1 : 2;
-    if (best > 2LL * L.emax) return false;
     return digit_scratch(L.w, L.k, a.dpc, a.hl, a.hh, L.n1max, L.l2max, L.emax).total <= L.item_u4;
 }
 
