@@ -26,8 +26,8 @@ constexpr int NLEV = PCMM_N_ITER;   // compression iterations N
 #ifndef PCMM_TABLE_INLINE
 #define PCMM_TABLE_INLINE 0
 #endif
-// The same for the digit build's chains: table of 1024 x 1024 x 256 at w = 8 12.6,
-// 12.7, 12.6 and 12.3 ms at 0, 1, 2 and 3.
+// The same for the digit build's chains: table of 1024 x 1024 x 256 at w = 8 (without
+// signed pairs) 12.6, 12.7, 12.6 and 12.3 ms at 0, 1, 2 and 3.
 #ifndef PCMM_DIGIT_INLINE
 #define PCMM_DIGIT_INLINE 3
 #endif
@@ -1275,8 +1275,9 @@ __device__ __forceinline__ const uint16_t* column_values(const PlanPtrs& P, int 
 }
 
 // Table of one warp item by digits; PAIRS: no signed pairs, pairs of one column's
-// digits or of two columns (a.pairs). One copy for all would slow each by 2-5%. All 128 threads of the block call (valid:
-// the warp has an item); sm: DIGIT_SHARED_U4 uint4 of shared memory.
+// digits or of two columns (a.pairs). One copy for all would slow each by 2-5%.
+// All 128 threads of the block call (valid: the warp has an item); sm:
+// DIGIT_SHARED_U4 uint4 of shared memory.
 template <int PAIRS>
 __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
                                             uint4* scratch, uint4* sm) {

@@ -11,7 +11,7 @@
 //         dropped from every level.  For the strip: the code of every row
 //         (its k entries packed w bits apiece), the sorted list of distinct
 //         non-zero codes, and each row's rank in that list (0xFFFF for 0).
-//  table  (one warp per strip, ciphertext component and 32 output columns)
+//  table  (one warp per strip and 32 ciphertext chains, lane_span)
 //         Level N: the compressed values times the ciphertext point B_c^(kj)
 //         by double-and-add (the ECSMs of Algorithm 3).  Levels N-1..1: each
 //         element of level w is the entry of level w + 1 its tracking pointer
@@ -26,11 +26,11 @@
 //         level-1 chains by walking Z^-2 and Z^-3 back along the factors the
 //         chain multiplied them by; the inversion is shared by the lanes of
 //         a warp and, when the block's four warps follow one strip's plan,
-//         by the whole block.  Where the strip's codes outnumber the tables
-//         of their halves (most strips) the same entries are built digit by
+//         by the whole block.  Wherever the scratch holds the tables of a
+//         code's halves (most strips) the same entries are built digit by
 //         digit in affine coordinates instead (table_block), from the
 //         values that the compressed levels expand to.
-//  gather (one warp per output row i, component c and 32 output columns)
+//  gather (one warp per output row i and 32 ciphertext chains)
 //         C_ij += T_s[rank_s(i)] for every strip s: the "un-sort and re-insert
 //         duplicates" step of Algorithm 2 fused with the accumulation of
 //         Algorithm 3, one mixed addition per strip into an accumulator in
@@ -166,8 +166,7 @@ __global__ void __launch_bounds__(128) combine_tree_kernel(const uint4* __restri
 }
 
 // Gather of a product of one strip: every output is its row's table entry (Z
-// = 1) or infinity, a copy bound by memory. One warp per row, component and
-// 32 columns. At 512 x 1 x 16384 (w = 4) it takes 241 us, where gather_kernel at
+// = 1) or infinity, a copy bound by memory. One warp per row and 32 chains. At 512 x 1 x 16384 (w = 4) it takes 241 us, where gather_kernel at
 // its 128 registers keeps too few loads in flight (514 us).
 __global__ void __launch_bounds__(128) gather_copy_kernel(GatherArgs a, PlanPtrs P) {
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
