@@ -105,44 +105,28 @@ __global__ void __launch_bounds__(128, PCMM_GATHER_MINBLOCKS) gather_kernel(Gath
     gather_item<false>(a, P, gw);
 }
 
-// Adds the parts partial sums (Montgomery domain) of every output point (and, after the first
-// pass, the accumulated value) into ctC: one thread per point.
-__global__ void __launch_bounds__(128) combine_kernel(const uint4* __restrict__ partial, int parts,
+// Adds the parts partial sums (Montgomery domain) of every output point (and,
+// after the first pass, the accumulated value) into ctC: G = 2^logG lanes a point
+// add every G-th part each, and their sums as a tree. One lane a point waits for
+// its chain of additions: with as many lanes as give two warps per scheduler, 66
+// x 750 x 14 (w = 7, 32 parts) takes 40 us for 162, 29 x 926 x 86 (w = 4) 74 for
+// 172; with four warps 76 and 66.
+__global__ void __launch_bounds__(128) combine_kernel(const uint4* __restrict__ partial, int parts, int logG,
                                                       uint4* __restrict__ ctC, size_t ml, bool first) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 2 * ml) return;
-    const size_t c = t / ml, idx = t % ml;
+    const int G = 1 << logG, p = (int)t & (G - 1);
+    const bool valid = (t >> logG) < 2 * ml;
+    const size_t o = valid ? t >> logG : 0;
+    const size_t c = o >= ml, idx = o - c * ml;
     uint4* Cc = ctC + c * 6 * ml;
     jac acc;
-    if (first) {
-        jac_set_inf(acc);
-    } else {
-        load_jac(acc, Cc, ml, idx);
-        jac_to_mont(acc);
-    }
-    for (int p = 0; p < parts; p++) {
+    jac_set_inf(acc);
+    for (int x = p; x < parts; x += G) {
         jac Q;
-        load_jac(Q, partial + (size_t)p * 12 * ml + c * 6 * ml, ml, idx);
+        load_jac(Q, partial + (size_t)x * 12 * ml + c * 6 * ml, ml, idx);
         jac_add(acc, Q);
     }
-    jac_from_mont(acc);
-    store_jac(Cc, ml, idx, acc);
-}
-
-// combine_kernel for few outputs, where its chain of additions would be the
-// time: G lanes (a power of two, at least parts) load a part each and add
-// them as a tree, log2 G additions instead of parts.
-__global__ void __launch_bounds__(128) combine_tree_kernel(const uint4* __restrict__ partial, int parts, int G,
-                                                           uint4* __restrict__ ctC, size_t ml, bool first) {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int p = (int)(t % G);
-    const bool valid = t / G < 2 * ml;
-    const size_t o = valid ? t / G : 0;
-    const size_t c = o / ml, idx = o % ml;
-    uint4* Cc = ctC + c * 6 * ml;
-    jac acc;
-    if (p < parts) load_jac(acc, partial + (size_t)p * 12 * ml + c * 6 * ml, ml, idx);
-    else jac_set_inf(acc);
+    __syncwarp();
     for (int d = G / 2; d >= 1; d >>= 1) {
         jac Q;
 #pragma unroll
@@ -166,8 +150,9 @@ __global__ void __launch_bounds__(128) combine_tree_kernel(const uint4* __restri
 }
 
 // Gather of a product of one strip: every output is its row's table entry (Z
-// = 1) or infinity, a copy bound by memory. One warp per row and 32 chains. At 512 x 1 x 16384 (w = 4) it takes 241 us, where gather_kernel at
-// its 128 registers keeps too few loads in flight (514 us).
+// = 1) or infinity, a copy bound by memory. One warp per row and 32 chains. At 512 x
+// 1 x 16384 (w = 4) it takes 241 us, where gather_kernel at its 128 registers keeps
+// too few loads in flight (514 us).
 __global__ void __launch_bounds__(128) gather_copy_kernel(GatherArgs a, PlanPtrs P) {
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (gw >= (long long)a.m * a.nq) return;
@@ -335,15 +320,10 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         PCMM_CUDA_CHECK_LAUNCH();
         if (pc > 1) {
             ProfScope ps(KID_COMBINE, st);
-            int G = 2;
-            while (G < pc) G *= 2;
-            const size_t lanes = 2 * ml * G;
-            if (lanes <= (size_t)SCHEDULERS * 32)
-                combine_tree_kernel<<<(unsigned)((lanes + 127) / 128), 128, 0, st>>>((const uint4*)partial, pc, G,
-                                                                                    (uint4*)ctC, ml, s0 == 0);
-            else
-                combine_kernel<<<(unsigned)((2 * ml + 127) / 128), 128, 0, st>>>((const uint4*)partial, pc,
-                                                                                (uint4*)ctC, ml, s0 == 0);
+            int logG = 0;
+            while ((1 << logG) < pc && logG < 5 && ((2 * ml) << (logG + 1)) <= (size_t)2 * SCHEDULERS * 32) logG++;
+            combine_kernel<<<(unsigned)((((2 * ml) << logG) + 127) / 128), 128, 0, st>>>(
+                (const uint4*)partial, pc, logG, (uint4*)ctC, ml, s0 == 0);
         }
         PCMM_CUDA_CHECK_LAUNCH();
     }

@@ -98,3 +98,11 @@ def test_columns_that_fill_no_block(m, n, w, k, l):
     want = pcmm.normalize(pcmm.schoolbook(A, ctB, l, w), m * l)
     for out in pcmm.cussen_batched([(A, ctB, l, w, k)] * 2):
         assert torch.equal(pcmm.normalize(out, m * l), want)
+
+
+@pytest.mark.parametrize("m,n,l", [(60, 600, 30), (33, 700, 70), (300, 80, 130), (150, 300, 128)])
+def test_lanes_that_add_several_parts(m, n, l):
+    # Fewer lanes a point than parts (8, 8, 1 and 1), in one pass and in several.
+    pr = inputs.pcmm_problem(7700 + m, m, n, l, 2)
+    _check(pr, m, n, l, 2, 1)
+    _check(pr, m, n, l, 2, 1, ws=pcmm.cussen_workspace_bytes_for(m, n, l, 2, 1, n // 2 + 1))
