@@ -1027,6 +1027,19 @@ static __device__ __noinline__ void pair_sum(aff& S, const aff& A, const aff& B,
 
 __device__ __forceinline__ bool words345_zero(const fe& a) { return (a.v[3] | a.v[4] | a.v[5]) == 0u; }
 
+// Canonical form of a sum's coordinate; LATE: behind a test that one value in
+// 2^32 passes (p's top word is all ones), 2% off the tables of one column's
+// signed pairs (w = 16 22.05 -> 21.6 ms) and 1% onto the others.
+template <bool LATE>
+__device__ __forceinline__ void canon_of(fe& r, const fe& a) {
+    if (!LATE) {
+        fe_canon(r, a);
+        return;
+    }
+    r = a;
+    if (r.v[7] == 0xffffffffu) fe_canon(r, r);
+}
+
 // With both signs the multiplications are called: inlined, two copies of the
 // sum outgrow the instruction cache (w = 8 below 11.1 against 10.5 ms).
 template <bool BOTH>
@@ -1043,7 +1056,7 @@ __device__ __forceinline__ fe batch_mul(const fe& a, const fe& b) {
 // difference of x and its inverse: 7M + 2S instead of 10M + 2S. pref: cnt field
 // elements of lane-planar scratch. All 128 threads of the block call; cnt may
 // differ from warp to warp. `turn` names the warp that inverts.
-template <bool BOTH, class Pair, class Put>
+template <bool BOTH, bool LATE, class Pair, class Put>
 __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4* pref, uint4* sm, unsigned turn) {
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, tid = threadIdx.x;
     const unsigned all = 0xffffffffu;
@@ -1122,11 +1135,11 @@ __device__ __forceinline__ void affine_batch(int cnt, Pair pair, Put put, uint4*
             }
             fe_sub_canon(t, t, A.x);
             fe_sub_canon(t, t, B.x);
-            fe_canon(S.x, t);
+            canon_of<LATE>(S.x, t);
             fe_sub_canon(t, A.x, S.x);
             t = batch_mul<BOTH>(lam, t);
             fe_sub_canon(S.y, t, A.y);
-            fe_canon(S.y, S.y);
+            canon_of<LATE>(S.y, S.y);
             put(i, sign, S);
         };
         if (!BOTH || (want & 1u)) finish(0);
@@ -1205,8 +1218,8 @@ __host__ __device__ inline int digit_bits(const TableArgs& a, int d) {
 //  - Columns of four bits: v P1 + u P0 is (v P1 + 8 P0) + (u - 8) P0, and the
 //    upper digit's chain goes on from 8 P0 where the lower one's ends.
 // Table times without and with signed pairs (ms): 1024 x 1024 x 256 at w = 8 12.6
-// and 10.5, with one value in ten not zero 7.0 and 6.5, at w = 4 6.2 and 5.3; 512
-// x 512 x 256 at w = 16 24.0 and 22.2.
+// and 10.2, with one value in ten not zero 7.0 and 6.3, at w = 4 6.2 and 5.3; 512
+// x 512 x 256 at w = 16 24.0 and 21.6.
 __host__ __device__ inline bool signed_pair(const TableArgs& a, int d, int end) {
     if (d + 1 >= end) return false;
     return a.dpc == 1 ? a.w == 4 : d % a.dpc + 1 < a.dpc && digit_bits(a, d + 1) >= 2;
@@ -1275,7 +1288,8 @@ __device__ __forceinline__ const uint16_t* column_values(const PlanPtrs& P, int 
 }
 
 // Table of one warp item by digits; PAIRS: no signed pairs, pairs of one column's
-// digits or of two columns (a.pairs). One copy for all would slow each by 2-5%.
+// digits (1; 3 as part of the batched kernel) or of two columns (a.pairs). One copy
+// for all would slow each by 2-5%.
 // All 128 threads of the block call (valid: the warp has an item); sm:
 // DIGIT_SHARED_U4 uint4 of shared memory.
 template <int PAIRS>
@@ -1608,7 +1622,7 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             pick(i, g, v, tab, pa);
             lp_store_aff(tab, minus ? v - g : v + g, lane, S);
         };
-        affine_batch<SIGNED>(n[0] + n[1], pair, put, pref, sm, turn++);
+        affine_batch<SIGNED, PAIRS == 1>(n[0] + n[1], pair, put, pref, sm, turn++);
     }
 
     // 3. The strip's entries.
@@ -1641,7 +1655,7 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             cnt += __popc(mask);
         }
         __syncwarp();
-        affine_batch<true>(
+        affine_batch<true, PAIRS == 1>(
             cnt,
             [&](int i, const uint4*& pa, const uint4*& pb) -> unsigned {
                 const uint32_t x = list[i];
@@ -1655,7 +1669,7 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
             },
             pref, sm, turn);
     } else if (a.nd > 1) {
-        affine_batch<false>(
+        affine_batch<false, PAIRS == 1>(
             E,
             [&](int e, const uint4*& pa, const uint4*& pb) -> unsigned {
                 const uint32_t code = codes[e];

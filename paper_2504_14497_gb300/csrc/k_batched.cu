@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) batched_plan_kernel(const Inst* 
 // signed pairs and one without as well (50.4).
 static __device__ __noinline__ void digit_item(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
                                                uint4* scratch, uint4* sm) {
-    table_block<1>(a, P, item, valid, scratch, sm);
+    table_block<3>(a, P, item, valid, scratch, sm);
 }
 
 // Resident blocks per SM requested from the compiler: 4 (128 registers, some

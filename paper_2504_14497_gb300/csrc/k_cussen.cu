@@ -79,8 +79,9 @@ __global__ void __launch_bounds__(128, BLOCKS) table_kernel(TableArgs a, PlanPtr
 // table_kernel by digits (table_block): two thirds of the multiplications and
 // hardly any spills, so it is faster than the chains and wants registers more
 // than warps. Table times of 1024 x 1024 x 256 (ms), chains and digits at 3, 4,
-// 5 and 6 blocks per SM: w = 8 21.5 / 10.9, 10.5, 10.5, 10.9; w = 4 8.3 / 5.5,
-// 5.3, 5.7, 6.0; 512 x 512 x 256, w = 16: 36.6 / 24.0, 22.1, 23.1, 25.4.
+// 5 and 6 blocks per SM: w = 8 21.5 / 10.9, 10.4, 10.4, 10.9; w = 4 8.3 / 5.5,
+// 5.3, 5.7, 6.0; 512 x 512 x 256, w = 16: 36.6 / 24.0, 22.1, 23.1, 25.4 (before canonical
+// forms moved behind a test, which took 2% off at 4).
 #ifndef PCMM_DIGIT_MINBLOCKS
 #define PCMM_DIGIT_MINBLOCKS 4
 #endif
