@@ -242,15 +242,17 @@ int part_strips(const Layout& L, size_t S) {
     return (long long)L.m * 2 * L.njb * (long long)(S / 4) <= 2 * SCHEDULERS ? 4 : 16;
 }
 
-int gather_parts(const Layout& L, size_t S) {
+int gather_parts(const Layout& L, size_t S, int least) {
     const long long warps = (long long)L.m * 2 * L.njb;
     if (warps >= GATHER_WARPS_TARGET) return 1;
     long long parts = (GATHER_WARPS_TARGET + warps - 1) / warps;
-    const long long by_strips = (long long)S / part_strips(L, S);
+    const long long by_strips = (long long)S / least;
     if (parts > by_strips) parts = by_strips;
     if (parts > 32) parts = 32;
     return parts < 1 ? 1 : (int)parts;
 }
+
+int gather_parts(const Layout& L, size_t S) { return gather_parts(L, S, part_strips(L, S)); }
 
 size_t partial_bytes(const Layout& L, int parts) {
     return parts > 1 ? align256((size_t)parts * 2 * L.m * L.l * 96) : 0;
@@ -350,19 +352,31 @@ size_t default_exec_bytes(const Layout& L) {
 
 // Splits `avail` bytes of execution workspace into the partial sums (when
 // the gather splits its strips) and passes of S strips; the partial sums are
-// dropped when both do not fit.  False when not even one strip fits.
+// dropped when both do not fit, and made of parts of at least 16 strips where
+// the room of smaller parts would cost passes: 73 x 41 x 63 (w = 1, k = 3) in a
+// workspace for its 14 strips and no partial sums took 14 passes, 977 us, with
+// parts of 4, and takes one, 111 us, without. False when not even one strip
+// fits.
 bool exec_space(const Layout& L, size_t avail, size_t& S, int& parts, size_t& pbytes) {
-    parts = gather_parts(L, default_strips(L));
-    pbytes = partial_bytes(L, parts);
-    if (parts > 1 && avail >= pbytes + L.per_strip_bytes) {
-        S = (avail - pbytes) / L.per_strip_bytes;
-    } else {
-        parts = 1;
-        pbytes = 0;
-        if (avail < L.per_strip_bytes) return false;
-        S = avail / L.per_strip_bytes;
+    if (avail < L.per_strip_bytes) return false;
+    const size_t S0 = default_strips(L);
+    size_t passes = 0;
+    for (int least = 16; least >= part_strips(L, S0); least -= 12) {
+        int p = gather_parts(L, S0, least);
+        size_t pb = partial_bytes(L, p);
+        if (p > 1 && avail < pb + L.per_strip_bytes) {
+            p = 1;
+            pb = 0;
+        }
+        size_t s = (avail - pb) / L.per_strip_bytes;
+        if (s > (size_t)L.nstrips) s = L.nstrips;
+        const size_t n = (L.nstrips + s - 1) / s;
+        if (passes && n > passes) break;
+        passes = n;
+        S = s;
+        parts = p;
+        pbytes = pb;
     }
-    if (S > (size_t)L.nstrips) S = L.nstrips;
     const int ps = gather_parts(L, S);
     if (ps < parts) parts = ps;
     return true;
