@@ -486,7 +486,10 @@ const char *pcmm_kernel_name(int id);
  * Unit-test entry points for the device arithmetic (device arrays of
  * `count` items, quad-planar like the point arrays).
  * pcmm_test_field: op 0 add, 1 sub, 2 mul, 3 sqr, 4 inv, 5 canonical
- *   form; a, b: 2 quads per element (b unused for ops 3-5); out canonical.
+ *   form, of standard residues; of the words as they are (any values below
+ *   2^256, R = 2^256): 6 the kernels' shared inversion, R^2 / a (0 for 0),
+ *   7 a - b for b <= p, 8 (a b - a' b') / R with x' = 2^256 - 1 - x, 9 a^2 / R^2;
+ *   a, b: 2 quads per element (b unused for ops 3-6 and 9); out canonical.
  * pcmm_test_point: op 0 dbl(P), 1 P + Q (mixed: Q affine), 2 P + Q (both
  *   Jacobian), 3 k P for a small scalar k (P affine, k = kscal[i]);
  *   P: Jacobian (6 quads) for ops 0-2, affine (4 quads) for op 3; Q: affine

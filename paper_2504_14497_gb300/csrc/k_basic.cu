@@ -331,14 +331,18 @@ __global__ void __launch_bounds__(128) normalize_kernel(const uint4* __restrict_
     }
 }
 
+// Ops up to 5 take and give standard residues; the others work on the words as
+// they are (include/pcmm.h).
 __global__ void __launch_bounds__(128) test_field_kernel(int op, const uint4* __restrict__ a,
                                                          const uint4* __restrict__ b,
                                                          uint4* __restrict__ out, size_t count) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
+    const bool valid = i < count;
+    const size_t ii = valid ? i : count - 1;
+    const bool two = op <= 2 || op == 7 || op == 8;
     fe x, y, r;
-    load_fe(x, a, count, i);
-    if (op <= 2) load_fe(y, b, count, i);
+    load_fe(x, a, count, ii);
+    if (two) load_fe(y, b, count, ii);
     if (op >= 2 && op <= 4) {
         fe_to_mont(x, x);
         if (op == 2) fe_to_mont(y, y);
@@ -349,11 +353,30 @@ __global__ void __launch_bounds__(128) test_field_kernel(int op, const uint4* __
         case 2: fe_mul(r, x, y); break;
         case 3: fe_sqr(r, x); break;
         case 4: fe_inv(r, x); break;
+        case 6:
+            // The warp inverts its lanes' values one after another.
+            for (int lane = 0; lane < 32; lane++) {
+                const fe t = warp_uniform_inv(fe_shfl(x, lane));
+                if ((int)(threadIdx.x & 31u) == lane) r = t;
+            }
+            break;
+        case 7: fe_sub_canon(r, x, y); break;
+        case 8: {
+            fe cx, cy;
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                cx.v[j] = ~x.v[j];
+                cy.v[j] = ~y.v[j];
+            }
+            r = fe_mulsub(x, y, cx, cy);
+            break;
+        }
+        case 9: r = fe_sqr_std(x); break;
         default: r = x; break;
     }
     if (op >= 2 && op <= 4) fe_from_mont(r, r);
     fe_canon(r, r);
-    store_fe(out, count, i, r);
+    if (valid) store_fe(out, count, i, r);
 }
 
 __global__ void __launch_bounds__(128) test_point_kernel(int op, const uint4* __restrict__ P,
@@ -604,7 +627,7 @@ extern "C" pcmm_status pcmm_test_wait(const int* ctr, int target, uint32_t* stat
 
 extern "C" pcmm_status pcmm_test_field(int op, const uint32_t* a, const uint32_t* b, uint32_t* out,
                                        size_t count, pcmm_stream_t stream) {
-    if (op < 0 || op > 5 || !a || !out || (op <= 2 && !b)) return PCMM_EINVAL;
+    if (op < 0 || op > 9 || !a || !out || ((op <= 2 || op == 7 || op == 8) && !b)) return PCMM_EINVAL;
     if (count == 0) return PCMM_OK;
     test_field_kernel<<<grid_for(count, 128), 128, 0, (cudaStream_t)stream>>>(
         op, (const uint4*)a, (const uint4*)b, (uint4*)out, count);
