@@ -84,12 +84,15 @@ __device__ __forceinline__ fe fe_shfl(const fe& a, int src) {
 // Bound by its serial chain in one warp: 18 batches with about 96 rounds of
 // the inner loop in all. Normalising 10 ciphertexts, which waits on one
 // inversion, takes 33 us, against 76 us with a binary extended Euclid that
-// every lane repeats on full-width values.
+// every lane repeats on full-width values.  A product of factors that are all 1
+// (points that are still affine, digits without a chain) is returned at once, as
+// that Euclid did: the baby steps of 256 messages take 19 us, not 25.
 static __device__ __noinline__ fe warp_uniform_inv(fe a) {
     const unsigned lane = threadIdx.x & 31u;
     const int M30 = 0x3fffffff;
     const unsigned all = 0xffffffffu;
     fe_canon(a, a);
+    if (fe_is_one(a)) return a;
     // The limbs of this lane's value W and its partner's V.
     int W[9], V[9];
     {

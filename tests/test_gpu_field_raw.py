@@ -62,3 +62,22 @@ def test_square_reduced_twice():
     ri = pow(R * R, -1, P)
     for x, g in zip(a, _run(9, a)):
         assert g == x * x * ri % P, hex(x)
+
+
+def test_shared_inversion_of_one_is_free():
+    # Products of factors that are all 1 (affine points) need no division steps.
+    import torch
+
+    dev = device()
+    count = 152 * 4 * 128
+    times = []
+    for v in (ONE, 3 * ONE % P):
+        a = pcmm.to_device_words(ints_to_planar_fe([v]), dev).view(2, 1, 4).expand(2, count, 4).reshape(-1).contiguous()
+        pcmm.test_field(6, a)
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        pcmm.test_field(6, a)
+        end.record()
+        end.synchronize()
+        times.append(start.elapsed_time(end))
+    assert times[0] < 0.5 * times[1], times
