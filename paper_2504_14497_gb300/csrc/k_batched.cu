@@ -48,13 +48,16 @@ struct Inst {
     PlanPtrs P;
     uint4* tables;              // two buffers of 4 * table_points uint4
     size_t table_points;        // points per buffer (S strips)
-    size_t item_u4;
     int m, n, l, w, k;
-    int nstrips, n1max, l2max, emax, lp, span, nq;
+    int nstrips, n1max, l2max, emax, lp, nq;
     int S, nchunks;
     int ctr_base;               // 2 counters per pass: tables done, gathers done
-    int digits, dpc, nd, ns, hl, hh;   // table build by digits (digit_split)
+    uint8_t packed;             // lane_span is l
+    uint8_t digits, dpc, ns, hl;   // table build by digits (digit_split)
 };
+// The instances lie in the workspace: a larger record would refuse workspaces of
+// sizes that callers keep.
+static_assert(sizeof(Inst) <= 184, "batched workspace sizes grow with Inst");
 
 struct Segment {
     long long start;            // first task index of the segment
@@ -151,14 +154,14 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
             const bool shared = (ips % BLOCK_TASKS) == 0;
             {
                 TableArgs ta;
-                ta.dpc = I.dpc; ta.nd = I.nd; ta.ns = I.ns; ta.hl = I.hl; ta.hh = I.hh;
+                ta.dpc = I.dpc; ta.nd = I.k * I.dpc; ta.ns = I.ns; ta.hl = I.hl; ta.hh = I.w * I.k - I.hl;
                 ta.ctB = I.ctB;
                 ta.bshare = shared;
                 ta.m = I.m; ta.n = I.n; ta.l = I.l; ta.w = I.w; ta.k = I.k;
-                ta.lp = I.lp; ta.span = I.span; ta.nq = I.nq; ta.n1max = I.n1max; ta.l2max = I.l2max; ta.emax = I.emax;
+                ta.lp = I.lp; ta.span = I.packed ? I.l : I.lp; ta.nq = I.nq;
+                ta.n1max = I.n1max; ta.l2max = I.l2max; ta.emax = I.emax;
                 ta.s0 = s0; ta.nstrips_chunk = sc;
                 ta.scratch = my_scratch;
-                ta.item_u4 = I.item_u4;
                 ta.table = tbuf;
                 ta.table_points = I.table_points;
                 if (I.digits) digit_item(ta, I.P, item, real, my_scratch, sh_inv);
@@ -166,7 +169,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
             }
         } else if (real) {
             GatherArgs ga;
-            ga.m = I.m; ga.l = I.l; ga.lp = I.lp; ga.span = I.span; ga.nq = I.nq; ga.emax = I.emax;
+            ga.m = I.m; ga.l = I.l; ga.lp = I.lp; ga.span = I.packed ? I.l : I.lp; ga.nq = I.nq; ga.emax = I.emax;
             ga.parts = 1; ga.partial = nullptr;
             ga.s0 = s0; ga.nstrips_chunk = sc;
             ga.first = (sg.chunk == 0);
@@ -265,10 +268,10 @@ pcmm_status build_layout(const pcmm_problem* probs, int count, int max_strips, i
         ctr += 2 * I.nchunks;
         I.m = L.m; I.n = L.n; I.l = L.l; I.w = L.w; I.k = L.k;
         I.nstrips = L.nstrips; I.n1max = L.n1max; I.l2max = L.l2max; I.emax = L.emax;
-        I.lp = L.lp; I.span = lane_span(L.l); I.nq = lane_blocks(L.l); I.item_u4 = L.item_u4;
+        I.lp = L.lp; I.packed = lane_span(L.l) == L.l ? 1 : 0; I.nq = lane_blocks(L.l);
         TableArgs split;
-        I.digits = digit_split(L, split);
-        I.dpc = split.dpc; I.nd = split.nd; I.ns = split.ns; I.hl = split.hl; I.hh = split.hh;
+        I.digits = digit_split(L, split) ? 1 : 0;
+        I.dpc = (uint8_t)split.dpc; I.ns = (uint8_t)split.ns; I.hl = (uint8_t)split.hl;
         H.scratch_u4 = std::max(H.scratch_u4, L.item_u4);
     }
     H.nctrs = ctr;
@@ -294,7 +297,7 @@ pcmm_status build_layout(const pcmm_problem* probs, int count, int max_strips, i
                 sg.type = ph == 0 ? TASK_TABLE : TASK_GATHER;
                 sg.inst = i;
                 sg.chunk = r;
-                sg.count = ph == 0 ? sc * I.nq : I.m * I.nq;
+                sg.count = (ph == 0 ? sc : I.m) * I.nq;
                 H.segs.push_back(sg);
                 // Segments start at multiples of BLOCK_TASKS: a block's tasks
                 // never straddle two segments (padding tasks do nothing).

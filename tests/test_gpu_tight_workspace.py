@@ -27,3 +27,13 @@ def test_all_strips_in_one_pass(m, n, l, w, k, extra):
     assert pcmm.workspace_status(ws) == 0
     assert torch.equal(pcmm.normalize(jac, m * l), want)
     assert gathers == 1
+
+
+@pytest.mark.parametrize("count", [1, 8, 39])
+def test_batched_workspace_holds_184_bytes_an_instance(count):
+    # Workspaces of sizes that callers keep are still large enough.
+    dev = device()
+    A = torch.ones((4, 4), dtype=torch.uint8, device=dev)
+    ctB = torch.zeros(32 * 4 * 2, dtype=torch.int32, device=dev)
+    info = pcmm.Batch([(A, ctB, 2, 1, 1)] * count).info
+    assert info.off_segs - info.off_insts <= (184 * count + 255) // 256 * 256
