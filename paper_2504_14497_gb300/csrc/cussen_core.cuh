@@ -471,6 +471,13 @@ struct TableArgs {
     int pairs;             // signed pairs: 0 none, 1 of one column's digits, 2 of two columns
 };
 
+// What strip_excess compares, and whether a pass of few codes goes by chains
+// (either; small: in launches of few blocks too).
+struct FewArgs {
+    bool either, small;
+    int fixed, entry;
+};
+
 __device__ __forceinline__ void lp_store_aff(uint4* base, int e, unsigned lane, const aff& Q) {
     uint4* b = base + (size_t)e * 4 * 32 + lane;
     b[0] = fe_lo(Q.x);
@@ -1689,9 +1696,51 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
     }
 }
 
+// What a strip's table costs by chains of prefix sums (table_item) beyond its cost by
+// digits. The digits' chains and the halves' tables are made whatever the
+// strip holds, so strips of few distinct codes (sparse columns, columns of few
+// values) are cheaper by chains, which cost what they hold. In tenths of the
+// microseconds that one of 608 warp schedulers takes, fitted to 840 table times (w = 1
+// to 16, strips of 1 to 6 columns, densities 0.003 to 1, columns of 1, 2 and 4 values);
+// the chains count 1.05 times, so that close calls go by digits. Tables of 256 columns of 256
+// (us) by digits and by chains: w = 8 with 3.6 values a column 841 and 659, w = 12
+// with 50 3833 and 3224, with 101 4383 and 4415, w = 16 with 3.2 5477 and 1214.
+__device__ __forceinline__ int strip_excess(int entries, const uint16_t* len, int columns, int w, const FewArgs& f) {
+    int chains = 0;
+    for (int t = 0; t < columns; t++, len += NLEV) {
+        const int l1 = len[0];
+        if (!l1) continue;
+        chains += 33 * (l1 - 1) + 19 * (w - 1) * len[NLEV - 1] + (w > 1 ? 144 : 0);
+        for (int q = 1; q < NLEV - 1; q++) chains += 36 * (len[q] - 1);
+    }
+    return entries > 0 ? chains - f.entry * entries - f.fixed : -f.fixed;
+}
+
+// Whether a pass's tables cost less by chains than by digits: the sum over its
+// strips, so that one of the two kernels builds them all (block by block, each kernel
+// took the time of a whole wave: 1024 x 256 x 256 at w = 16 with 21 values a column 7.3 ms,
+// 4.5 as it is). All 128 threads of the block call; sm: 2 uint4.
+static __device__ __noinline__ bool pass_few(const int32_t* nent, const uint16_t* col_len, int s0, int strips, int n, int k,
+                                             int w, int emax, FewArgs f, uint4* sm) {
+    long long sum = 0;
+    for (int x = (int)threadIdx.x; x < strips; x += 128) {
+        const int s = s0 + x, c0 = s * k, E = nent[s];
+        sum += strip_excess(E < emax ? E : emax, col_len + (size_t)c0 * NLEV, c0 + k <= n ? k : n - c0, w, f);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+    long long* part = (long long*)sm;
+    if ((threadIdx.x & 31u) == 0) part[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    sum = part[0] + part[1] + part[2] + part[3];
+    __syncthreads();
+    return sum < 0;
+}
+
 // The digits and halves of a strip code, and whether the digit build takes
 // the tables of this layout.
-inline bool digit_split(const Layout& L, TableArgs& a) {
+inline bool digit_split(const Layout& L, TableArgs& a, FewArgs& few) {
     a.dpc = (L.w + 3) / 4;
     a.nd = L.k * a.dpc;
     a.ns = 1;
@@ -1716,7 +1765,33 @@ inline bool digit_split(const Layout& L, TableArgs& a) {
     a.w = L.w;
     const bool any = (a.nd == 2 && signed_pair(a, 0, 2)) || signed_pair(a, 0, a.ns) || signed_pair(a, a.ns, a.nd);
     a.pairs = !any ? 0 : a.dpc > 1 ? 1 : 2;
-    return digit_scratch(L.w, L.k, a.dpc, a.hl, a.hh, L.n1max, L.l2max, L.emax).total <= L.item_u4;
+    // Costs for strip_excess: the steps of the digits' chains, the halves' sums and
+    // the inversions of a strip, its columns, and for each entry its sum by
+    // digits less the sums of its parts by chains.
+    const bool two = a.nd == 2 && signed_pair(a, 0, 2);
+    const bool sp[2] = {two || signed_pair(a, 0, a.ns), signed_pair(a, a.ns, a.nd)};
+    int steps = 0, digit_entries = 0;
+    for (int d = 0; d < a.nd; d++) {
+        const bool more = d % a.dpc + 1 < a.dpc;
+        const bool lower = (sp[0] && d == 0) || (sp[1] && d == a.ns);
+        const bool upper = (sp[0] && d == 1) || (sp[1] && d == a.ns + 1);
+        const int all = 1 << digit_bits(a, d);
+        steps += (lower ? (a.dpc == 1 ? 8 : 9) : all - (more || upper ? 0 : 1)) - 1;
+        digit_entries += all;
+    }
+    const int sums = a.nd > 1 ? (1 << a.hl) + (1 << a.hh) - digit_entries : 0;
+    const int rounds = (a.ns > a.nd - a.ns ? a.ns : a.nd - a.ns) - 1;
+    const int inversions = (L.w > 1 ? a.dpc : 0) + rounds + (a.nd > 1 ? 1 : 0);
+    few.fixed = (int)(38.8 * steps + 14.0 * (sums > 0 ? sums : 0) + 77.1 * inversions + 8.4 * L.k - 184.0);
+    few.entry = (int)((a.nd > 1 ? 13.9 : 0.0) - (L.k > 1 ? 34.0 * (L.k * (1.0 - 1.0 / (1 << L.w)) - 1.0) : 0.0));
+    const bool fits = digit_scratch(L.w, L.k, a.dpc, a.hl, a.hh, L.n1max, L.l2max, L.emax).total <= L.item_u4;
+    // A second launch costs a small call 5 to 7 us (10 x 128 x 1 at w = 4 175 and
+    // 182, 512 x 1 x 16384 814 and 821). There the time is the latency of one strip's
+    // build, and that of the digits is short with one place of digits and no round
+    // between it and the entries: 98 us where a nearly empty strip takes 44 by chains.
+    few.either = fits;
+    few.small = fits && (L.w == 1 || inversions > 2);
+    return fits;
 }
 
 struct GatherArgs {

@@ -270,7 +270,8 @@ pcmm_status build_layout(const pcmm_problem* probs, int count, int max_strips, i
         I.nstrips = L.nstrips; I.n1max = L.n1max; I.l2max = L.l2max; I.emax = L.emax;
         I.lp = L.lp; I.packed = lane_span(L.l) == L.l ? 1 : 0; I.nq = lane_blocks(L.l);
         TableArgs split;
-        I.digits = digit_split(L, split) ? 1 : 0;
+        FewArgs few;
+        I.digits = digit_split(L, split, few) ? 1 : 0;
         I.dpc = (uint8_t)split.dpc; I.ns = (uint8_t)split.ns; I.hl = (uint8_t)split.hl;
         H.scratch_u4 = std::max(H.scratch_u4, L.item_u4);
     }

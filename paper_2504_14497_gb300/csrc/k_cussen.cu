@@ -69,9 +69,13 @@ __global__ void __launch_bounds__(PLAN_THREADS) plan_kernel(const TA* __restrict
 }
 
 template <int BLOCKS>
-__global__ void __launch_bounds__(128, BLOCKS) table_kernel(TableArgs a, PlanPtrs P) {
+__global__ void __launch_bounds__(128, BLOCKS) table_kernel(TableArgs a, PlanPtrs P, FewArgs f) {
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nitems = (long long)a.nstrips_chunk * a.nq;
+    if (f.either) {
+        __shared__ uint4 sm[2];
+        if (!pass_few(P.nent, P.col_len, a.s0, a.nstrips_chunk, a.n, a.k, a.w, a.emax, f, sm)) return;
+    }
     if (item >= nitems) return;
     table_item(a, P, item, a.scratch + (size_t)item * a.item_u4);
 }
@@ -92,10 +96,12 @@ __global__ void __launch_bounds__(128, BLOCKS) table_kernel(TableArgs a, PlanPtr
 // blocks per SM the copies lose (256 x 784 x 64 1.01 -> 1.35 ms).
 constexpr unsigned FEW_BLOCKS = 2 * 152;
 template <int PAIRS, int BLOCKS>
-__global__ void __launch_bounds__(128, BLOCKS) digit_table_kernel(TableArgs a, PlanPtrs P) {
+__global__ void __launch_bounds__(128, BLOCKS) digit_table_kernel(TableArgs a, PlanPtrs P, FewArgs f) {
     __shared__ uint4 sm[DIGIT_SHARED_U4];
     const long long item = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const bool valid = item < (long long)a.nstrips_chunk * a.nq;
+    // As a jump out of the kernel, a return cost the tables of w = 16 3% (spills).
+    if (f.either && pass_few(P.nent, P.col_len, a.s0, a.nstrips_chunk, a.n, a.k, a.w, a.emax, f, sm)) asm volatile("exit;");
     uint4* scratch = a.scratch + (valid ? (size_t)item : (size_t)0) * a.item_u4;
     table_block<PAIRS>(a, P, item, valid, scratch, sm);
 }
@@ -267,7 +273,8 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
     uint4* table = (uint4*)(chunk + align256(S * L.items_per_strip * L.item_u4 * 16));
     const size_t ml = (size_t)L.m * L.l;
     TableArgs split;
-    const bool digits = digit_split(L, split);
+    FewArgs fa;
+    const bool digits = digit_split(L, split, fa);
     for (int s0 = 0; s0 < L.nstrips; s0 += (int)S) {
         const int sc = (int)((size_t)(L.nstrips - s0) < S ? (size_t)(L.nstrips - s0) : S);
         TableArgs ta = split;
@@ -284,22 +291,22 @@ pcmm_status launch_exec(const Layout& L, const PlanPtrs& P, const uint32_t* ctB,
         // full and its warps follow the same plan, and share inversions.
         ta.bshare = (ta.nq % 4) == 0;
         const long long items = (long long)sc * ta.nq;
-        {
+        const unsigned blocks = (unsigned)((items + 3) / 4);
+        const bool few = blocks <= FEW_BLOCKS;
+        FewArgs f = fa;
+        f.either = few ? fa.small : fa.either;
+        if (digits) {
             ProfScope ps(KID_TABLE, st);
-            const unsigned blocks = (unsigned)((items + 3) / 4);
-            const int kind = digits ? 1 + split.pairs : 0;
-            auto* kernel = table_kernel<PCMM_TABLE_MINBLOCKS>;
-            if (blocks <= FEW_BLOCKS) {
-                if (kind == 0) kernel = table_kernel<1>;
-                else if (kind == 1) kernel = digit_table_kernel<0, 1>;
-                else if (kind == 2) kernel = digit_table_kernel<1, 1>;
-                else kernel = digit_table_kernel<2, 1>;
-            } else if (kind) {
-                if (kind == 1) kernel = digit_table_kernel<0, PCMM_DIGIT_MINBLOCKS>;
-                else if (kind == 2) kernel = digit_table_kernel<1, PCMM_DIGIT_MINBLOCKS>;
-                else kernel = digit_table_kernel<2, PCMM_DIGIT_MINBLOCKS>;
-            }
-            kernel<<<blocks, 128, 0, st>>>(ta, P);
+            auto* kernel = few ? digit_table_kernel<0, 1> : digit_table_kernel<0, PCMM_DIGIT_MINBLOCKS>;
+            if (split.pairs == 1) kernel = few ? digit_table_kernel<1, 1> : digit_table_kernel<1, PCMM_DIGIT_MINBLOCKS>;
+            if (split.pairs == 2) kernel = few ? digit_table_kernel<2, 1> : digit_table_kernel<2, PCMM_DIGIT_MINBLOCKS>;
+            kernel<<<blocks, 128, 0, st>>>(ta, P, f);
+            PCMM_CUDA_CHECK_LAUNCH();
+        }
+        if (!digits || f.either) {   // which of the two builds the tables is decided on the device
+            ProfScope ps(KID_TABLE, st);
+            auto* kernel = few ? table_kernel<1> : table_kernel<PCMM_TABLE_MINBLOCKS>;
+            kernel<<<blocks, 128, 0, st>>>(ta, P, f);
         }
         PCMM_CUDA_CHECK_LAUNCH();
         GatherArgs ga;
