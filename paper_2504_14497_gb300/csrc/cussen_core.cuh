@@ -1713,7 +1713,8 @@ __device__ __forceinline__ int strip_excess(int entries, const uint16_t* len, in
         chains += 33 * (l1 - 1) + 19 * (w - 1) * len[NLEV - 1] + (w > 1 ? 144 : 0);
         for (int q = 1; q < NLEV - 1; q++) chains += 36 * (len[q] - 1);
     }
-    return entries > 0 ? chains - f.entry * entries - f.fixed : -f.fixed;
+    // f.fixed counts the chains' own constant, which an empty strip does not have.
+    return entries > 0 ? chains - f.entry * entries - f.fixed : -(f.fixed + 184 + 80 * columns);
 }
 
 // Whether a pass's tables cost less by chains than by digits: the sum over its
