@@ -52,8 +52,10 @@ struct Inst {
     int nstrips, n1max, l2max, emax, lp, nq;
     int S, nchunks;
     int ctr_base;               // 2 counters per pass: tables done, gathers done
-    uint8_t packed;             // lane_span is l
-    uint8_t digits, dpc, ns, hl;   // table build by digits (digit_split)
+    uint8_t packed : 1;         // lane_span is l
+    uint8_t digits : 1;         // table build by digits (digit_split), or by chains where those cost less
+    uint8_t dpc, ns, hl;
+    int16_t few_fixed, few_entry;   // FewArgs
 };
 // The instances lie in the workspace: a larger record would refuse workspaces of
 // sizes that callers keep.
@@ -82,6 +84,22 @@ __global__ void __launch_bounds__(PLAN_THREADS) batched_plan_kernel(const Inst* 
 static __device__ __noinline__ void digit_item(const TableArgs& a, const PlanPtrs& P, long long item, bool valid,
                                                uint4* scratch, uint4* sm) {
     table_block<3>(a, P, item, valid, scratch, sm);
+}
+
+// Whether the strips of a block's table tasks (items from `item` on, the last of
+// them below `count`) cost less by chains than by digits (strip_excess). Blocks take
+// their tasks one by one, so each may choose for itself.
+__device__ __forceinline__ bool block_few(const Inst& I, int s0, int item, int count) {
+    FewArgs f;
+    f.fixed = I.few_fixed;
+    f.entry = I.few_entry;
+    const int last = min(item + BLOCK_TASKS, count) - 1;
+    for (int s = s0 + item / I.nq; s <= s0 + last / I.nq; s++) {
+        const int c0 = s * I.k;
+        if (strip_excess(min(I.P.nent[s], I.emax), I.P.col_len + (size_t)c0 * NLEV, min(I.k, I.n - c0), I.w, f) >= 0)
+            return false;
+    }
+    return true;
 }
 
 // Resident blocks per SM requested from the compiler: 4 (128 registers, some
@@ -124,6 +142,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
                 const int sc = min(I.S, I.nstrips - sg.chunk * I.S);
                 if (sg.type == TASK_TABLE) {
                     if (sg.chunk >= 2) go = wait_at_least(tdone - 4 + 1, I.m * I.nq, &hdr->status);
+                    if (go && I.digits && !block_few(I, sg.chunk * I.S, (int)(t0 - sg.start), sg.count)) go = 3;
                 } else {
                     go = wait_at_least(tdone, sc * I.nq, &hdr->status);
                     if (go && sg.chunk > 0) go = wait_at_least(tdone - 2 + 1, I.m * I.nq, &hdr->status);
@@ -164,7 +183,7 @@ __global__ void __launch_bounds__(BATCH_THREADS, PCMM_BATCH_MINBLOCKS) batched_k
                 ta.scratch = my_scratch;
                 ta.table = tbuf;
                 ta.table_points = I.table_points;
-                if (I.digits) digit_item(ta, I.P, item, real, my_scratch, sh_inv);
+                if (go & 2) digit_item(ta, I.P, item, real, my_scratch, sh_inv);
                 else if (real) table_item(ta, I.P, item, my_scratch);
             }
         } else if (real) {
@@ -273,6 +292,7 @@ pcmm_status build_layout(const pcmm_problem* probs, int count, int max_strips, i
         FewArgs few;
         I.digits = digit_split(L, split, few) ? 1 : 0;
         I.dpc = (uint8_t)split.dpc; I.ns = (uint8_t)split.ns; I.hl = (uint8_t)split.hl;
+        I.few_fixed = (int16_t)few.fixed; I.few_entry = (int16_t)few.entry;
         H.scratch_u4 = std::max(H.scratch_u4, L.item_u4);
     }
     H.nctrs = ctr;

@@ -53,6 +53,44 @@ def test_few_beside_dense(w, k, m, l):
         assert torch.equal(got, want)
 
 
+@pytest.mark.parametrize("w,m", [(8, 300), (4, 90), (5, 40), (1, 70)])
+def test_few_beside_dense_in_a_batch(w, m):
+    # Blocks choose one by one, some of them with strips of both kinds.
+    dev = device()
+    items, want = [], []
+    for l, k in ((5, 1), (40, 2), (97, 1), (130, 1)):
+        n = 15 * k + 1
+        A = _device_matrix(_matrix(m, n, w, 20 * w + l), w, dev)
+        ctB = encrypt_gpu(dev, inputs.pcmm_problem(8350 + l, 1, n, l, 1))
+        items.append((A, ctB, l, w, k))
+        want.append(pcmm.normalize(pcmm.schoolbook(A, ctB, l, w), m * l))
+    for max_strips in (0, 4):
+        batch = pcmm.Batch(items, max_strips=max_strips)
+        outs = batch.run()
+        for out, (A, _, l, _, _), ref in zip(outs, items, want):
+            assert torch.equal(pcmm.normalize(out, m * l), ref)
+        assert pcmm.workspace_status(batch.ws) == 0
+
+
+def test_batched_tables_of_few_codes_cost_what_they_hold():
+    # Half a percent of the entries not zero against dense (about a tenth; tables that
+    # make every digit's multiples take a quarter).
+    dev = device()
+    m, n, l, w = 128, 256, 256, 8
+    ctB = encrypt_gpu(dev, inputs.pcmm_problem(8450, 1, n, l, 1))
+    rng = np.random.default_rng(2)
+    dense = rng.integers(1, 1 << w, (m, n))
+    times = []
+    for A in (dense * (rng.random((m, n)) < 0.005), dense):
+        batch = pcmm.Batch([(_device_matrix(A.astype(np.uint8), w, dev), ctB, l, w, 1)])
+        batch.run()
+        pcmm.profile_enable(64)
+        batch.run()
+        times.append(pcmm.profile_read()["batched"][0])
+        pcmm.profile_enable(0)
+    assert times[0] < 0.17 * times[1], times
+
+
 @pytest.mark.parametrize("w", [12, 16])
 def test_tables_of_few_codes_cost_what_they_hold(w):
     # 256 columns of one value against dense ones (about an eleventh and a fifteenth).
