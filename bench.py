@@ -372,8 +372,8 @@ def run_ours(args, dist):
     props = torch.cuda.get_device_properties(dev)
     prod_peak = peaks["product"]
     alu_peak = peaks["add_carry"]
-    prods = {"gather": sum(counts.gather_imad(r["counts"]) for r in runs) // counts.IMAD_PER_PRODUCT,
-             "table": sum(counts.table_imad(r["counts"]) for r in runs) // counts.IMAD_PER_PRODUCT}
+    prods = {"gather": sum(counts.gather_products(r["counts"]) for r in runs),
+             "table": sum(counts.table_products(problems[r["w"]]["A"], r["w"], r["k"], l) for r in runs)}
     units = {"gather": sum(r["counts"]["gather_madd"] for r in runs),
              "table": sum(counts.point_ops(r["counts"]) - r["counts"]["gather_madd"] for r in runs)}
     kernels = {nm: {"ms_per_step": v[0] / args.steps, "launches_per_step": v[1] / args.steps}
@@ -665,7 +665,7 @@ def run_sweep(args, dist):
             del ws
             c = counts.cussen_counts(A_h, w, k, n)
             ops = counts.point_ops(c)
-            imad = counts.gather_imad(c) + counts.table_imad(c)
+            imad = counts.IMAD_PER_PRODUCT * (counts.gather_products(c) + counts.table_products(A_h, w, k, n))
             ops_row = 2.0 * n * n * (1.5 * w + 1)          # schoolbook point operations per row
             ms_rows = int(min(n, max(8, 4e9 // ops_row)))
             sb = timed(lambda: pcmm.schoolbook(A[:ms_rows], ctB, n, w, out=out), reps=1)
