@@ -195,15 +195,18 @@ pcmm_status pcmm_schoolbook16(const uint16_t *A, int m, int n, int w, const uint
                               uint32_t *ctC, pcmm_stream_t stream);
 
 /* Strip width chosen by the built-in cost model for a problem shape: the k
- * in [1, 16/w] minimising the modelled work (table build, normalisation and
- * gather, the table work weighted by its lower measured issue efficiency).
+ * in [1, 16/w] minimising the modelled work (table build by prefix sums,
+ * normalisation and gather, the table work weighted by its lower issue
+ * efficiency).
  * Accepts 1 <= w <= 16; returns 0 for invalid arguments. */
 int pcmm_cussen_choose_k(int m, int n, int l, int w);
 
 /* Workspace bytes with which pcmm_cussen (or pcmm_cussen16) processes
  * `strips` strips per pass (the pass size: table warps of a launch, and the
  * scratch and tables they hold), for strip width k >= 1; 0 for invalid
- * arguments.  strips is capped at the strips of the matrix. */
+ * arguments.  strips is capped at the strips of the matrix.  The size includes
+ * the gather's partial sums; smaller workspaces run without them, down to the
+ * plan and one strip. */
 size_t pcmm_cussen_workspace_bytes_for(int m, int n, int l, int w, int k, int strips);
 
 /* Workspace bytes pcmm_cussen (w <= 8) or pcmm_cussen16 (w <= 16) needs for
@@ -241,7 +244,9 @@ size_t pcmm_workspace_bytes(int op, int m, int n, int l, int w, int k);
  * each ciphertext of that row of Enc(B), reconstruction by prefix sums of
  * points rebuilds the multiples of every distinct value, and each output
  * ciphertext adds the multiple its entry selects (the un-sort step fused
- * with the accumulation).  k > 1 (an extension, not in the paper) also
+ * with the accumulation).  Passes whose strips hold many distinct values make
+ * the same multiples from those of the values' 4-bit digits, with fewer
+ * operations.  k > 1 (an extension, not in the paper) also
  * combines k adjacent columns into one table of the distinct k-tuples of
  * the strip, so the gather adds once per strip instead of once per column.
  * The result is identical for every k.

@@ -62,12 +62,15 @@ __device__ __forceinline__ fe fe_shfl(const fe& a, int src) {
 // of them must call.
 //
 // Division steps (Bernstein and Yang, "Fast constant-time gcd computation
-// and modular inversion", 2019) in batches of 30: from f = p, g = a a batch
+// and modular inversion", 2019) in batches of 30, with delta = k + 1/2 and several
+// steps at once as in the variable-time inversion of libsecp256k1
+// (src/modinv32_impl.h): from f = p, g = a a batch
 // reads only the low words of f and g and yields integers u, v, q, r with
 //   (f, g) <- (u f + v g, q f + r g) / 2^30,
 // and the same map, with a multiple of p that makes the division exact, keeps
 // d a = C f and e a = C g (mod p), starting from d = 0, e = C = R^2.  When g
-// reaches 0 (after about 530 steps, 741 at most), f = +-1 and d = +-R^2 / a.
+// reaches 0 (after about 530 steps; 590 at most from that delta, 741 from the
+// paper's, and the loop allows 750), f = +-1 and d = +-R^2 / a.
 // A step with delta = k + 1/2 > 0 and g odd takes (f, g) <- (g, (g - f) / 2),
 // delta <- 1 - delta; any other (f, g) <- (f, (g + (g mod 2) f) / 2), delta <-
 // delta + 1.  Runs of the second kind are taken at once: w f with w = -g / f

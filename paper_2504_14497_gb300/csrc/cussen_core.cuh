@@ -1919,9 +1919,10 @@ inline double expected_distinct_nonzero(int m, int bits) {
 // tables (k > 1); for k > 1 the
 // tuple entries by affine additions (6 per further non-zero component).  The
 // table work is weighted by 1.9, fitted to GB300 timings of the
-// 1024 x 1024 x 256 product for every w and k (the table build issues its
-// multiplications less efficiently than the gather, and its tuple rounds
-// reload their operands from scratch).
+// 1024 x 1024 x 256 product for every w and k with tables by chains, which
+// issue their multiplications less efficiently than the gather.  Of tables by digits,
+// which most are now, it says too much: at w = 1 seven columns take 7.9 ms, the
+// chosen six 8.7.
 inline double model_cost(int m, int n, int l, int w, int k) {
     const double MADD = 11, DBL = 8, NORM = 5, AFF = 6, TABLE_WEIGHT = 1.9;
     const double chains = 2.0 * l;

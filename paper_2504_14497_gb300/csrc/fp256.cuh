@@ -22,8 +22,10 @@
 // in with addc took a register move per product beside 57 additions:
 // 385 cycles a product against 290, 530 a multiplication against 437.
 // Squaring: 28 cross products, doubled, plus 8 diagonal squares.  Products
-// and reductions live in out-of-line functions (fmul, fsqr): inlining them
-// into every call site of a point formula overflows the instruction cache.
+// and reductions also live in out-of-line functions (fmul, fsqr), which the
+// table builds call: a call moves its operands on the pipe that multiplies, but
+// their code inlined at every site outgrows the instruction cache.  Loops of
+// one addition or doubling inline them (gather, encryption, decryption).
 //
 // Reduction of the 512-bit product t to t / R mod p: since p = -1 mod 2^96,
 // the three lowest words q of t cancel against q p, which leaves (after the

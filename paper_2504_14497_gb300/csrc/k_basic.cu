@@ -517,9 +517,10 @@ static pcmm_status launch_encrypt(const void* keytable, const uint8_t* msg, cons
     uint4* gtab = nullptr;
     if (cudaGetSymbolAddress((void**)&gtab, g_comb_G) != cudaSuccess) return PCMM_ECUDA;
     ProfScope ps(KID_ENCRYPT, st);
-    // One thread a component from three warps per scheduler on; below, the
-    // windows' serial additions are the time, and threads up to one or two warps
-    // per scheduler share them. Time (us) with both components in one thread, and
+    // The windows' serial additions are the time of a small call, so threads share
+    // them: eight a component as long as that is one warp per scheduler (1216
+    // ciphertexts), two up to two warps (9728). The true crossovers lie higher, as the
+    // times say. Time (us) with both components in one thread, and
     // with 1, 2 and 8 threads each: 1 ciphertext 282 / -, 78, 57; 1000 282 / -, 82,
     // 60; 4000 284 / 119, 83, 139; 10000 285 / 163, 145, 270; 30000 389 / 280, 332, -.
     const int G = count <= 1216 ? 8 : count <= 9728 ? 2 : 1;

@@ -27,9 +27,10 @@
 //         chain multiplied them by; the inversion is shared by the lanes of
 //         a warp and, when the block's four warps follow one strip's plan,
 //         by the whole block.  Wherever the scratch holds the tables of a
-//         code's halves (most strips) the same entries are built digit by
-//         digit in affine coordinates instead (table_block), from the
-//         values that the compressed levels expand to.
+//         code's halves (most strips) and the pass's strips hold more than a
+//         few codes (pass_few) the same entries are built digit by digit
+//         in affine coordinates instead (table_block), from the values that
+//         the compressed levels expand to.
 //  gather (one warp per output row i and 32 ciphertext chains)
 //         C_ij += T_s[rank_s(i)] for every strip s: the "un-sort and re-insert
 //         duplicates" step of Algorithm 2 fused with the accumulation of
@@ -202,12 +203,13 @@ extern "C" int pcmm_cussen_choose_k(int m, int n, int l, int w) {
     return best;
 }
 
-// Table items (warps) per pass come in whole waves of the table kernel on a
-// 152-SM GB300 (PCMM_TABLE_MINBLOCKS blocks of 4 warps per SM), so that only a
-// pass's last wave can run partly empty: four waves when one pass's scratch
-// and tables fit in PASS_BYTES_CAP, else as many whole waves as fit, at
-// least one.  Whole-wave passes measured 3 ms per headline step faster than
-// passes of 4096 items (at 4 blocks per SM).
+// Table items (warps, counted without packing) per pass come in whole waves of
+// the chains' table kernel on a 152-SM GB300 (PCMM_TABLE_MINBLOCKS blocks of 4 warps
+// per SM): four waves when one pass's scratch and tables fit in PASS_BYTES_CAP, else
+// as many whole waves as fit, at least one.  With chains, whole-wave passes
+// measured 3 ms per headline step faster than passes of 4096 items (at 4 blocks
+// per SM).  The digit kernel's waves are of 2432 items and its scratch is smaller, so
+// its last wave is partly empty; the sizes of workspaces follow from this rule.
 #ifndef PCMM_TARGET_WAVES
 #define PCMM_TARGET_WAVES 4
 #endif
@@ -233,8 +235,9 @@ pcmm_status launch_plan(const Layout& L, const TA* A, const PlanPtrs& P, cudaStr
 }
 
 // Warps per output for the gather of a pass of S strips: when the outputs
-// alone give fewer than GATHER_WARPS_TARGET warps (about four waves of the
-// gather on 152 SMs), each output's strips are split into up to 32 parts of
+// alone give fewer than GATHER_WARPS_TARGET warps (about five waves of the
+// gather on 152 SMs; both components' warps counted without packing, up to twice the
+// warps there are for l <= 16), each output's strips are split into up to 32 parts of
 // at least part_strips strips, and a combine kernel adds the partial sums
 // (one full addition per part against at least part_strips mixed additions).
 // Parts go down to 4 strips while all of them still leave the 608 schedulers
