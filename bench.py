@@ -169,11 +169,19 @@ class ClockSampler:
 
 # -------------------------------------------------------------- workload
 
+def record_digest(rec: dict) -> str:
+    """What a profile record's "sha256" holds: a digest of its counters and of the
+    source hash they were captured at, so that neither is replaced alone."""
+    import hashlib
+    body = {key: value for key, value in rec.items() if key != "sha256"}
+    return hashlib.sha256(json.dumps(body, sort_keys=True).encode()).hexdigest()
+
+
 def recorded_profile(kernel: str):
     """The committed ncu record of `kernel` in profiles/ (a JSON block with
     per-launch DRAM traffic scaled to the headline launch and the kernel's
     instruction mix per unit of work), or None when the kernel's source has
-    changed since it was taken."""
+    changed since it was taken, or the record since it was written."""
     import glob
     import hashlib
     for path in sorted(glob.glob(os.path.join(ROOT, "profiles", "*.md"))):
@@ -186,7 +194,7 @@ def recorded_profile(kernel: str):
         h = hashlib.sha256()
         for f in rec["source_files"]:
             h.update(open(os.path.join(ROOT, f), "rb").read())
-        if h.hexdigest() == rec["source_sha256"]:
+        if h.hexdigest() == rec["source_sha256"] and rec.get("sha256") == record_digest(rec):
             return rec
     return None
 
