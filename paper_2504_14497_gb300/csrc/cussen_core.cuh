@@ -1706,12 +1706,12 @@ __device__ __forceinline__ void table_block(const TableArgs& a, const PlanPtrs& 
 // (us) by digits and by chains: w = 8 with 3.6 values a column 841 and 659, w = 12
 // with 50 3833 and 3224, with 101 4383 and 4415, w = 16 with 3.2 5477 and 1214.
 __device__ __forceinline__ int strip_excess(int entries, const uint16_t* len, int columns, int w, const FewArgs& f) {
+    static_assert(NLEV == 4, "a column's lengths are read as one ushort4");
     int chains = 0;
+#pragma unroll 1
     for (int t = 0; t < columns; t++, len += NLEV) {
-        const int l1 = len[0];
-        if (!l1) continue;
-        chains += 33 * (l1 - 1) + 19 * (w - 1) * len[NLEV - 1] + (w > 1 ? 144 : 0);
-        for (int q = 1; q < NLEV - 1; q++) chains += 36 * (len[q] - 1);
+        const ushort4 q = *(const ushort4*)len;
+        if (q.x) chains += 33 * (q.x - 1) + 36 * (q.y + q.z - 2) + 19 * (w - 1) * q.w + (w > 1 ? 144 : 0);
     }
     // f.fixed counts the chains' own constant, which an empty strip does not have.
     return entries > 0 ? chains - f.entry * entries - f.fixed : -(f.fixed + 184 + 80 * columns);
@@ -1724,6 +1724,7 @@ __device__ __forceinline__ int strip_excess(int entries, const uint16_t* len, in
 static __device__ __noinline__ bool pass_few(const int32_t* nent, const uint16_t* col_len, int s0, int strips, int n, int k,
                                              int w, int emax, FewArgs f, uint4* sm) {
     long long sum = 0;
+#pragma unroll 1
     for (int x = (int)threadIdx.x; x < strips; x += 128) {
         const int s = s0 + x, c0 = s * k, E = nent[s];
         sum += strip_excess(E < emax ? E : emax, col_len + (size_t)c0 * NLEV, c0 + k <= n ? k : n - c0, w, f);
