@@ -106,7 +106,8 @@ size_t pcmm_encrypt_workspace_bytes(void);
  * msg: device uint8[count].  r: device scalars (quad-planar, 8 * count
  * words); each r is used modulo q, and is not checked against [1, q-1].
  * ct: device, affine ciphertext array of count elements (32 * count words),
- * written canonical.
+ * written canonical.  r may lie in ct as two consecutive ones of its eight
+ * quads (words 4 * q * count on); msg and r otherwise do not overlap ct.
  * ws: device, 256-byte aligned, >= pcmm_encrypt_workspace_bytes() bytes.
  * It caches the comb table of H: a call whose workspace already holds the
  * table of the same H (from an earlier pcmm_encrypt on the same stream

@@ -140,18 +140,18 @@ __device__ __forceinline__ void block_normalize_jacz(aff out[E], const jacz P[E]
 
 // Enc(b) = (rG, rH + bG): 32 window lookups per base point, added into an
 // (X, Y, Z^2, Z^3) accumulator (8M + 2S each, and the standard comb entries
-// need no conversion). G threads (a power of two) take one component (first, then
-// the other) of a ciphertext, every G-th window each, and add their sums as a
+// need no conversion). G threads (a power of two) take one component
+// (blockIdx.y) of a ciphertext, every G-th window each, and add their sums as a
 // tree.
 template <int G, int INL, int BLOCKS>
 __global__ void __launch_bounds__(128, BLOCKS) encrypt_kernel(const uint4* __restrict__ gtab,
                                                               const uint4* __restrict__ htab,
                                                               const uint8_t* __restrict__ msg,
-                                                              const uint4* r, size_t count, uint4* ct,
-                                                              unsigned first) {
+                                                              const uint4* __restrict__ r, size_t count,
+                                                              uint4* __restrict__ ct) {
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t i = t / G;
-    const int part = (int)(t % G), c = (int)(blockIdx.y ^ first);
+    const int part = (int)(t % G), c = blockIdx.y;
     const bool valid = i < count;
     const size_t ii = valid ? i : 0;
     const uint4* tab = c ? htab : gtab;
@@ -199,6 +199,44 @@ __global__ void __launch_bounds__(128, BLOCKS) encrypt_kernel(const uint4* __res
     aff out[1];
     block_normalize_jacz<1>(out, P);
     if (valid && part == 0) store_aff(ct + (size_t)c * 4 * count, count, i, out[0]);
+}
+
+// The same for nonces that lie in the output: a thread takes both components and
+// writes when it has read its nonce.
+__global__ void __launch_bounds__(128) encrypt_in_place_kernel(const uint4* __restrict__ gtab,
+                                                               const uint4* __restrict__ htab,
+                                                               const uint8_t* msg, const uint4* r, size_t count,
+                                                               uint4* ct) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool valid = i < count;
+    fe rr;
+    fe_zero(rr);
+    if (valid) fe_from_quads(rr, r[i], r[count + i]);
+    jacz P[2];
+    jacz_set_inf(P[0]);
+    jacz_set_inf(P[1]);
+    aff T;
+    for (int win = 0; win < COMB_WINDOWS; win++) {
+        const uint32_t v = (rr.v[win >> 2] >> (8 * (win & 3))) & 0xffu;
+        if (v) {
+            load_aff(T, gtab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
+            jacz_madd_t<0, true>(P[0], T);
+            load_aff(T, htab, COMB_POINTS, (size_t)win * COMB_ENTRIES + v);
+            jacz_madd_t<0, true>(P[1], T);
+        }
+    }
+    const uint32_t b = valid ? msg[i] : 0u;
+    if (b) {
+        load_aff(T, gtab, COMB_POINTS, b);
+        jacz_madd_t<0, true>(P[1], T);
+    }
+    __syncwarp();
+    aff out[2];
+    block_normalize_jacz<2>(out, P);
+    if (valid) {
+        store_aff(ct, count, i, out[0]);
+        store_aff(ct + 4 * count, count, i, out[1]);
+    }
 }
 
 // s G for count scalars (key generation: H = x G), one thread per scalar.
@@ -526,14 +564,13 @@ static pcmm_status launch_encrypt(const void* keytable, const uint8_t* msg, cons
     const int G = count <= 1216 ? 8 : count <= 9728 ? 2 : 1;
     auto* kernel = G == 8 ? encrypt_kernel<8, 31, 2> : G == 2 ? encrypt_kernel<2, 31, 2>
                                                               : encrypt_kernel<1, 31, PCMM_ENCRYPT_MINBLOCKS>;
-    // Nonces that lie in one component of the output are still read by the other:
-    // that one is computed first, in a launch of its own.
     const char *r0 = (const char*)r, *c0 = (const char*)ct;
-    const bool apart = r0 >= c0 + 128 * count || r0 + 32 * count <= c0;
-    const unsigned first = !apart && r0 < c0 + 64 * count ? 1u : 0u;
-    for (unsigned c = 0; c < (apart ? 1u : 2u); c++)
-        kernel<<<dim3(grid_for(count * G, 128), apart ? 2 : 1), 128, 0, st>>>(
-            gtab, (const uint4*)keytable, msg, (const uint4*)r, count, (uint4*)ct, first ^ c);
+    if (r0 < c0 + 128 * count && c0 < r0 + 32 * count)
+        encrypt_in_place_kernel<<<grid_for(count, 128), 128, 0, st>>>(gtab, (const uint4*)keytable, msg,
+                                                                     (const uint4*)r, count, (uint4*)ct);
+    else
+        kernel<<<dim3(grid_for(count * G, 128), 2), 128, 0, st>>>(gtab, (const uint4*)keytable, msg,
+                                                                  (const uint4*)r, count, (uint4*)ct);
     PCMM_CUDA_CHECK_LAUNCH();
     return PCMM_OK;
 }

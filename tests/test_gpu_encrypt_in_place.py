@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("quad", [0, 2, 4, 6])
+@pytest.mark.parametrize("quad", [0, 2, 3, 4, 6])
 @pytest.mark.parametrize("count", [5, 3000, 250000])
 def test_nonces_inside_the_output(count, quad):
     # The nonces' two quads are two of the eight that the ciphertexts of the same
